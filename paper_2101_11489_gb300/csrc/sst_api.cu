@@ -29,6 +29,7 @@ KParams kparams(const sst_ctx* c) {
   k.calq = c->calq;
   k.badmask = c->badmask;
   k.qmul = c->qmul;
+  k.mul = c->mul;
   return k;
 }
 
@@ -98,9 +99,9 @@ cudaError_t ensure_scratch(Scratch& s, size_t items, size_t events, size_t stage
       size_t c6 = s.items_cap, c7 = s.items_cap;
       if ((e = grow(s.lb, cap, items))) return e;
       if ((e = grow(s.fed_off, c2, items))) return e;
-      if ((e = grow(s.fed_cnt, c3, items))) return e;
-      if ((e = grow(s.fed_start, c4, items))) return e;
-      if ((e = grow(s.fed_dest, c5, items))) return e;
+      if ((e = grow(s.fed_cnt, c3, 2 * items))) return e;
+      if ((e = grow(s.fed_start, c4, 2 * items))) return e;
+      if ((e = grow(s.fed_dest, c5, 2 * items))) return e;
       if ((e = grow(s.unit_desc, c6, items))) return e;
       if ((e = grow(s.big_list, c7, items))) return e;
       s.items_cap = items;
@@ -211,6 +212,7 @@ sst_status sst_destroy(sst_ctx* ctx) {
   if (ctx->calq) cudaFree(ctx->calq);
   if (ctx->badmask) cudaFree(ctx->badmask);
   if (ctx->qmul) cudaFree(ctx->qmul);
+  if (ctx->mul) cudaFree(ctx->mul);
   if (ctx->pitch) cudaFree(ctx->pitch);
   delete ctx;
   return SST_OK;
@@ -245,25 +247,34 @@ sst_status sst_calib_upload(sst_ctx* ctx, const float* noise, const float* gain,
     if ((e = cudaMalloc(&ctx->calq, n * sizeof(uint2)))) return cuda_err(ctx, e, "cudaMalloc calq");
     if ((e = cudaMalloc(&ctx->badmask, n / 8))) return cuda_err(ctx, e, "cudaMalloc badmask");
     if ((e = cudaMalloc(&ctx->qmul, n_apv * sizeof(float)))) return cuda_err(ctx, e, "cudaMalloc qmul");
+    if ((e = cudaMalloc(&ctx->mul, n_apv * sizeof(int32_t)))) return cuda_err(ctx, e, "cudaMalloc mul");
   }
   // staging of the raw tables, freed once the kernels' tables are built
   uint8_t* bad_dev = nullptr;
-  float* noise_dev = nullptr;
+  float *noise_dev = nullptr, *gain_dev = nullptr;
   if ((e = cudaMalloc(&bad_dev, n))) return cuda_err(ctx, e, "cudaMalloc bad");
   if ((e = cudaMalloc(&noise_dev, n * sizeof(float)))) {
     cudaFree(bad_dev);
     return cuda_err(ctx, e, "cudaMalloc noise");
+  }
+  if ((e = cudaMalloc(&gain_dev, n_apv * sizeof(float)))) {
+    cudaFree(bad_dev);
+    cudaFree(noise_dev);
+    return cuda_err(ctx, e, "cudaMalloc gain");
   }
   // Copies are stream-ordered after earlier work on `st`; synchronise before the
   // host buffers go out of the caller's hands and before freeing the staging.
   if (!e) e = cudaMemcpyAsync(noise_dev, noise, n * sizeof(float), cudaMemcpyHostToDevice, st);
   if (!e) e = cudaMemcpyAsync(ctx->qmul, qmul.data(), n_apv * sizeof(float), cudaMemcpyHostToDevice, st);
   if (!e) e = cudaMemcpyAsync(bad_dev, bad, n, cudaMemcpyHostToDevice, st);
+  if (!e) e = cudaMemcpyAsync(gain_dev, gain, n_apv * sizeof(float), cudaMemcpyHostToDevice, st);
+  if (!e) e = build_gain(gain_dev, ctx->mul, (uint32_t)n_apv, st);
   if (!e) e = build_badmask(bad_dev, ctx->badmask, n, st);
   if (!e) e = build_calib(noise_dev, ctx->badmask, ctx->calq, n, *params, st);
   if (!e) e = cudaStreamSynchronize(st);
   cudaFree(bad_dev);
   cudaFree(noise_dev);
+  cudaFree(gain_dev);
   if (e) return cuda_err(ctx, e, "sst_calib_upload");
   ctx->params = *params;
   ctx->has_calib = true;
@@ -452,10 +463,11 @@ sst_status sst_autotune(sst_ctx* ctx, const uint8_t* raw, const uint64_t* event_
         s.block = b;
         s.units = u;
         s.ctas_per_sm = p;
-        if (!shape_valid(s) || batch_smem(u, b) * (size_t)p > 227u * 1024u) continue;
+        if (!shape_valid(s)) continue;
         int grid = 0, ipf = 0;
         size_t smem = 0;
         if ((ce = batch_launch_info(s, n_events, n_feds, ctx->n_sm, &grid, &smem, &ipf))) break;
+        if (smem * (size_t)p > 227u * 1024u) continue;
         bool dup = false;  // the occupancy clamps p: the same launch was timed already
         for (auto& pr : timed)
           if (pr.first == grid && pr.second.block == b && pr.second.units == u) dup = true;

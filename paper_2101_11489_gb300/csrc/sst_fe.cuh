@@ -494,9 +494,7 @@ __device__ uint32_t form_unit(W& w, const KParams& kp, int n, int k_begin, int n
       lo = (uint32_t)lo_i;
       wd = (uint32_t)(hi - lo_i + 1);
       if (pass && (stage || keep))
-        bary = q_sum == 0 ? __fadd_rn((float)lo_i, __fmul_rn(0.5f, (float)wd))
-                          : __fadd_rn(__fadd_rn((float)lo_i, 0.5f),
-                                      __fdiv_rn(__uint2float_rn(moment), __uint2float_rn(q_sum)));
+        bary = centroid((uint32_t)lo_i, wd, q_sum, moment);
     }
     const unsigned b = __ballot_sync(0xffffffffu, pass);
     if (keep && k0 == k_begin) {

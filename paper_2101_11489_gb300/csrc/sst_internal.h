@@ -20,6 +20,7 @@ constexpr int kChPerFe = SST_CH_PER_FE;      // channels per FE unit
 constexpr int kApv = SST_STRIPS_PER_APV;     // strips per APV
 constexpr int kHdr = SST_FED_HEADER_BYTES;   // FED header bytes
 constexpr int kFedStrips = kCh * kStrips;    // 24,576 strips per FED
+constexpr int kMulShift = 22;                // fixed-point charge multipliers: binary places
 constexpr int kMaskWords = kStrips / 32;     // 8 words of 32 strips per channel
 
 // Calibration and thresholds as the kernels see them.  The per-strip tables are
@@ -33,6 +34,7 @@ struct KParams {
   const uint32_t* badmask;  // [n_strips / 32], bit (s & 31) of word s / 32
   const float* qmul;        // [n_strips / 128]: per APV, a multiplier certified to give the
                             // gain-corrected charge of every ADC 0..253, or -gain (divide)
+  const int32_t* mul;       // [n_strips / 128]: per APV, the fixed-point charge multiplier, or the bits of -gain (k_gain_pack)
   uint4* spill = nullptr;   // the launch's spill areas (one per warp of the grid, kSpillRecords records each)
   uint32_t spill_warps = 0; // warps that have one
   const uint32_t* big_list = nullptr;  // batched launches: the work items too large to stage (their
@@ -81,7 +83,7 @@ struct Scratch {
   size_t amp_items_cap = 0, amp_ev_cap = 0;
 };
 constexpr uint32_t kNoAmp = 0xFFFFFFFFu;
-constexpr uint32_t kSpillRecords = 1024;  // records per warp spill area (16 KiB)
+constexpr uint32_t kSpillRecords = 1608;  // records per warp spill area (25 KiB)
 constexpr int kMaxWarpsPerSm = 32;        // resident warps of the batched kernel per SM (its register use)
 
 size_t smem_bytes(int tile);
@@ -117,6 +119,7 @@ cudaError_t launch_batch(const uint8_t* raw, const uint64_t* event_off, const ui
 cudaError_t build_badmask(const uint8_t* bad_dev, uint32_t* mask_dev, uint64_t n_strips, cudaStream_t st);
 // Adds base to the first *count (device) values of amp_first, kNoAmp excepted.
 cudaError_t rebase_amp_first(uint32_t* amp_first, const uint64_t* count, uint32_t base, int n_sm, cudaStream_t st);
+cudaError_t build_gain(const float* gain_dev, int32_t* mul_dev, uint32_t n_apv, cudaStream_t st);
 cudaError_t build_calib(const float* noise_dev, const uint32_t* mask_dev, uint2* calq_dev,
                         uint64_t n_strips, const sst_params& p, cudaStream_t st);
 
@@ -133,6 +136,7 @@ struct sst_ctx {
   sst_params params{};
   uint2* calq = nullptr;       // per strip: channel and seed thresholds as ADC limits and linking gap; noise^2
   uint32_t* badmask = nullptr;
+  int32_t* mul = nullptr;      // per APV: fixed-point charge multiplier or the bits of -gain
   float* qmul = nullptr;       // per APV: certified multiplier or -gain
   sst::Scratch scratch;
   sst::Shape shape{};

@@ -32,6 +32,7 @@
 // Every device wait (the look-back) has an iteration limit; when it runs out the
 // event is flagged SST_EV_TIMEOUT and the CTA carries on without the value.
 #include <cstddef>
+#include <type_traits>
 #include <utility>
 
 #include "sst_internal.h"
@@ -424,7 +425,18 @@ __device__ void emit_channels(Shm<TILE>& s, const uint8_t* src, int c0, int c1, 
 
 __device__ __forceinline__ bool bit(const uint32_t* m, int t) { return (m[t >> 5] >> (t & 31)) & 1u; }
 
+// Centroid of a cluster (a6): its middle without charge, else first + 1/2 + moment /
+// charge, the moment taken about its first strip; each operation one binary32
+// rounding.  A moment of 0 (every one-strip cluster) is kept from the division, whose
+// slow path zeros take: half the instructions of the ordering pass.
+__device__ __forceinline__ float centroid(uint32_t lo, uint32_t wd, uint32_t q, uint32_t moment) {
+  if (q == 0) return __fadd_rn((float)lo, __fmul_rn(0.5f, (float)wd));
+  const float f = __fdiv_rn(__uint2float_rn(moment ? moment : 1u), __uint2float_rn(q));
+  return __fadd_rn(__fadd_rn((float)lo, 0.5f), moment ? f : 0.f);
+}
+
 #include "sst_fe.cuh"
+#include "sst_stream.cuh"
 
 // Greedy channel-aligned chunk [c0, c1) holding at most TILE digis.
 template <int TILE>
@@ -716,22 +728,29 @@ __global__ void __launch_bounds__(256) k_compact(const uint4* __restrict__ stage
 // a6, output without amplitudes: orders and copies the staged clusters in one
 // pass.  CTA c of event e takes the event's segments [c * SEGS, (c + 1) * SEGS):
 // it sums the counts of the event's segments before them (its place in the
-// event), scans its own counts in shared memory, and copies its clusters to one
-// contiguous range of the output, thread t taking output records t, t + 256, ...
-// (four loads in flight per thread) and finding each one's segment by binary
-// search over the scanned counts (coalesced stores; each segment's staged records
-// are contiguous).  The event's
+// event), scans its own counts in shared memory, notes every output record's
+// segment there, and copies its clusters to one contiguous range of the output,
+// thread t taking records t, t + 256, ... (four loads in flight per thread,
+// coalesced stores; each segment's staged records are contiguous).  For the 4.8 M
+// clusters of 64 full-detector events it moves 116 MB; 33 us from a cold L2, half of
+// its issue slots busy.  (8 threads to a segment, without the map: 50 us, the stores
+// no longer coalesced.)  The event's
 // clusters start at clu_off[e] (its slice; 0 without clu_off), or at pack_off[e]
 // when pack_off is given (k_clu_scan computed it and the events' counts); the
 // event's last CTA otherwise stores its cluster count.
-template <int SEGS>
+// PACKED: the staged records are cs::staged_cluster's 8 bytes, `chans` channels to a
+// segment, and the centroid is formed here.
+template <int SEGS, bool PACKED>
 __global__ void __launch_bounds__(256) k_order(const uint4* __restrict__ stage, const uint64_t* __restrict__ clu_off,
                                                const uint64_t* __restrict__ pack_off,
                                                const uint32_t* __restrict__ seg_cnt,
                                                const uint32_t* __restrict__ seg_start, uint32_t n_segs, uint32_t cpe,
-                                               sst_clusters out, sst_event_status* status) {
-  static_assert(SEGS <= 256 && (SEGS & (SEGS - 1)) == 0, "one scan entry per thread, binary search");
+                                               sst_clusters out, sst_event_status* status, uint32_t chans) {
+  static_assert(SEGS <= 256, "one scan entry per thread, a byte per segment");
+  constexpr bool kNoted = SEGS > 16;             // few segments: searched for instead (4 steps, no barriers)
+  constexpr uint32_t kMap = kNoted ? 4096 : 1;   // output records whose segments are noted at once
   __shared__ uint32_t s_dest[SEGS + 1], s_start[SEGS];
+  __shared__ uint8_t s_seg[kMap];
   __shared__ uint32_t wsum[32];
   pdl_wait();  // the staged clusters and counts
   const uint32_t e = blockIdx.x / cpe, c = blockIdx.x % cpe;
@@ -739,6 +758,8 @@ __global__ void __launch_bounds__(256) k_order(const uint4* __restrict__ stage, 
   const uint32_t nseg = n_segs - seg0 < (uint32_t)SEGS ? n_segs - seg0 : (uint32_t)SEGS;
   const uint32_t* cnt_e = seg_cnt + (size_t)e * n_segs;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t v = tid < (int)nseg ? __ldg(cnt_e + seg0 + tid) : 0u;
+  if (tid < SEGS) s_start[tid] = tid < (int)nseg ? __ldg(seg_start + (size_t)e * n_segs + seg0 + tid) : 0u;
   // clusters of the event's segments before this CTA's
   uint32_t part = 0;
   for (uint32_t i = tid; i < seg0; i += blockDim.x) part += __ldg(cnt_e + i);
@@ -749,40 +770,69 @@ __global__ void __launch_bounds__(256) k_order(const uint4* __restrict__ stage, 
   for (int k = 0; k < (int)(blockDim.x >> 5); k++) pre += wsum[k];
   __syncthreads();
   // this CTA's segments: exclusive scan of their counts
-  const uint32_t v = tid < (int)nseg ? __ldg(cnt_e + seg0 + tid) : 0u;
-  if (tid < SEGS) s_start[tid] = tid < (int)nseg ? __ldg(seg_start + (size_t)e * n_segs + seg0 + tid) : 0u;
   uint32_t tot;
   const uint32_t ex = block_excl_scan(v, wsum, &tot);
   if (tid < SEGS) s_dest[tid] = ex;
   if (tid == 0) s_dest[SEGS] = tot;
-  __syncthreads();
   const uint64_t off = clu_off ? clu_off[e] : 0;
   const uint4* src = stage + off;
+  const uint2* src2 = reinterpret_cast<const uint2*>(stage) + off;
   const uint64_t dst = (pack_off ? pack_off[e] : off) + pre;
+  uint32_t* const det = out.det + dst;
+  uint16_t* const first = out.first + dst;
+  uint16_t* const width = out.width + dst;
+  uint32_t* const charge = out.charge + dst;
+  float* const bary = out.barycenter + dst;
   constexpr int kU = 4;  // records per thread in flight
-  for (uint32_t d0 = tid; d0 < tot; d0 += kU * blockDim.x) {
-    uint4 r[kU];
+  if (!kNoted) __syncthreads();
+  for (uint32_t m0 = 0; m0 < tot; m0 += kNoted ? kMap : tot) {
+    const uint32_t m1 = kNoted && m0 + kMap < tot ? m0 + kMap : tot;
+    if (kNoted) __syncthreads();
+    if (kNoted && tid < SEGS)
+      for (uint32_t d = ex > m0 ? ex : m0; d < ex + v && d < m1; d++) s_seg[d - m0] = (uint8_t)tid;
+    if (kNoted) __syncthreads();
+    for (uint32_t d0 = m0 + tid; d0 < m1; d0 += kU * blockDim.x) {
+      uint4 r[kU];
 #pragma unroll
-    for (int u = 0; u < kU; u++) {
-      const uint32_t d = d0 + u * blockDim.x;
-      if (d < tot) {
-        int lo = 0;  // the last segment starting at or before d: it holds d
+      for (int u = 0; u < kU; u++) {
+        const uint32_t d = d0 + u * blockDim.x;
+        if (d < m1) {
+          uint32_t sg = 0;
+          if (kNoted) {
+            sg = s_seg[d - m0];
+          } else {
 #pragma unroll
-        for (int step = SEGS / 2; step > 0; step >>= 1)
-          if (s_dest[lo + step] <= d) lo += step;
-        r[u] = __ldg(src + s_start[lo] + (d - s_dest[lo]));
+            for (int step = SEGS / 2; step > 0; step >>= 1)
+              if (s_dest[sg + step] <= d) sg += step;
+          }
+          const uint32_t at = s_start[sg] + (d - s_dest[sg]);
+          if (PACKED) {
+            const uint2 v2 = __ldg(src2 + at);
+            r[u] = make_uint4(v2.x, v2.y, (seg0 + sg) * chans, 0u);
+          } else {
+            r[u] = __ldg(src + at);
+          }
+        }
       }
-    }
 #pragma unroll
-    for (int u = 0; u < kU; u++) {
-      const uint32_t d = d0 + u * blockDim.x;
-      if (d < tot) {
-        const uint64_t o = dst + d;
-        out.det[o] = r[u].x;
-        out.first[o] = (uint16_t)(r[u].y & 0xFFFFu);
-        out.width[o] = (uint16_t)(r[u].y >> 16);
-        out.charge[o] = r[u].z;
-        out.barycenter[o] = __uint_as_float(r[u].w);
+      for (int u = 0; u < kU; u++) {
+        const uint32_t d = d0 + u * blockDim.x;
+        if (d < m1) {
+          if (PACKED) {
+            const uint32_t lo = r[u].x & 255u, wd = ((r[u].x >> 8) & 255u) + 1u, q = r[u].x >> 16;
+            det[d] = r[u].z + (r[u].y >> 24);
+            first[d] = (uint16_t)lo;
+            width[d] = (uint16_t)wd;
+            charge[d] = q;
+            bary[d] = centroid(lo, wd, q, r[u].y & 0xFFFFFFu);
+          } else {
+            det[d] = r[u].x;
+            first[d] = (uint16_t)(r[u].y & 0xFFFFu);
+            width[d] = (uint16_t)(r[u].y >> 16);
+            charge[d] = r[u].z;
+            bary[d] = __uint_as_float(r[u].w);
+          }
+        }
       }
     }
   }
@@ -1046,6 +1096,119 @@ __global__ void __launch_bounds__(256, 4) k_batch(const uint8_t* __restrict__ ra
   pdl_release();
 }
 
+// One slot's FE unit `u` of FED item (event, FED), as the prologue described it.
+__device__ __forceinline__ cs::SlotSrc slot_src(const uint8_t* __restrict__ raw, const uint64_t* __restrict__ fed_off,
+                                                const uint2* __restrict__ unit_desc, size_t item, uint32_t u) {
+  const uint2 d = unit_desc[item * kFe + u];
+  const uint64_t fo = fed_off[item];
+  cs::SlotSrc r{raw, 0u, (d.y >> 16) & 255u, ((d.y >> 24) & 1u) != 0u};
+  if (r.data && fo != kBadOff) {
+    r.src = raw + fo + d.x;
+    r.len = d.y & 0xFFFFu;
+  }
+  return r;
+}
+
+// a7: the FE units of a batch of many events.  A CTA of W warps holds the
+// calibration entries of C = 3 W / 2 channels (24 KB for W = 8: one FE unit) in
+// shared memory and runs every event's records of those channels against them, 4 U
+// events per warp at a time.
+//
+// Bound by instruction issue (about 70% of the slots) and shared-memory latency.  On
+// 64 full-detector events (79.5 MB of records, 29.4 M digis) it takes 185 us where
+// k_batch, which finds each digi's run and candidate by warp ballots, takes 351: 5,460
+// against 11,700 warp instructions per 96 channels, and the calibration is read from
+// DRAM once (86 MB) instead of gathered from L2 digi by digi (840 MB of sectors).
+// What the tile costs is its load, so it needs events to share it (kStreamEvents).
+template <int W, int U>
+__global__ void __launch_bounds__(W * 32, 32 / W) k_stream(const uint8_t* __restrict__ raw,
+                                                           const uint64_t* __restrict__ fed_off, uint32_t n_events,
+                                                           uint32_t n_feds, const uint64_t* __restrict__ clu_off,
+                                                           uint64_t out_cap, sst_event_status* status, KParams kp,
+                                                           uint4* stage, uint32_t* ev_alloc, uint32_t* seg_cnt,
+                                                           uint32_t* seg_start, uint32_t* ticket,
+                                                           const uint2* __restrict__ unit_desc, uint32_t per_warp,
+                                                           uint32_t resident) {
+  constexpr int C = 3 * W / 2, kParts = kChPerFe / C;  // channels of the tile, tiles per FE unit
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint2* tile = reinterpret_cast<uint2*>(smem_raw);
+  cs::WarpT<U>* warps = reinterpret_cast<cs::WarpT<U>*>(smem_raw + sizeof(uint2) * C * kStrips);
+  __shared__ int2 mul[C];
+  __shared__ uint32_t s_next;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  cs::WarpT<U>& w = warps[warp];
+  uint4* spill = kp.spill + (size_t)(blockIdx.x * W + warp) * kSpillRecords;
+  const uint32_t n_tiles = n_feds * kFe * kParts;
+  // Tiles: the CTAs that fit the GPU at once (`resident`) start on the tile of their
+  // own index, while the prologue still runs; all further tiles come from the ticket.
+  bool first = true, fresh = true;
+  cs::SlotSrc src{raw, 0u, 0u, false};
+  uint32_t t = blockIdx.x;
+  if (t >= resident) {
+    pdl_wait();
+    first = false;
+    if (threadIdx.x == 0) s_next = resident + atomicAdd(ticket, 1u);
+    __syncthreads();
+    t = s_next;
+    __syncthreads();
+  }
+  while (t < n_tiles) {
+    const uint32_t fu = t / kParts;                                       // FE unit of the detector
+    const uint32_t ch0 = fu * kChPerFe + (t % kParts) * C;                // first channel of the tile
+    const uint8_t* g = reinterpret_cast<const uint8_t*>(kp.calq + (size_t)ch0 * kStrips);
+    for (uint32_t i = threadIdx.x; i < C * kStrips * sizeof(uint2) / 16; i += W * 32)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                       (uint32_t)__cvta_generic_to_shared(smem_raw + 16 * i)),
+                   "l"(g + 16 * i)
+                   : "memory");
+    int2 m2 = make_int2(0, 0);
+    if (threadIdx.x < C) mul[threadIdx.x] = m2 = __ldg(reinterpret_cast<const int2*>(kp.mul) + ch0 + threadIdx.x);
+    if (first) pdl_wait();  // the prologue's tickets, offsets, unit descriptors and counts
+    first = false;
+    if (threadIdx.x == 0) s_next = resident + atomicAdd(ticket, 1u);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    const bool any_div = __syncthreads_or(m2.x < 0 || m2.y < 0);
+    const uint32_t next = s_next;
+    for (uint32_t e0 = warp * per_warp; e0 < n_events; e0 += W * per_warp) {
+      const uint32_t n = n_events - e0 < per_warp ? n_events - e0 : per_warp;
+      const uint32_t e = e0 + (lane < (int)n ? lane : 0);
+      if (fresh && lane < (int)n) src = slot_src(raw, fed_off, unit_desc, (size_t)e * n_feds + fu / kFe, fu % kFe);
+      if (lane >= (int)n) src = cs::SlotSrc{raw, 0u, 0u, false};
+      // what this warp takes next: the same events' records of the next tile, or the next
+      // events' of this one
+      const bool same = e0 + W * per_warp < n_events;
+      const uint32_t fu2 = same ? fu : next / kParts, e2 = (same ? e0 + W * per_warp : warp * per_warp) + lane;
+      cs::SlotSrc src2{raw, 0u, 0u, false};
+      if (lane < (int)per_warp && e2 < n_events && fu2 < n_feds * kFe)
+        src2 = slot_src(raw, fed_off, unit_desc, (size_t)e2 * n_feds + fu2 / kFe, fu2 % kFe);
+      cs::process_slots<C>(
+          w, (int)n, (int)(t % kParts) * C, src, e, (((size_t)e * n_feds + fu / kFe) * kFe + fu % kFe) * kParts + t % kParts,
+          kp, clu_off, out_cap, status, reinterpret_cast<uint2*>(stage), ev_alloc, seg_cnt, seg_start, spill, tile, mul,
+          any_div, ch0, [&] {
+            // its bytes on their way to L2 (up to 512 a unit)
+            const int s = lane >> 2;
+            const uint8_t* g = reinterpret_cast<const uint8_t*>(
+                                   __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(src2.src), s)) +
+                               128 * (lane & 3);
+            const uint32_t len = __shfl_sync(0xffffffffu, src2.len, s);
+            if (128u * (lane & 3) < len) asm volatile("prefetch.global.L2 [%0];" ::"l"(g));
+          });
+      src = src2;
+      fresh = false;
+    }
+    // the next tile's calibration entries
+    if (next < n_tiles) {
+      const uint8_t* g2 = reinterpret_cast<const uint8_t*>(
+          kp.calq + ((size_t)(next / kParts) * kChPerFe + (next % kParts) * C) * kStrips);
+      for (uint32_t i = threadIdx.x; i < C * kStrips * sizeof(uint2) / 128; i += W * 32)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(g2 + 128 * i));
+    }
+    __syncthreads();
+    t = next;
+  }
+  pdl_release();
+}
+
 // Host batches with amplitudes: the chunk's amp_first values index the chunk's
 // amplitude arena; adding the chunk's first byte in the caller's array makes them
 // absolute.  The first *count records are rebased (kNoAmp stays).
@@ -1063,6 +1226,36 @@ __global__ void k_badmask(const uint8_t* __restrict__ bad, uint32_t* __restrict_
   uint32_t m = 0;
   for (int b = 0; b < 32; b++) m |= (bad[w * 32 + b] != 0 ? 1u : 0u) << b;
   mask[w] = m;
+}
+
+// Per APV, the charge multiplier of the clusterizers: M with (adc * M + 2^21) >> 22
+// equal, for every ADC 1..253, to the ADC divided by the APV's gain, rounded half
+// up and capped at 254, each operation one binary32 rounding (section 2: charge
+// corrected by the strip's gain); checked here for all of them.  Of U[0.8, 1.2]
+// gains all but 5 in 100,000 have one within 4 of 2^22 / gain (a quotient that
+// rounds up to a half has none); for those, and for gains below 1/4, where the
+// product would pass 32 bits, the bits of -gain: the kernels then divide.
+__global__ void k_gain_pack(const float* __restrict__ gain, int32_t* __restrict__ mul, uint32_t n_apv) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n_apv) return;
+  const float g = gain[i];
+  int32_t found = __float_as_int(-g);
+  if (g >= 0.2500005f) {
+    const int32_t m0 = __float2int_rn(__fdiv_rn((float)(1u << kMulShift), g));
+    for (int k = 0; k < 9 && found < 0; k++) {
+      const int32_t m = m0 + ((k & 1) ? (k + 1) / 2 : -(k / 2));
+      if (m < 0) continue;
+      bool ok = true;
+      for (uint32_t a = 1; a < 254u && ok; a++) {
+        const float y = __fadd_rn(__fdiv_rn((float)a, g), 0.5f);
+        const uint32_t want = y >= 254.f ? 254u : (uint32_t)y;
+        const uint32_t q = (a * (uint32_t)m + (1u << (kMulShift - 1))) >> kMulShift;
+        ok = (q < 254u ? q : 254u) == want;
+      }
+      if (ok) found = m;
+    }
+  }
+  mul[i] = found;
 }
 
 // The per-strip calibration word the clusterizers read, built once per upload:
@@ -1243,6 +1436,25 @@ cudaError_t launch_cluster_fe(const sst_digis& in, uint32_t n_feds, const KParam
   return cudaGetLastError();
 }
 
+template <int W, int U>
+cudaError_t stream_grid(const Shape& sh, uint32_t n_feds, int n_sm, int* grid, int* resident, size_t* smem) {
+  *smem = sizeof(uint2) * (3 * W / 2) * kStrips + W * sizeof(cs::WarpT<U>);
+  int per_sm = 0;
+  cudaError_t e = prepare((const void*)k_stream<W, U>, W * 32, *smem, &per_sm);
+  if (e) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const size_t tiles = (size_t)n_feds * kFe * (8 / W);
+  const size_t ctas = (size_t)n_sm * (sh.ctas_per_sm < kMaxWarpsPerSm / W ? sh.ctas_per_sm : kMaxWarpsPerSm / W), fit = (size_t)n_sm * per_sm;
+  *grid = (int)(ctas < tiles ? ctas : tiles);
+  *resident = (int)(fit < (size_t)*grid ? fit : (size_t)*grid);
+  return cudaSuccess;
+}
+
+// Batches of at least this many events without amplitudes take k_stream: a tile is
+// 24 KB and an event's gathers of the same channels about 4 KB.
+constexpr uint32_t kStreamEvents = 8;
+bool use_stream(uint32_t n_events, bool amps) { return !amps && n_events >= kStreamEvents; }
+
 template <bool AMP, int U>
 cudaError_t launch_batch_t(const uint8_t* raw, const uint32_t* fed_len, uint32_t n_events, uint32_t n_feds,
                            const uint64_t* clu_off, uint64_t out_cap, sst_event_status* status, const KParams& kp,
@@ -1271,13 +1483,38 @@ cudaError_t launch_batch_t(const uint8_t* raw, const uint32_t* fed_len, uint32_t
   return cudaGetLastError();
 }
 
+template <int W, int U>
+cudaError_t launch_stream_t(const uint8_t* raw, uint32_t n_events, uint32_t n_feds, const uint64_t* clu_off,
+                            uint64_t out_cap, sst_event_status* status, const KParams& kp, const Scratch& s,
+                            const Shape& sh, int n_sm, cudaStream_t st) {
+  int grid = 0, resident = 0;
+  size_t sm = 0;
+  cudaError_t e = stream_grid<W, U>(sh, n_feds, n_sm, &grid, &resident, &sm);
+  if (e) return e;
+  const KParams kps = with_spill(kp, s);
+  if ((size_t)grid * W > s.spill_warps) return cudaErrorInvalidConfiguration;
+  // events per warp and pass over the tile (at most 32, one lane each): all warps of the CTA busy
+  const uint32_t passes = (n_events + W * 32 - 1) / (W * 32);
+  const uint32_t per_warp = (n_events + W * passes - 1) / (W * passes);
+  return launch_pdl(k_stream<W, U>, (unsigned)grid, (unsigned)(W * 32), sm, st, raw, (const uint64_t*)s.fed_off,
+                    n_events, n_feds, clu_off, out_cap, status, kps, s.stage, s.ev_alloc, s.fed_cnt, s.fed_start,
+                    s.tickets, (const uint2*)s.unit_desc, per_warp, (uint32_t)resident);
+}
+
 cudaError_t launch_batch_fe(const uint8_t* raw, const uint32_t* fed_len, uint32_t n_events, uint32_t n_feds,
                             const uint64_t* clu_off, uint64_t out_cap, sst_event_status* status, const KParams& kp,
                             const Scratch& s, const Shape& sh, int n_sm, const AmpArgs& am, cudaStream_t st,
                             cudaEvent_t ev_begin, cudaEvent_t ev_end) {
   cudaError_t e;
   if (ev_begin && (e = cudaEventRecord(ev_begin, st))) return e;
-  if (sh.units == 1)
+  if (use_stream(n_events, am.stage != nullptr)) {
+    if (sh.block == 128)
+      e = sh.units == 1 ? launch_stream_t<4, 1>(raw, n_events, n_feds, clu_off, out_cap, status, kp, s, sh, n_sm, st)
+                        : launch_stream_t<4, 2>(raw, n_events, n_feds, clu_off, out_cap, status, kp, s, sh, n_sm, st);
+    else
+      e = sh.units == 1 ? launch_stream_t<8, 1>(raw, n_events, n_feds, clu_off, out_cap, status, kp, s, sh, n_sm, st)
+                        : launch_stream_t<8, 2>(raw, n_events, n_feds, clu_off, out_cap, status, kp, s, sh, n_sm, st);
+  } else if (sh.units == 1)
     e = am.stage ? launch_batch_t<true, 1>(raw, fed_len, n_events, n_feds, clu_off, out_cap, status, kp, s, sh, n_sm, am, st)
                  : launch_batch_t<false, 1>(raw, fed_len, n_events, n_feds, clu_off, out_cap, status, kp, s, sh, n_sm, am, st);
   else
@@ -1288,10 +1525,11 @@ cudaError_t launch_batch_fe(const uint8_t* raw, const uint32_t* fed_len, uint32_
   return cudaSuccess;
 }
 
-// Per-event cluster order and the copy into the caller's SoA.
+// Per-event cluster order and the copy into the caller's SoA.  chans: channels per
+// segment when the records are staged packed (k_stream), else 0.
 cudaError_t launch_order(const uint64_t* clu_off, uint32_t n_events, uint32_t n_segs, const sst_clusters& out,
                          sst_event_status* status, const Scratch& s, uint64_t* pack_off, const AmpArgs& am,
-                         cudaStream_t st) {
+                         cudaStream_t st, uint32_t chans = 0) {
   cudaError_t e;
   if (am.stage || pack_off) {
     k_clu_scan<<<n_events, 1024, 0, st>>>(s.fed_cnt, n_segs, s.fed_dest, status, pack_off, s.tickets + 1, am);
@@ -1302,21 +1540,18 @@ cudaError_t launch_order(const uint64_t* clu_off, uint32_t n_events, uint32_t n_
     k_compact<<<(unsigned)((items + 7) / 8), 256, 0, st>>>(s.stage, clu_off, pack_off, s.fed_cnt, s.fed_start,
                                                           s.fed_dest, n_events, n_segs, out, am);
   } else {
-    // 64 segments per CTA for a batch; 16 when that would give a small grid (one
+    // 64 segments per CTA (128 of the shorter ones of k_stream) for a batch; 16 when that would give a small grid (one
     // event, a short chunk), so that enough CTAs share the copy
-    const uint32_t cpe64 = (n_segs + 63) / 64;
+    const uint32_t many = chans ? 128u : 64u, cpe64 = (n_segs + many - 1) / many;
     const uint4* stage = s.stage;
     const uint64_t* pack = pack_off;
     const uint32_t* cnt = s.fed_cnt;
     const uint32_t* start = s.fed_start;
-    if ((uint64_t)n_events * cpe64 >= 256) {
-      e = launch_pdl(k_order<64>, (unsigned)((uint64_t)n_events * cpe64), 256u, 0, st, stage, clu_off, pack, cnt, start,
-                     n_segs, cpe64, out, status);
-    } else {
-      const uint32_t cpe16 = (n_segs + 15) / 16;
-      e = launch_pdl(k_order<16>, (unsigned)((uint64_t)n_events * cpe16), 256u, 0, st, stage, clu_off, pack, cnt, start,
-                     n_segs, cpe16, out, status);
-    }
+    const bool wide = (uint64_t)n_events * cpe64 >= 256;
+    const uint32_t cpe = wide ? cpe64 : (n_segs + 15) / 16;
+    auto* k = chans ? (wide ? k_order<128, true> : k_order<16, true>) : (wide ? k_order<64, false> : k_order<16, false>);
+    e = launch_pdl(k, (unsigned)((uint64_t)n_events * cpe), 256u, 0, st, stage, clu_off, pack, cnt, start, n_segs, cpe,
+                   out, status, chans);
     if (e) return e;
   }
   return cudaGetLastError();
@@ -1352,6 +1587,15 @@ bool shape_valid(const Shape& s) {
 
 cudaError_t batch_launch_info(const Shape& sh, uint32_t n_events, uint32_t n_feds, int n_sm, int* grid, size_t* smem,
                               int* items_per_fed) {
+  *items_per_fed = kFe / sh.units;
+  if (use_stream(n_events, false)) {
+    int resident = 0;
+    if (sh.block == 128)
+      return sh.units == 1 ? stream_grid<4, 1>(sh, n_feds, n_sm, grid, &resident, smem)
+                           : stream_grid<4, 2>(sh, n_feds, n_sm, grid, &resident, smem);
+    return sh.units == 1 ? stream_grid<8, 1>(sh, n_feds, n_sm, grid, &resident, smem)
+                         : stream_grid<8, 2>(sh, n_feds, n_sm, grid, &resident, smem);
+  }
   const size_t sm = batch_smem(sh.units, sh.block);
   const void* fn = sh.units == 1 ? (const void*)k_batch<false, 1> : (const void*)k_batch<false, 2>;
   int per_sm = 0;
@@ -1363,7 +1607,6 @@ cudaError_t batch_launch_info(const Shape& sh, uint32_t n_events, uint32_t n_fed
   const size_t need = (units + nw - 1) / nw;
   *grid = (int)(ctas < need ? ctas : need);
   *smem = sm;
-  *items_per_fed = kFe / sh.units;
   return cudaSuccess;
 }
 
@@ -1409,7 +1652,10 @@ cudaError_t launch_batch(const uint8_t* raw, const uint64_t* event_off, const ui
   e = launch_batch_fe(raw, fed_len, n_events, n_feds, clu_off, out.capacity, status, kp, s, sh, n_sm, am, st,
                       ev_begin, ev_end);
   if (e) return e;
-  return launch_order(clu_off, n_events, n_feds * (kFe / (sh.units == 1 ? 1 : 2)), out, status, s, pack_off, am, st);
+  const bool stream = use_stream(n_events, am.stage != nullptr);
+  const uint32_t per_fed = stream ? kFe * (256 / sh.block) : kFe / sh.units;
+  return launch_order(clu_off, n_events, n_feds * per_fed, out, status, s, pack_off, am, st,
+                      stream ? (uint32_t)kCh / per_fed : 0u);
 }
 
 cudaError_t rebase_amp_first(uint32_t* amp_first, const uint64_t* count, uint32_t base, int n_sm, cudaStream_t st) {
@@ -1420,6 +1666,11 @@ cudaError_t rebase_amp_first(uint32_t* amp_first, const uint64_t* count, uint32_
 cudaError_t build_badmask(const uint8_t* bad_dev, uint32_t* mask_dev, uint64_t n_strips, cudaStream_t st) {
   const uint64_t words = n_strips / 32;
   k_badmask<<<(unsigned)((words + 255) / 256), 256, 0, st>>>(bad_dev, mask_dev, words);
+  return cudaGetLastError();
+}
+
+cudaError_t build_gain(const float* gain_dev, int32_t* mul_dev, uint32_t n_apv, cudaStream_t st) {
+  k_gain_pack<<<(n_apv + 127) / 128, 128, 0, st>>>(gain_dev, mul_dev, n_apv);
   return cudaGetLastError();
 }
 
