@@ -14,7 +14,7 @@ BUILD_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libsst.so")
 SOURCES = ["sst_kernels.cu", "sst_api.cu", "sst_server.cpp", "sst_host.cpp", "sst_noalloc.cu", "sst_geom.cu",
            "sst_load.cpp"]
-HEADERS = ["sst_internal.h", "sst_fe.cuh", "sst_stream.cuh"]
+HEADERS = ["sst_internal.h", "sst_stream.cuh", "sst_event.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

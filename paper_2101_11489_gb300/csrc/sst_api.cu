@@ -23,52 +23,11 @@ sst_status cuda_err(sst_ctx* c, cudaError_t e, const char* where) {
 KParams kparams(const sst_ctx* c) {
   KParams k;
   k.t_cluster = c->params.t_cluster;
-  k.max_holes = c->params.max_seq_holes;
-  k.max_bad = c->params.max_seq_bad;
   k.max_adj = c->params.max_adj_bad;
   k.calq = c->calq;
   k.badmask = c->badmask;
-  k.qmul = c->qmul;
   k.mul = c->mul;
   return k;
-}
-
-// Gain-corrected charge of a non-saturated ADC (section 2: charge corrected by the
-// strip's gain): the ADC divided by the APV gain, rounded half up, capped at 254;
-// each operation one binary32 rounding.  `mul` selects the form the kernels use
-// with a certified multiplier m: the ADC times m instead of divided by the gain.
-static uint32_t charge_of(uint32_t adc, float g, bool mul) {
-  const float a = (float)adc;
-  const float x = mul ? a * g : a / g;
-  const float y = x + 0.5f;
-  return y >= 254.0f ? 254u : (uint32_t)y;  // (uint32_t)y truncates; y >= 0
-}
-
-// A multiplier for one APV: the binary32 reciprocal of the gain, or a neighbour of
-// it within a few units in the last place, that gives exactly the quotient form's
-// charge for every ADC 0..253 (checked here, exhaustively).  When none does, -gain:
-// the kernels then divide.  Needs binary32 arithmetic without contraction (the
-// library's host code is compiled with -ffp-contract=off).
-static float certified_multiplier(float g) {
-  uint32_t want[254];
-  for (uint32_t a = 0; a < 254; a++) want[a] = charge_of(a, g, false);
-  const float r = 1.0f / g;
-  float cand[9];
-  cand[0] = r;
-  float up = r, dn = r;
-  for (int k = 1; k <= 4; k++) {
-    up = std::nextafter(up, INFINITY);
-    dn = std::nextafter(dn, 0.0f);
-    cand[2 * k - 1] = up;
-    cand[2 * k] = dn;
-  }
-  for (float m : cand) {
-    if (!(m > 0.f) || !std::isfinite(m)) continue;
-    bool ok = true;
-    for (uint32_t a = 1; a < 254 && ok; a++) ok = charge_of(a, m, true) == want[a];
-    if (ok) return m;
-  }
-  return -g;
 }
 
 template <typename T>
@@ -80,6 +39,22 @@ static cudaError_t grow(T*& p, size_t& cap, size_t need) {
   cudaError_t e = cudaMalloc(&p, need * sizeof(T));
   if (e == cudaSuccess) cap = need;
   return e;
+}
+
+// Two cleared sets of shared state for `events` events of `feds` FEDs in all.
+static cudaError_t grow_look(LookState& l, size_t events, size_t feds) {
+  const size_t words = LookState::words_for(events, 1) + feds + 3 * (feds / 1024 + 1);
+  if (words <= l.cap) return cudaSuccess;
+  const bool replayed = l.replayed;
+  if (l.words) cudaFree(l.words);
+  l = LookState{};
+  cudaError_t e = cudaMalloc(&l.words, 2 * words * sizeof(*l.words));
+  if (!e) e = cudaMemset(l.words, 0, 2 * words * sizeof(*l.words));
+  if (!e) e = cudaDeviceSynchronize();  // cleared for every stream
+  if (e) return e;
+  l.cap = words;
+  l.replayed = replayed;
+  return cudaSuccess;
 }
 
 cudaError_t ensure_scratch(Scratch& s, size_t items, size_t events, size_t stage_records) {
@@ -95,19 +70,16 @@ cudaError_t ensure_scratch(Scratch& s, size_t items, size_t events, size_t stage
     // growing: wait for all work that may still use the old buffers
     if ((e = cudaDeviceSynchronize())) return e;
     if (items > s.items_cap) {
-      size_t cap = s.items_cap, c2 = s.items_cap, c3 = s.items_cap, c4 = s.items_cap, c5 = s.items_cap;
-      size_t c6 = s.items_cap, c7 = s.items_cap;
-      if ((e = grow(s.lb, cap, items))) return e;
-      if ((e = grow(s.fed_off, c2, items))) return e;
-      if ((e = grow(s.fed_cnt, c3, 2 * items))) return e;
-      if ((e = grow(s.fed_start, c4, 2 * items))) return e;
-      if ((e = grow(s.fed_dest, c5, 2 * items))) return e;
-      if ((e = grow(s.unit_desc, c6, items))) return e;
-      if ((e = grow(s.big_list, c7, items))) return e;
+      size_t c1 = s.items_cap, c2 = s.items_cap, c3 = s.items_cap, c4 = s.items_cap;
+      if ((e = grow(s.fed_off, c1, items))) return e;
+      if ((e = grow(s.fed_cnt, c2, 2 * items))) return e;  // two segments per FE unit at most
+      if ((e = grow(s.fed_start, c3, 2 * items))) return e;
+      if ((e = grow(s.unit_desc, c4, items))) return e;
       s.items_cap = items;
     }
     if ((e = grow(s.ev_alloc, s.ev_cap, events))) return e;
     if ((e = grow(s.stage, s.stage_cap, stage_records))) return e;
+    if ((e = grow_look(s.look, s.ev_cap, s.items_cap / kFe))) return e;
   }
   return cudaSuccess;
 }
@@ -124,39 +96,16 @@ cudaError_t ensure_spill(Scratch& s, size_t warps) {
   return cudaSuccess;
 }
 
-cudaError_t ensure_amp_scratch(Scratch& s, size_t items, size_t events, size_t amp_bytes) {
-  items = items ? items : 1;
-  events = events ? events : 1;
-  amp_bytes = amp_bytes ? amp_bytes : 1;
-  if (items <= s.amp_items_cap && events <= s.amp_ev_cap && amp_bytes <= s.amp_stage_cap) return cudaSuccess;
-  cudaError_t e = cudaDeviceSynchronize();  // growing: wait for all work that may still use the old buffers
-  if (e) return e;
-  if (items > s.amp_items_cap) {
-    size_t c1 = s.amp_items_cap, c2 = s.amp_items_cap, c3 = s.amp_items_cap;
-    if ((e = grow(s.seg_amp_cnt, c1, items))) return e;
-    if ((e = grow(s.seg_amp_start, c2, items))) return e;
-    if ((e = grow(s.seg_amp_dest, c3, items))) return e;
-    s.amp_items_cap = items;
-  }
-  if ((e = grow(s.amp_alloc, s.amp_ev_cap, events))) return e;
-  return grow(s.amp_stage, s.amp_stage_cap, amp_bytes);
-}
-
 void free_scratch(Scratch& s) {
-  if (s.lb) cudaFree(s.lb);
+  if (s.look.words) cudaFree(s.look.words);
   if (s.fed_off) cudaFree(s.fed_off);
   if (s.fed_cnt) cudaFree(s.fed_cnt);
   if (s.fed_start) cudaFree(s.fed_start);
-  if (s.fed_dest) cudaFree(s.fed_dest);
   if (s.unit_desc) cudaFree(s.unit_desc);
-  if (s.big_list) cudaFree(s.big_list);
   if (s.ev_alloc) cudaFree(s.ev_alloc);
   if (s.stage) cudaFree(s.stage);
   if (s.tickets) cudaFree(s.tickets);
   if (s.spill) cudaFree(s.spill);
-  for (void* p : {(void*)s.amp_stage, (void*)s.amp_alloc, (void*)s.seg_amp_cnt, (void*)s.seg_amp_start,
-                  (void*)s.seg_amp_dest})
-    if (p) cudaFree(p);
   s = Scratch{};
 }
 
@@ -185,7 +134,7 @@ sst_status sst_create(sst_ctx** out, int device, uint32_t n_feds) {
   c->shape = default_shape();
   DeviceGuard g(device);
   cudaError_t e = cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, device);
-  if (e == cudaSuccess) e = ensure_scratch(c->scratch, (size_t)n_feds, 1, 1);
+  if (e == cudaSuccess) e = ensure_scratch(c->scratch, (size_t)n_feds * kFe, 1, 1);
   if (e != cudaSuccess) {
     free_scratch(c->scratch);
     delete c;
@@ -211,7 +160,6 @@ sst_status sst_destroy(sst_ctx* ctx) {
   free_scratch(ctx->scratch);
   if (ctx->calq) cudaFree(ctx->calq);
   if (ctx->badmask) cudaFree(ctx->badmask);
-  if (ctx->qmul) cudaFree(ctx->qmul);
   if (ctx->mul) cudaFree(ctx->mul);
   if (ctx->pitch) cudaFree(ctx->pitch);
   delete ctx;
@@ -238,15 +186,12 @@ sst_status sst_calib_upload(sst_ctx* ctx, const float* noise, const float* gain,
   for (uint64_t i = 0; i < n_apv; i++)
     if (!(gain[i] > 0.f) || !std::isfinite(gain[i]))
       return set_err(ctx, SST_ERR_INVALID_ARG, "sst_calib_upload: gain must be finite and > 0");
-  std::vector<float> qmul(n_apv);
-  for (uint64_t i = 0; i < n_apv; i++) qmul[i] = certified_multiplier(gain[i]);
   DeviceGuard g(ctx->device);
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e = cudaSuccess;
   if (!ctx->calq) {
     if ((e = cudaMalloc(&ctx->calq, n * sizeof(uint2)))) return cuda_err(ctx, e, "cudaMalloc calq");
     if ((e = cudaMalloc(&ctx->badmask, n / 8))) return cuda_err(ctx, e, "cudaMalloc badmask");
-    if ((e = cudaMalloc(&ctx->qmul, n_apv * sizeof(float)))) return cuda_err(ctx, e, "cudaMalloc qmul");
     if ((e = cudaMalloc(&ctx->mul, n_apv * sizeof(int32_t)))) return cuda_err(ctx, e, "cudaMalloc mul");
   }
   // staging of the raw tables, freed once the kernels' tables are built
@@ -265,7 +210,6 @@ sst_status sst_calib_upload(sst_ctx* ctx, const float* noise, const float* gain,
   // Copies are stream-ordered after earlier work on `st`; synchronise before the
   // host buffers go out of the caller's hands and before freeing the staging.
   if (!e) e = cudaMemcpyAsync(noise_dev, noise, n * sizeof(float), cudaMemcpyHostToDevice, st);
-  if (!e) e = cudaMemcpyAsync(ctx->qmul, qmul.data(), n_apv * sizeof(float), cudaMemcpyHostToDevice, st);
   if (!e) e = cudaMemcpyAsync(bad_dev, bad, n, cudaMemcpyHostToDevice, st);
   if (!e) e = cudaMemcpyAsync(gain_dev, gain, n_apv * sizeof(float), cudaMemcpyHostToDevice, st);
   if (!e) e = build_gain(gain_dev, ctx->mul, (uint32_t)n_apv, st);
@@ -290,7 +234,7 @@ sst_status sst_unpack(sst_ctx* ctx, const uint8_t* raw, uint64_t raw_bytes, cons
   if (n_feds == 0 || n_feds > ctx->n_feds)
     return set_err(ctx, SST_ERR_INVALID_ARG, "sst_unpack: n_feds outside 1..context FEDs");
   DeviceGuard g(ctx->device);
-  cudaError_t e = ensure_scratch(ctx->scratch, n_feds, 1, 1);
+  cudaError_t e = ensure_scratch(ctx->scratch, (size_t)n_feds * kFe, 1, 1);
   if (e) return cuda_err(ctx, e, "sst_unpack scratch");
   e = launch_unpack(raw, raw_bytes, fed_len, n_feds, *out, ctx->scratch, ctx->shape, (cudaStream_t)stream);
   return cuda_err(ctx, e, "sst_unpack");
@@ -307,11 +251,9 @@ sst_status sst_cluster(sst_ctx* ctx, const sst_digis* in, uint32_t n_feds, const
   if (out->amp && (!out->amp_first || out->amp_capacity == 0 || out->amp_capacity >= kNoAmp))
     return set_err(ctx, SST_ERR_INVALID_ARG, "sst_cluster: amp needs amp_first and 1 <= amp_capacity < 2^32 - 1");
   DeviceGuard g(ctx->device);
-  cudaError_t e = ensure_scratch(ctx->scratch, (size_t)n_feds * kFe, 1, out->capacity);
-  if (!e && out->amp) e = ensure_amp_scratch(ctx->scratch, (size_t)n_feds * kFe, 1, out->amp_capacity);
-  if (!e) e = ensure_spill(ctx->scratch, (size_t)n_feds * kFe);
+  cudaError_t e = ensure_scratch(ctx->scratch, (size_t)n_feds * kFe, 1, 1);
   if (e) return cuda_err(ctx, e, "sst_cluster scratch");
-  e = launch_cluster(*in, n_feds, *out, kparams(ctx), ctx->scratch, ctx->shape, (cudaStream_t)stream);
+  e = launch_cluster(*in, n_feds, *out, kparams(ctx), ctx->scratch, (cudaStream_t)stream);
   return cuda_err(ctx, e, "sst_cluster");
 }
 
@@ -334,7 +276,6 @@ sst_status sst_batch(sst_ctx* ctx, const uint8_t* raw, const uint64_t* event_off
   DeviceGuard g(ctx->device);
   const size_t items = (size_t)n_events * n_feds;
   cudaError_t e = ensure_scratch(ctx->scratch, items * kFe, n_events, out->capacity);
-  if (!e && out->amp) e = ensure_amp_scratch(ctx->scratch, items * kFe, n_events, out->amp_capacity);
   if (!e) e = ensure_spill(ctx->scratch, (size_t)ctx->n_sm * kMaxWarpsPerSm);
   if (e) return cuda_err(ctx, e, "sst_batch scratch");
   cudaEvent_t eb = nullptr, ee = nullptr;
@@ -421,12 +362,12 @@ sst_status sst_get_tune(const sst_ctx* ctx, sst_tune* t) {
 sst_status sst_get_launch_info(sst_ctx* ctx, uint32_t n_events, uint32_t n_feds, sst_launch_info* info) {
   if (!ctx || !info || n_events == 0 || n_feds == 0) return SST_ERR_INVALID_ARG;
   DeviceGuard g(ctx->device);
-  int grid = 0, ipf = 0;
+  int grid = 0, block = 0, ipf = 0;
   size_t smem = 0;
-  const cudaError_t e = batch_launch_info(ctx->shape, n_events, n_feds, ctx->n_sm, &grid, &smem, &ipf);
+  const cudaError_t e = batch_launch_info(ctx->shape, n_events, n_feds, ctx->n_sm, &grid, &smem, &block, &ipf);
   if (e) return cuda_err(ctx, e, "sst_get_launch_info");
   info->grid = (uint32_t)grid;
-  info->block = (uint32_t)ctx->shape.block;
+  info->block = (uint32_t)block;
   info->smem_bytes = (uint32_t)smem;
   info->items_per_fed = (uint32_t)ipf;
   info->host_chunks = host_chunks(n_events, ctx->shape.host_chunk);
@@ -464,9 +405,9 @@ sst_status sst_autotune(sst_ctx* ctx, const uint8_t* raw, const uint64_t* event_
         s.units = u;
         s.ctas_per_sm = p;
         if (!shape_valid(s)) continue;
-        int grid = 0, ipf = 0;
+        int grid = 0, block = 0, ipf = 0;
         size_t smem = 0;
-        if ((ce = batch_launch_info(s, n_events, n_feds, ctx->n_sm, &grid, &smem, &ipf))) break;
+        if ((ce = batch_launch_info(s, n_events, n_feds, ctx->n_sm, &grid, &smem, &block, &ipf))) break;
         if (smem * (size_t)p > 227u * 1024u) continue;
         bool dup = false;  // the occupancy clamps p: the same launch was timed already
         for (auto& pr : timed)

@@ -20,24 +20,21 @@ namespace {
 constexpr uint32_t kMaxFeds = SST_NOALLOC_MAX_FEDS;
 constexpr int kMaxDevices = 64;
 
-// Scratch for one call: kMaxFeds look-back states, kMaxFeds FED byte offsets, and
-// 8 words of work tickets (16 KiB + 64 B).
-static __device__ __align__(256) unsigned long long g_scratch[2 * kMaxFeds + 8];
+// The launches' shared state: two sets (sst::LookState), about 16 KiB.
+constexpr size_t kWords = sst::LookState::words_for(1, kMaxFeds);
+static __device__ __align__(256) unsigned long long g_scratch[2 * kWords];
 
 std::mutex g_mu;
-void* g_addr[kMaxDevices];  // device address of g_scratch, per device, once known
+sst::Scratch g_state[kMaxDevices];  // per device; look.words is g_scratch's address there, once known
 
-// Device address of g_scratch on the current device (looked up on the first call
-// for that device).
-cudaError_t scratch_address(int dev, void** out) {
-  std::lock_guard<std::mutex> lock(g_mu);
-  if (!g_addr[dev]) {
-    void* p = nullptr;
-    const cudaError_t e = cudaGetSymbolAddress(&p, g_scratch);
-    if (e != cudaSuccess) return e;
-    g_addr[dev] = p;
-  }
-  *out = g_addr[dev];
+// Finds g_scratch's address on the current device (on the first call for that device).
+cudaError_t find_scratch(sst::LookState& l) {
+  if (l.words) return cudaSuccess;
+  void* p = nullptr;
+  const cudaError_t e = cudaGetSymbolAddress(&p, g_scratch);
+  if (e != cudaSuccess) return e;
+  l.words = static_cast<unsigned long long*>(p);
+  l.cap = kWords;
   return cudaSuccess;
 }
 
@@ -52,15 +49,9 @@ extern "C" sst_status sst_unpack_noalloc(const uint8_t* raw, uint64_t raw_bytes,
   if (n_feds > kMaxFeds) return SST_ERR_TOO_LARGE;
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return SST_ERR_CUDA;
-  void* base = nullptr;
-  if (scratch_address(dev, &base) != cudaSuccess) return SST_ERR_CUDA;
-  unsigned long long* words = static_cast<unsigned long long*>(base);
-  sst::Scratch s;
-  s.lb = words;
-  s.fed_off = reinterpret_cast<uint64_t*>(words + kMaxFeds);
-  s.tickets = reinterpret_cast<uint32_t*>(words + 2 * kMaxFeds);
-  // the launcher clears the look-back states, the tickets and the event status
-  // before its kernels run, on the caller's stream
+  std::lock_guard<std::mutex> lock(g_mu);
+  sst::Scratch& s = g_state[dev];
+  if (find_scratch(s.look) != cudaSuccess) return SST_ERR_CUDA;
   const cudaError_t e = sst::launch_unpack(raw, raw_bytes, fed_len, n_feds, *out, s, sst::default_shape(),
                                            static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? SST_OK : SST_ERR_CUDA;

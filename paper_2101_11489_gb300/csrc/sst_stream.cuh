@@ -71,6 +71,38 @@ struct List {
   }
 };
 
+// The cluster threshold: a cluster is kept when its raw charge s is larger than the
+// binary32 product t x sqrt(n2).  s^2 and t^2 n2 decide that whenever they differ by
+// more than four parts in a million (the roundings of either form stay below 2^-21
+// relative); the rest, and thresholds whose square leaves the normal range, take the
+// product.
+struct Threshold {
+  float t, t2, margin;
+  __device__ __forceinline__ explicit Threshold(float t_cluster) {
+    t = t_cluster;
+    t2 = __fmul_rn(t, t);
+    margin = t2 > 1e-20f && t2 < 1e20f ? 4e-6f : __int_as_float(0x7f800000);
+  }
+  __device__ __forceinline__ bool pass(uint32_t charge, float n2) const {
+    const float s = __uint2float_rn(charge), a = __fmul_rn(s, s), b = __fmul_rn(t2, n2);
+    bool p = a > b;
+    if (!(fabsf(__fsub_rn(a, b)) > __fmul_rn(margin, b))) p = s > __fmul_rn(t, __fsqrt_rn(n2));
+    return p;
+  }
+};
+
+// Gain-corrected charge (section 2): the ADC times the APV's certified fixed-point
+// multiplier m, half up (k_gain_pack); for the rare APV without one, m negative, the
+// bits of -gain: the quotient itself.  Capped at 254; saturation codes are kept.
+__device__ __forceinline__ uint32_t charge(uint32_t adc, int32_t m) {
+  uint32_t q = (adc * (uint32_t)m + (1u << (kMulShift - 1))) >> kMulShift;
+  if (m < 0) {
+    const float y = __fadd_rn(__fdiv_rn(__uint2float_rn(adc), -__int_as_float(m)), 0.5f);
+    q = y >= 254.f ? 254u : (uint32_t)y;
+  }
+  return adc >= 254u ? adc : (q < 254u ? q : 254u);
+}
+
 // A lane's place in its channel record and its open candidate.
 struct Walk {
   uint32_t p;          // next byte
@@ -247,15 +279,7 @@ __device__ void walk_any(Walk& k, const uint8_t* src, uint32_t end, const uint2*
     const bool start = act && s - k.last1 >= (c.x >> 16);
     list.append(start && k.seeded, k.record());
     if (act) {
-      const int32_t m = s < (uint32_t)kApv ? m0 : m1;
-      uint32_t q;
-      if (m >= 0) {
-        q = (a * (uint32_t)m + (1u << (kMulShift - 1))) >> kMulShift;
-      } else {  // no certified multiplier: the bits of -gain, and the quotient itself
-        const float y = __fadd_rn(__fdiv_rn(__uint2float_rn(a), -__int_as_float(m)), 0.5f);
-        q = y >= 254.f ? 254u : (uint32_t)y;
-      }
-      q = a >= 254u ? a : (q < 254u ? q : 254u);
+      const uint32_t q = charge(a, s < (uint32_t)kApv ? m0 : m1);
       if (start) {
         k.first = s + task17;
         k.sums = k.moment = k.seeded = 0;
@@ -284,28 +308,19 @@ __device__ __forceinline__ uint32_t stop_status(const Walk& k, uint32_t end, Rd 
 // Cluster threshold of every record and the kept ones' places within their
 // channel: record i's z becomes the number of kept records of its channel before
 // it, or kNotKept; w.kept counts them.  A channel's records are in strip order.
-//
-// A cluster is kept when its raw charge s is larger than the binary32 product
-// t x sqrt(n2).  s^2 and t^2 n2 decide that whenever they differ by more than four
-// parts in a million (every rounding of either form is below 2^-23 relative); the
-// rest, and thresholds whose square leaves the normal range, take the product.
 template <class W>
 __device__ __forceinline__ void rank_records(W& w, const List& list, float t_cluster) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   for (int i = lane; i < W::kTasks / 4; i += 32) reinterpret_cast<uint32_t*>(w.kept)[i] = 0;
   __syncwarp();
-  const float t2 = __fmul_rn(t_cluster, t_cluster);
-  const float margin = t2 > 1e-20f && t2 < 1e20f ? 4e-6f : __int_as_float(0x7f800000);
+  const Threshold thr(t_cluster);
   const uint4 none = make_uint4(0u, 0u, 0x7f800000u, 0u);
   uint4 ahead = (uint32_t)lane < list.n ? list.rec[lane] : none;
   for (uint32_t i = lane; i - lane < list.n; i += 32) {
     const uint4 r = ahead;
     if (i - lane + 32 < list.n) ahead = i + 32 < list.n ? list.rec[i + 32] : none;
-    const float s = __uint2float_rn(r.y & 0xFFFFu), n2 = __uint_as_float(r.z);
-    const float a = __fmul_rn(s, s), b = __fmul_rn(t2, n2);
-    bool pass = a > b;
-    if (!(fabsf(__fsub_rn(a, b)) > __fmul_rn(margin, b))) pass = s > __fmul_rn(t_cluster, __fsqrt_rn(n2));
+    const bool pass = thr.pass(r.y & 0xFFFFu, __uint_as_float(r.z));
     const uint32_t t = r.x >> 17;
     const unsigned same = __match_any_sync(0xffffffffu, pass ? t : 128u);
     const uint32_t rank = (pass ? (uint32_t)w.kept[t] : 0u) + __popc(same & lt);
@@ -395,12 +410,12 @@ struct SlotSrc {
   bool data;           // the FED record is there and its header is valid
 };
 
-// The channel length chain of one FE unit (the paper's map of channel locations):
-// each length at least 3, within the unit, and all of them adding up to the unit's
-// length; otherwise no channel of the unit is read.  Channels c0 .. c0 + C - 1 go to
-// out.  p: the unit's first byte.
-template <int C, typename Rd>
-__device__ __forceinline__ bool walk_lengths(uint32_t p, uint32_t len, int c0, uint32_t* out, Rd rd) {
+// The channel length chain of one FE unit of len bytes from p (the paper's map of
+// channel locations): each length at least 3, within the unit, and all of them adding
+// up to the unit's length; otherwise false, and no channel of the unit is read.
+// put(k, pos, length) takes channel k (it may have been called when the chain breaks).
+template <typename Rd, typename Put>
+__device__ __forceinline__ bool walk_lengths(uint32_t p, uint32_t len, Rd rd, Put put) {
   const uint32_t end = p + len;
   bool good = true;
 #pragma unroll
@@ -409,13 +424,12 @@ __device__ __forceinline__ bool walk_lengths(uint32_t p, uint32_t len, int c0, u
     uint32_t l = 0;
     if (good) l = rd(p) | (rd(p + 1) << 8);
     good = good && l >= 3 && p + l <= end;
-    if (k >= c0 && k < c0 + C) out[k - c0] = good ? p | (l << 16) : 0u;
-    if (good) p += l;
+    if (good) {
+      put(k, p, l);
+      p += l;
+    }
   }
-  good = good && p == end;
-  if (!good)
-    for (int k = 0; k < C; k++) out[k] = 0u;
-  return good;
+  return good && p == end;
 }
 
 // Unpacks and clusters n <= 32 slots (lane s < n holds slot s's FE unit in `me`, its event
@@ -486,12 +500,16 @@ __device__ void process_slots(W& w, int n, int c0, const SlotSrc& me, uint32_t e
     if (mine) {
       const int s = lane - done;
       bool good = false;
-      if (staged) {
-        if (me.data) good = walk_lengths<C>(at, me.len, c0, w.task + s * C, [&](uint32_t i) { return (uint32_t)w.buf[i]; });
-      } else if (me.data) {
-        good = walk_lengths<C>(0u, me.len, c0, w.task + s * C, [&](uint32_t i) { return (uint32_t)src0[i]; });
+      auto put = [&](int k, uint32_t pos, uint32_t l) {
+        if (k >= c0 && k < c0 + C) w.task[s * C + k - c0] = pos | (l << 16);
+      };
+      if (me.data) {
+        if (staged)
+          good = walk_lengths(at, me.len, [&](uint32_t i) { return (uint32_t)w.buf[i]; }, put);
+        else
+          good = walk_lengths(0u, me.len, [&](uint32_t i) { return (uint32_t)src0[i]; }, put);
       }
-      if (!me.data)
+      if (!good)
         for (int k = 0; k < C; k++) w.task[s * C + k] = 0u;
       st = good ? 0u : me.data ? (uint32_t)SST_CH_FRAMING : me.status;
       w.base[s] = off < out_cap ? off : 0;
