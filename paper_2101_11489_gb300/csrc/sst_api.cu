@@ -96,6 +96,26 @@ cudaError_t ensure_spill(Scratch& s, size_t warps) {
   return cudaSuccess;
 }
 
+bool amp_scratch_fits(const Scratch& s, size_t amp_bytes) {
+  return amp_bytes <= s.amp_stage_cap && s.amp_items_cap >= s.items_cap && s.amp_ev_cap >= s.ev_cap &&
+         s.stage_amp_cap >= s.stage_cap && s.amp_spill_warps >= s.spill_warps;
+}
+
+cudaError_t ensure_amp_scratch(Scratch& s, size_t amp_bytes) {
+  if (amp_scratch_fits(s, amp_bytes)) return cudaSuccess;
+  cudaError_t e = cudaDeviceSynchronize();  // growing: wait for all work that may still use the old buffers
+  if (e) return e;
+  size_t c1 = 2 * s.amp_items_cap, c2 = 2 * s.amp_items_cap, c3 = s.amp_spill_warps * kAmpSpill;
+  if ((e = grow(s.seg_amp_cnt, c1, 2 * s.items_cap))) return e;
+  if ((e = grow(s.seg_amp_start, c2, 2 * s.items_cap))) return e;
+  s.amp_items_cap = s.items_cap;
+  if ((e = grow(s.amp_spill, c3, s.spill_warps * kAmpSpill))) return e;
+  s.amp_spill_warps = s.spill_warps;
+  if ((e = grow(s.amp_alloc, s.amp_ev_cap, s.ev_cap))) return e;
+  if ((e = grow(s.stage_amp, s.stage_amp_cap, s.stage_cap))) return e;
+  return grow(s.amp_stage, s.amp_stage_cap, amp_bytes);
+}
+
 void free_scratch(Scratch& s) {
   if (s.look.words) cudaFree(s.look.words);
   if (s.fed_off) cudaFree(s.fed_off);
@@ -106,6 +126,9 @@ void free_scratch(Scratch& s) {
   if (s.stage) cudaFree(s.stage);
   if (s.tickets) cudaFree(s.tickets);
   if (s.spill) cudaFree(s.spill);
+  for (void* p : {(void*)s.amp_stage, (void*)s.stage_amp, (void*)s.amp_alloc, (void*)s.seg_amp_cnt,
+                  (void*)s.seg_amp_start, (void*)s.amp_spill})
+    if (p) cudaFree(p);
   s = Scratch{};
 }
 
@@ -135,6 +158,8 @@ sst_status sst_create(sst_ctx** out, int device, uint32_t n_feds) {
   DeviceGuard g(device);
   cudaError_t e = cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, device);
   if (e == cudaSuccess) e = ensure_scratch(c->scratch, (size_t)n_feds * kFe, 1, 1);
+  // (its one size: launches captured into a graph keep its address)
+  if (e == cudaSuccess) e = ensure_spill(c->scratch, (size_t)c->n_sm * kMaxWarpsPerSm);
   if (e != cudaSuccess) {
     free_scratch(c->scratch);
     delete c;
@@ -276,7 +301,7 @@ sst_status sst_batch(sst_ctx* ctx, const uint8_t* raw, const uint64_t* event_off
   DeviceGuard g(ctx->device);
   const size_t items = (size_t)n_events * n_feds;
   cudaError_t e = ensure_scratch(ctx->scratch, items * kFe, n_events, out->capacity);
-  if (!e) e = ensure_spill(ctx->scratch, (size_t)ctx->n_sm * kMaxWarpsPerSm);
+  if (!e && out->amp) e = ensure_amp_scratch(ctx->scratch, out->amp_capacity);
   if (e) return cuda_err(ctx, e, "sst_batch scratch");
   cudaEvent_t eb = nullptr, ee = nullptr;
   if (ctx->profiling) {

@@ -18,6 +18,7 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kFedBuf = 8192;      // bytes of FED record staged on chip (larger ones are read in place)
 constexpr int kRunSlots = (kFedBuf + 2) / 3;  // a run header takes at least 3 bytes with its ADC
+constexpr uint32_t kFedClusters = kCh * kStrips / 2;  // most clusters of a FED
 constexpr uint32_t kLbBlock = 1024;  // FEDs whose counts a CTA sums one by one
 constexpr unsigned long long kSet = 1ull << 63;
 
@@ -603,14 +604,22 @@ struct Out {
   uint64_t a_off = 0, a_room = 0;  // and of the amplitudes
 };
 
+// Threads to a channel that leave none idle in a chunk of n channels.
+__device__ __forceinline__ int lanes_for(int n) {
+  int l = 32;
+  while (l > 2 && l * n > kThreads) l /= 2;
+  return l;
+}
+
 // Clusters one FED whose `total` digis load(c0, c1) brings into the tile, classified,
-// chunk by chunk, and writes its clusters in order; a FED of more than one chunk goes
-// through them twice, first to count.  place(found, amps) publishes the counts and
+// chunk by chunk, and writes its clusters in order.  A FED of more than one chunk leaves
+// its clusters in `spill` (kFedClusters of them) until it knows their place; with
+// amplitudes, or without a spill area, it goes through the chunks again.  place(found, amps) publishes the counts and
 // returns those of the FEDs before.  Returns the clusters found; *amps_found their
 // strips.
 template <bool AMP, int TILE, class S, typename Load, typename Place>
 __device__ __forceinline__ uint32_t cluster_fed(S& s, const KParams& kp, uint32_t fed, uint32_t total, Load load,
-                                                Place place, const Out& o, const sst_clusters& out,
+                                                Place place, const Out& o, const sst_clusters& out, uint2* spill,
                                                 uint32_t* amps_found) {
   const bool single = total <= (uint32_t)TILE;
   uint32_t in_tile = 0;  // kept clusters of the chunk in the tile
@@ -625,6 +634,17 @@ __device__ __forceinline__ uint32_t cluster_fed(S& s, const KParams& kp, uint32_
   for (int c0 = 0; c0 < kCh;) {
     const int c1 = single ? kCh : chunk_end<TILE>(s, c0);
     chunk(c0, c1);
+    if (!AMP && !single && spill)
+      for (uint32_t r = threadIdx.x; r < in_tile; r += kThreads) {
+        int lo, hi;
+        uint32_t c;
+        const uint32_t i = s.list[r];
+        cluster_strips(s, kp, fed, i, &lo, &hi, &c);
+        const uint2 v = s.cal()[i];
+        spill[found + r] =
+            cs::staged_cluster((uint32_t)lo, (uint32_t)(hi - lo + 1), v.x >> 16, v.y - (uint32_t)lo * (v.x >> 16), c);
+      }
+    if (!single) __syncthreads();  // the tile is filled again
     found += in_tile;
     if (AMP) {
       uint32_t w = 0;
@@ -641,6 +661,20 @@ __device__ __forceinline__ uint32_t cluster_fed(S& s, const KParams& kp, uint32_
   const Counts before = place(found, amps);
   const unsigned long long n0 = before.clusters, a0 = before.amps;
   const bool amp_fits = !AMP || a0 + amps <= o.a_room;
+  *amps_found = amps;
+  if (!AMP && !single && spill) {
+    for (uint32_t r = threadIdx.x; r < found && n0 + r < o.room; r += kThreads) {
+      const uint2 v = spill[r];
+      const uint32_t lo = v.x & 255u, wd = ((v.x >> 8) & 255u) + 1u, q = v.x >> 16;
+      const uint64_t at = o.off + n0 + r;
+      out.det[at] = fed * (uint32_t)kCh + (v.y >> 24);
+      out.first[at] = (uint16_t)lo;
+      out.width[at] = (uint16_t)wd;
+      out.charge[at] = q;
+      out.barycenter[at] = centroid(lo, wd, q, v.y & 0xFFFFFFu);
+    }
+    return found;
+  }
   uint32_t run = 0, arun = 0;  // clusters and strips of the chunks before
   for (int c0 = 0; c0 < kCh && found > 0;) {
     const int c1 = single ? kCh : chunk_end<TILE>(s, c0);
@@ -687,7 +721,6 @@ __device__ __forceinline__ uint32_t cluster_fed(S& s, const KParams& kp, uint32_
     run += in_tile;
     c0 = c1;
   }
-  *amps_found = amps;
   return found;
 }
 

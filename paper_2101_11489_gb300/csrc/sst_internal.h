@@ -78,11 +78,24 @@ struct Scratch {
   uint32_t* tickets = nullptr;       // [16]: [0] k_stream's tiles, [1] k_clu_scan's CTAs done
   uint4* spill = nullptr;            // per warp of k_stream, kSpillRecords candidate records
   size_t spill_warps = 0;            // warps that have them
+  // clusters with amplitudes (k_stream)
+  uint8_t* amp_stage = nullptr;      // staged amplitudes, sliced per event like the output
+  size_t amp_stage_cap = 0;
+  uint32_t* stage_amp = nullptr;     // per staged cluster: its first amplitude within its segment
+  size_t stage_amp_cap = 0;
+  uint32_t* amp_alloc = nullptr;     // amplitude allocation counter per event
+  size_t amp_ev_cap = 0;
+  uint32_t* seg_amp_cnt = nullptr;   // amplitudes per segment; 0 when they did not fit
+  uint32_t* seg_amp_start = nullptr; // their offset in the event's slice, or kNoAmp
+  size_t amp_items_cap = 0;
+  uint32_t* amp_spill = nullptr;     // per warp that has a spill area, kAmpSpill words
+  size_t amp_spill_warps = 0;
   uint32_t lb_spin_limit = 0;        // polls before a look-back wait gives up (0: the default, about a second)
   int32_t lb_withhold = -1;          // failure tests: the FED that never publishes its count (-1: none)
 };
 constexpr uint32_t kNoAmp = 0xFFFFFFFFu;
 constexpr uint32_t kSpillRecords = 1608;  // records per warp spill area (25 KiB)
+constexpr uint32_t kAmpSpill = kSpillRecords + 128;  // words per warp beside them for clusters with amplitudes
 constexpr int kMaxWarpsPerSm = 32;        // resident warps of the batched kernel per SM (its register use)
 
 // Grid, block, shared memory per CTA and work items per FED of the batched kernel's
@@ -152,6 +165,10 @@ KParams kparams(const sst_ctx* c);
 cudaError_t ensure_scratch(Scratch& s, size_t items, size_t events, size_t stage_records);
 // Candidate lists for `warps` warps of k_stream; grows only.
 cudaError_t ensure_spill(Scratch& s, size_t warps);
+// What k_stream needs for amplitudes beside the above (after ensure_scratch and
+// ensure_spill); grows only.
+cudaError_t ensure_amp_scratch(Scratch& s, size_t amp_bytes);
+bool amp_scratch_fits(const Scratch& s, size_t amp_bytes);
 void free_scratch(Scratch& s);
 void free_host_pipe(sst_ctx* ctx);
 

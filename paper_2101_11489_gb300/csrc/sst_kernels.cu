@@ -157,14 +157,14 @@ __device__ void describe_fed(const uint8_t* __restrict__ raw, uint64_t fo, uint3
 // lengths of the FEDs before them itself.  Every FED's header is checked and its FE
 // units described (describe_fed).  It is also the launch sequence's prologue: the
 // event's last CTA writes its status (zero but SST_EV_SIZE), its first clears the
-// staging counter, the very first clears the work tickets.  Event e's bytes are
+// staging counters (amp_alloc: when given), the very first clears the work tickets.  Event e's bytes are
 // [event_off[e], event_end[e]) when event_end is given (events that do not follow
 // one another, e.g. read in place from host memory), else [event_off[e],
 // event_off[e + 1]).
 __global__ void k_fed_scan(const uint64_t* __restrict__ event_off, const uint64_t* __restrict__ event_end,
                            const uint32_t* __restrict__ fed_len, uint32_t n_feds, uint32_t cpe,
                            uint64_t* __restrict__ fed_off, sst_event_status* status, uint32_t* ev_alloc,
-                           uint32_t* tickets, const uint8_t* __restrict__ raw, uint2* unit_desc) {
+                           uint32_t* tickets, const uint8_t* __restrict__ raw, uint2* unit_desc, uint32_t* amp_alloc) {
   __shared__ uint32_t wsum[32];
   __shared__ unsigned long long psum[32];
   pdl_release();
@@ -172,7 +172,10 @@ __global__ void k_fed_scan(const uint64_t* __restrict__ event_off, const uint64_
   const uint32_t f0 = c * blockDim.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint64_t ev0 = event_off[e], ev1 = event_end ? event_end[e] : event_off[e + 1];
-  if (c == 0 && threadIdx.x == 0) ev_alloc[e] = 0;
+  if (c == 0 && threadIdx.x == 0) {
+    ev_alloc[e] = 0;
+    if (amp_alloc) amp_alloc[e] = 0;
+  }
   if (e == 0 && c == 0 && threadIdx.x < 2) tickets[threadIdx.x] = 0;
   const uint32_t* len_e = fed_len + (size_t)e * n_feds;
   // bytes of the event's FEDs before this CTA's
@@ -211,26 +214,35 @@ __device__ __forceinline__ cs::SlotSrc slot_src(const uint8_t* __restrict__ raw,
   return r;
 }
 
+// The bytes that a warp takes next (lane s: slot s) on their way to L2, up to 512 a unit.
+__device__ __forceinline__ void prefetch_slots(const cs::SlotSrc& src) {
+  const int lane = threadIdx.x & 31, s = lane >> 2;
+  const uint8_t* g =
+      reinterpret_cast<const uint8_t*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(src.src), s)) +
+      128 * (lane & 3);
+  const uint32_t len = __shfl_sync(0xffffffffu, src.len, s);
+  if (128u * (lane & 3) < len) asm volatile("prefetch.global.L2 [%0];" ::"l"(g));
+}
+
 // a7: the FE units of a batch of many events.  A CTA of W warps holds the
 // calibration entries of C = 3 W / 2 channels (24 KB for W = 8: one FE unit) in
-// shared memory and runs every event's records of those channels against them, 4 U
-// events per warp at a time.
+// shared memory and runs the events' records of those channels against them (`chunk`
+// events per tile and CTA), up to 4 U at a time per warp.
 //
 // Bound by instruction issue (about 70% of the slots) and shared-memory latency.  On
-// 64 full-detector events (79.5 MB of records, 29.4 M digis) it takes 185 us where
-// k_batch, which finds each digi's run and candidate by warp ballots, takes 351: 5,460
-// against 11,700 warp instructions per 96 channels, and the calibration is read from
-// DRAM once (86 MB) instead of gathered from L2 digi by digi (840 MB of sectors).
-// What the tile costs is its load, so it needs events to share it (kStreamEvents).
-template <int W, int U>
+// 64 full-detector events (79.5 MB of records, 29.4 M digis) it takes 185 us, 5,460
+// warp instructions per 96 channels, and the calibration is read from DRAM once
+// (86 MB).  (The kernel before it expanded every digi into a tile and found its run and
+// candidate by warp ballots: 351 us, 11,700 instructions, 840 MB of gathers from L2.)
+template <bool AMP, int W, int U>
 __global__ void __launch_bounds__(W * 32, 32 / W) k_stream(const uint8_t* __restrict__ raw,
                                                            const uint64_t* __restrict__ fed_off, uint32_t n_events,
                                                            uint32_t n_feds, const uint64_t* __restrict__ clu_off,
                                                            uint64_t out_cap, sst_event_status* status, KParams kp,
                                                            uint2* stage, uint32_t* ev_alloc, uint32_t* seg_cnt,
                                                            uint32_t* seg_start, uint32_t* ticket,
-                                                           const uint2* __restrict__ unit_desc, uint32_t per_warp,
-                                                           uint32_t resident) {
+                                                           const uint2* __restrict__ unit_desc, uint32_t chunk,
+                                                           uint32_t per_warp, uint32_t resident, cs::Amps am) {
   constexpr int C = 3 * W / 2, kParts = kChPerFe / C;  // channels of the tile, tiles per FE unit
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint2* tile = reinterpret_cast<uint2*>(smem_raw);
@@ -240,9 +252,11 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_stream(const uint8_t* __rest
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   cs::WarpT<U>& w = warps[warp];
   uint4* spill = kp.spill + (size_t)(blockIdx.x * W + warp) * kSpillRecords;
-  const uint32_t n_tiles = n_feds * kFe * kParts;
-  // Tiles: the CTAs that fit the GPU at once (`resident`) start on the tile of their
-  // own index, while the prologue still runs; all further tiles come from the ticket.
+  uint32_t* amp_spill = AMP ? am.spill + (size_t)(blockIdx.x * W + warp) * kAmpSpill : nullptr;
+  const uint32_t chunks = (n_events + chunk - 1) / chunk, n_items = n_feds * kFe * kParts * chunks;
+  // Items (a tile and a chunk of events): the CTAs that fit the GPU at once (`resident`)
+  // start on the item of their own index, while the prologue still runs; all further
+  // ones come from the ticket.
   bool first = true, fresh = true;
   cs::SlotSrc src{raw, 0u, 0u, false};
   uint32_t t = blockIdx.x;
@@ -254,9 +268,10 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_stream(const uint8_t* __rest
     t = s_next;
     __syncthreads();
   }
-  while (t < n_tiles) {
-    const uint32_t fu = t / kParts;                                       // FE unit of the detector
-    const uint32_t ch0 = fu * kChPerFe + (t % kParts) * C;                // first channel of the tile
+  while (t < n_items) {
+    const uint32_t tl = t / chunks, fu = tl / kParts, part = tl % kParts;  // tile, FE unit of the detector, half of it
+    const uint32_t e_first = t % chunks * chunk, e_end = e_first + chunk < n_events ? e_first + chunk : n_events;
+    const uint32_t ch0 = fu * kChPerFe + part * C;                         // first channel of the tile
     const uint8_t* g = reinterpret_cast<const uint8_t*>(kp.calq + (size_t)ch0 * kStrips);
     for (uint32_t i = threadIdx.x; i < C * kStrips * sizeof(uint2) / 16; i += W * 32)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
@@ -271,41 +286,96 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_stream(const uint8_t* __rest
     asm volatile("cp.async.wait_all;" ::: "memory");
     const bool any_div = __syncthreads_or(m2.x < 0 || m2.y < 0);
     const uint32_t next = s_next;
-    for (uint32_t e0 = warp * per_warp; e0 < n_events; e0 += W * per_warp) {
-      const uint32_t n = n_events - e0 < per_warp ? n_events - e0 : per_warp;
-      const uint32_t e = e0 + (lane < (int)n ? lane : 0);
-      if (fresh && lane < (int)n) src = slot_src(raw, fed_off, unit_desc, (size_t)e * n_feds + fu / kFe, fu % kFe);
-      if (lane >= (int)n) src = cs::SlotSrc{raw, 0u, 0u, false};
-      // what this warp takes next: the same events' records of the next tile, or the next
-      // events' of this one
-      const bool same = e0 + W * per_warp < n_events;
-      const uint32_t fu2 = same ? fu : next / kParts, e2 = (same ? e0 + W * per_warp : warp * per_warp) + lane;
-      cs::SlotSrc src2{raw, 0u, 0u, false};
-      if (lane < (int)per_warp && e2 < n_events && fu2 < n_feds * kFe)
-        src2 = slot_src(raw, fed_off, unit_desc, (size_t)e2 * n_feds + fu2 / kFe, fu2 % kFe);
-      cs::process_slots<C>(
-          w, (int)n, (int)(t % kParts) * C, src, e, (((size_t)e * n_feds + fu / kFe) * kFe + fu % kFe) * kParts + t % kParts,
-          kp, clu_off, out_cap, status, stage, ev_alloc, seg_cnt, seg_start, spill, tile, mul,
-          any_div, ch0, [&] {
-            // its bytes on their way to L2 (up to 512 a unit)
-            const int s = lane >> 2;
-            const uint8_t* g = reinterpret_cast<const uint8_t*>(
-                                   __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(src2.src), s)) +
-                               128 * (lane & 3);
-            const uint32_t len = __shfl_sync(0xffffffffu, src2.len, s);
-            if (128u * (lane & 3) < len) asm volatile("prefetch.global.L2 [%0];" ::"l"(g));
-          });
-      src = src2;
-      fresh = false;
-    }
-    // the next tile's calibration entries
-    if (next < n_tiles) {
-      const uint8_t* g2 = reinterpret_cast<const uint8_t*>(
-          kp.calq + ((size_t)(next / kParts) * kChPerFe + (next % kParts) * C) * kStrips);
+    if (next < n_items) {  // the next tile's entries on their way to L2
+      const uint8_t* g2 = reinterpret_cast<const uint8_t*>(kp.calq + (size_t)(next / chunks) * C * kStrips);
       for (uint32_t i = threadIdx.x; i < C * kStrips * sizeof(uint2) / 128; i += W * 32)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(g2 + 128 * i));
     }
+    const cs::Channels<C, false> chans{tile, mul, ch0};
+    for (uint32_t e0 = e_first + warp * per_warp; e0 < e_end; e0 += W * per_warp) {
+      const uint32_t n = e_end - e0 < per_warp ? e_end - e0 : per_warp;
+      const uint32_t e = e0 + (lane < (int)n ? lane : 0);
+      if (fresh && lane < (int)n) src = slot_src(raw, fed_off, unit_desc, (size_t)e * n_feds + fu / kFe, fu % kFe);
+      if (lane >= (int)n) src = cs::SlotSrc{raw, 0u, 0u, false};
+      // what this warp takes next: the next events of this item, or its share of the next
+      const bool same = e0 + W * per_warp < e_end;
+      const uint32_t fu2 = same ? fu : next / chunks / kParts;
+      const uint32_t e2 = (same ? e0 + W * per_warp : next % chunks * chunk + warp * per_warp) + lane;
+      cs::SlotSrc src2{raw, 0u, 0u, false};
+      if (lane < (int)per_warp && e2 < n_events && fu2 < n_feds * kFe)
+        src2 = slot_src(raw, fed_off, unit_desc, (size_t)e2 * n_feds + fu2 / kFe, fu2 % kFe);
+      cs::process_slots<AMP, C>(
+          w, (int)n, (int)part * C, src, e, (((size_t)e * n_feds + fu / kFe) * kFe + fu % kFe) * kParts + part, kp,
+          clu_off, out_cap, status, stage, ev_alloc, seg_cnt, seg_start, spill, chans, any_div, am, amp_spill,
+          [&] { prefetch_slots(src2); });
+      src = src2;
+      fresh = false;
+    }
+    if (e_first + warp * per_warp >= e_end) fresh = true;  // nothing was read ahead
     __syncthreads();
+    t = next;
+  }
+  pdl_release();
+}
+
+// a7 for batches of fewer events: a warp takes `units` adjacent FE units of one FED of
+// one event (units x 12 channels) and reads their calibration entries from global
+// memory, digi by digi.  The tile of k_stream would cost more than these gathers (24 KB
+// against about 4 KB per FE unit and event), and its warps would each have only a few
+// channels.  FED-major order, so that the warps at work read the same FEDs' entries.
+constexpr int kFedWarps = 8;
+struct FedWarp {
+  cs::WarpT<2> w;
+  int2 mul[kCh];  // the units' APV multipliers
+};
+template <bool AMP>
+__global__ void __launch_bounds__(kFedWarps * 32, 3) k_stream_fed(
+    const uint8_t* __restrict__ raw, const uint64_t* __restrict__ fed_off, uint32_t n_events, uint32_t n_feds,
+    const uint64_t* __restrict__ clu_off, uint64_t out_cap, sst_event_status* status, KParams kp, uint2* stage,
+    uint32_t* ev_alloc, uint32_t* seg_cnt, uint32_t* seg_start, uint32_t* ticket, const uint2* __restrict__ unit_desc,
+    uint32_t units, cs::Amps am) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  FedWarp& w = reinterpret_cast<FedWarp*>(smem_raw)[warp];
+  const uint32_t id = blockIdx.x * kFedWarps + warp, n_warps = gridDim.x * kFedWarps;
+  uint4* spill = kp.spill + (size_t)id * kSpillRecords;
+  uint32_t* amp_spill = AMP ? am.spill + (size_t)id * kAmpSpill : nullptr;
+  const uint32_t parts = kFe / units, per_fed = n_events * parts, n_items = n_feds * per_fed;
+  pdl_wait();
+  auto unit_of = [&](uint32_t t, uint32_t* e, uint32_t* f, uint32_t* u) {
+    const uint32_t r = t % per_fed;
+    *f = t / per_fed;
+    *e = r / parts;
+    *u = r % parts * units;
+  };
+  auto src_of = [&](uint32_t t) {
+    uint32_t e, f, u;
+    unit_of(t, &e, &f, &u);
+    cs::SlotSrc src{raw, 0u, 0u, false};
+    if (t < n_items && lane < (int)units) src = slot_src(raw, fed_off, unit_desc, (size_t)e * n_feds + f, u + lane);
+    return src;
+  };
+  uint32_t t = id;
+  cs::SlotSrc src = src_of(t);
+  while (t < n_items) {
+    uint32_t next = 0, e, f, u;
+    if (lane == 0) next = n_warps + atomicAdd(ticket, 1u);
+    unit_of(t, &e, &f, &u);
+    const uint32_t ch0 = f * kCh + u * kChPerFe;
+    bool div = false;
+    for (uint32_t i = lane; i < units * kChPerFe; i += 32) {
+      w.mul[i] = __ldg(reinterpret_cast<const int2*>(kp.mul) + ch0 + i);
+      div |= w.mul[i].x < 0 || w.mul[i].y < 0;
+    }
+    div = __any_sync(0xffffffffu, div);
+    next = __shfl_sync(0xffffffffu, next, 0);
+    const cs::SlotSrc src2 = src_of(next);
+    const cs::Channels<kChPerFe, true> chans{kp.calq + (size_t)ch0 * kStrips, w.mul, ch0};
+    cs::process_slots<AMP, kChPerFe>(w.w, (int)units, 0, src, e,
+                                     ((size_t)e * n_feds + f) * kFe + u + (lane < (int)units ? lane : 0), kp, clu_off,
+                                     out_cap, status, stage, ev_alloc, seg_cnt, seg_start, spill, chans, div, am,
+                                     amp_spill, [&] { prefetch_slots(src2); });
+    src = src2;
     t = next;
   }
   pdl_release();
@@ -370,12 +440,15 @@ __global__ void __launch_bounds__(1024) k_clu_scan(const uint32_t* __restrict__ 
 // clusters start at clu_off[e] (its slice; 0 without clu_off), or at pack_off[e]
 // when pack_off is given (k_clu_scan computed it and the events' counts); the
 // event's last CTA otherwise stores its cluster count.
-template <int SEGS>
+// AMP: the segments' amplitudes are ordered the same way, and each cluster's amp_first
+// is its segment's place plus its own within the segment.
+template <int SEGS, bool AMP>
 __global__ void __launch_bounds__(256) k_order(const uint2* __restrict__ stage, const uint64_t* __restrict__ clu_off,
                                                const uint64_t* __restrict__ pack_off,
                                                const uint32_t* __restrict__ seg_cnt,
                                                const uint32_t* __restrict__ seg_start, uint32_t n_segs, uint32_t cpe,
-                                               sst_clusters out, sst_event_status* status, uint32_t chans) {
+                                               sst_clusters out, sst_event_status* status, uint32_t chans,
+                                               cs::Amps am) {
   static_assert(SEGS <= 256, "one scan entry per thread, a byte per segment");
   constexpr bool kNoted = SEGS > 16;             // few segments: searched for instead (4 steps, no barriers)
   constexpr uint32_t kMap = kNoted ? 4096 : 1;   // output records whose segments are noted at once
@@ -412,6 +485,40 @@ __global__ void __launch_bounds__(256) k_order(const uint2* __restrict__ stage, 
   uint16_t* const width = out.width + dst;
   uint32_t* const charge = out.charge + dst;
   float* const bary = out.barycenter + dst;
+  // the amplitudes, a warp per segment
+  __shared__ uint32_t s_amp[AMP ? SEGS : 1];  // place of the segment's first amplitude, or kNoAmp
+  __shared__ uint32_t s_acnt[AMP ? SEGS : 1], s_afrom[AMP ? SEGS : 1];
+  if (AMP) {
+    const uint32_t* acnt_e = am.seg_cnt + (size_t)e * n_segs;
+    uint32_t before = 0, atot, slice, slice_end;
+    for (uint32_t i = tid; i < seg0; i += blockDim.x) before += __ldg(acnt_e + i);
+    const uint32_t mine = tid < (int)nseg ? __ldg(acnt_e + seg0 + tid) : 0u;
+    __syncthreads();
+    block_excl_scan(before, wsum, &before);  // the sum
+    const uint32_t place = block_excl_scan(mine, wsum, &atot);
+    cs::amp_slice(am.off, am.cap, e, &slice, &slice_end);
+    if (tid < (int)nseg) {
+      const uint32_t from = __ldg(am.seg_start + (size_t)e * n_segs + seg0 + tid);
+      s_acnt[tid] = mine;
+      s_afrom[tid] = from == kNoAmp ? 0u : from;
+      s_amp[tid] = from == kNoAmp ? kNoAmp : slice + before + place;
+    }
+    __syncthreads();
+    // 16 threads to a segment, four bytes of it in flight each
+    for (uint32_t g = tid / 16; g < nseg; g += 16) {
+      const uint32_t n = s_acnt[g];
+      const uint8_t* from = am.bytes + slice + s_afrom[g];
+      uint8_t* to = out.amp + s_amp[g];
+      for (uint32_t k = tid % 16; k < n; k += 64) {
+        uint8_t b[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) b[u] = k + 16 * u < n ? __ldg(from + k + 16 * u) : (uint8_t)0;
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+          if (k + 16 * u < n) to[k + 16 * u] = b[u];
+      }
+    }
+  }
   constexpr int kU = 4;  // records per thread in flight
   if (!kNoted) __syncthreads();
   for (uint32_t m0 = 0; m0 < tot; m0 += kNoted ? kMap : tot) {
@@ -423,6 +530,7 @@ __global__ void __launch_bounds__(256) k_order(const uint2* __restrict__ stage, 
     for (uint32_t d0 = m0 + tid; d0 < m1; d0 += kU * blockDim.x) {
       uint2 r[kU];
       uint32_t m[kU];  // the segment's first module
+      uint32_t af[kU];
 #pragma unroll
       for (int u = 0; u < kU; u++) {
         const uint32_t d = d0 + u * blockDim.x;
@@ -438,6 +546,7 @@ __global__ void __launch_bounds__(256) k_order(const uint2* __restrict__ stage, 
           const uint32_t at = s_start[sg] + (d - s_dest[sg]);
           r[u] = __ldg(src + at);
           m[u] = (seg0 + sg) * chans;
+          if (AMP) af[u] = s_amp[sg] == kNoAmp ? kNoAmp : s_amp[sg] + __ldg(am.first + off + at);
         }
       }
 #pragma unroll
@@ -450,6 +559,7 @@ __global__ void __launch_bounds__(256) k_order(const uint2* __restrict__ stage, 
           width[d] = (uint16_t)wd;
           charge[d] = q;
           bary[d] = centroid(lo, wd, q, r[u].y & 0xFFFFFFu);
+          if (AMP) out.amp_first[dst + d] = af[u];
         }
       }
     }
@@ -520,6 +630,12 @@ __global__ void __launch_bounds__(ev::kThreads) k_unpack(const uint8_t* __restri
     out.status->n_bad_channels = __ldcg(sh.acc + 1);
     ev::write_flags(sh, 0, (size_ok ? 0u : SST_EV_SIZE) | (all > cap ? SST_EV_DIGI_CAPACITY : 0u), out.status);
   }
+}
+
+// The CTA's spill area for a FED of several chunks, or null.
+__device__ __forceinline__ uint2* fed_spill(const KParams& kp) {
+  const size_t have = (size_t)kp.spill_warps * kSpillRecords * 2 / ev::kFedClusters;  // in 8-byte records
+  return blockIdx.x < have ? reinterpret_cast<uint2*>(kp.spill) + (size_t)blockIdx.x * ev::kFedClusters : nullptr;
 }
 
 // a3 - a6 per event: one CTA per FED over the digi SoA.
@@ -603,7 +719,7 @@ __global__ void __launch_bounds__(ev::kThreads) k_cluster(sst_digis in, KParams 
         if (tid == 0) ev::publish(sh, f, 0, own, 0, 0);
         return before = ev::look_back<AMP>(s, sh, f, 0, own, (f & (ev::kLbBlock - 1u)) == ev::kLbBlock - 1u, &timed_out);
       },
-      o, out, &amps);
+      o, out, fed_spill(kp), &amps);
   if (tid != 0) return;
   if (timed_out) ev::flag_timeout(sh, 0, in.status);
   if (f == sh.n_feds - 1) {
@@ -678,7 +794,7 @@ __global__ void __launch_bounds__(ev::kThreads) k_event(const uint8_t* __restric
         // (the calibration entries take the staged record's place: a FED of several
         // chunks is read from global memory again)
         if (staged && total <= (uint32_t)kEvTile) ev::emit_slots(s, len);
-        else ev::emit_channels(s, g, c0, c1, 2);
+        else ev::emit_channels(s, g, c0, c1, ev::lanes_for(c1 - c0));
         ev::classify_tile(s, cal0, s.chan_cnt[c1] - s.chan_cnt[c0]);
       },
       [&](uint32_t n, uint32_t a) {
@@ -699,7 +815,7 @@ __global__ void __launch_bounds__(ev::kThreads) k_event(const uint8_t* __restric
         }
         return before;
       },
-      o, out, &amps);
+      o, out, fed_spill(kp), &amps);
   if (tid != 0) return;
   if (timed_out) ev::flag_timeout(sh, e, status + e);
   auto place = [&](uint64_t n) { return n < o.room ? n : o.room; };  // clusters stored of n
@@ -898,6 +1014,21 @@ cudaError_t launch_pdl(void (*k)(KArgs...), unsigned grid, unsigned block, size_
   return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
 }
 
+// k_stream's amplitude arguments: none unless the caller asked for them.
+cs::Amps amp_args(const sst_clusters& out, const Scratch& s) {
+  cs::Amps a;
+  if (!out.amp) return a;
+  a.spill = s.amp_spill;
+  a.bytes = s.amp_stage;
+  a.first = s.stage_amp;
+  a.off = out.amp_off;
+  a.cap = out.amp_capacity;
+  a.alloc = s.amp_alloc;
+  a.seg_cnt = s.seg_amp_cnt;
+  a.seg_start = s.seg_amp_start;
+  return a;
+}
+
 // The shared state of a launch of one CTA per FED of n_events events: one of the two
 // sets of l in turn, cleared by the launch before (which had the other).  A launch
 // that a graph may replay has the same set every time, and the replays are not seen
@@ -962,73 +1093,146 @@ cudaError_t launch_event(const uint8_t* raw, const uint64_t* event_off, const ui
   auto* k = out.amp ? k_event<true> : k_event<false>;
   return launch_feds((const void*)k, sm, s.look, n_events, n_feds, s.lb_spin_limit, st, [&](ev::Shared& sh) {
     return launch_pdl(k, n_events * n_feds, (unsigned)ev::kThreads, sm, st, raw, event_off, event_end, fed_len,
-                      n_events, clu_off, out, status, kp, pack_off, sh);
+                      n_events, clu_off, out, status, with_spill(kp, s), pack_off, sh);
   });
 }
 
+// Which kernel a batch takes, by its events and its FED records (events x FEDs).
+// Measured on full-detector events (440 FEDs) unless noted, us a batch:
+//   k_event (a CTA per record, one launch) has the shortest critical path but the least
+//   throughput: 1 event 28 (k_stream_fed 31), 2 events 50 (41); 120 FEDs x 4 events 25
+//   (27); with amplitudes, whose second launch is the longer one, 2 events 57 (54), 200
+//   FEDs x 6 events 58 (63);
+//   k_stream pays for its tiles: while they all fit the GPU at once (up to 76 FEDs) it is
+//   the fastest of the three from 4 events on (61 FEDs x 4: 20, 23 and 23; x 37: 37, 51
+//   and 64); beyond, from 12 events on (8 events 104, k_stream_fed 91; 16: 118 and 130).
+constexpr uint32_t kEventRecords = 240, kEventRecordsWide = 700, kEventRecordsAmps = 1600;
+constexpr uint32_t kTileEvents = 12, kTileRecords = 3600;
+constexpr uint32_t kTileChunk = 32;
+
+// How a batch is launched.
+struct Plan {
+  enum Kind { kFeds, kUnits, kTiles } kind = kFeds;  // k_event, k_stream_fed, k_stream
+  int grid = 0, block = 0, resident = 0;
+  size_t smem = 0;
+  uint32_t segs_per_fed = kFe;     // segments of the staging buffer per FED and event
+  uint32_t units = 0;              // kUnits: FE units per warp
+  uint32_t chunk = 0, per_warp = 0;  // kTiles: events per item, and per warp of it
+};
+
 template <int W, int U>
-cudaError_t stream_grid(const Shape& sh, uint32_t n_feds, int n_sm, int* grid, int* resident, size_t* smem) {
-  *smem = sizeof(uint2) * (3 * W / 2) * kStrips + W * sizeof(cs::WarpT<U>);
+cudaError_t plan_tiles(const Shape& sh, uint32_t n_events, uint32_t n_feds, int n_sm, Plan* p) {
+  p->block = W * 32;
+  p->smem = sizeof(uint2) * (3 * W / 2) * kStrips + W * sizeof(cs::WarpT<U>);
+  p->segs_per_fed = kFe * (8 / W);
   int per_sm = 0;
-  cudaError_t e = prepare((const void*)k_stream<W, U>, W * 32, *smem, &per_sm);
+  cudaError_t e = prepare((const void*)k_stream<false, W, U>, p->block, p->smem, &per_sm);
   if (e) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const size_t tiles = (size_t)n_feds * kFe * (8 / W);
-  const size_t ctas = (size_t)n_sm * (sh.ctas_per_sm < kMaxWarpsPerSm / W ? sh.ctas_per_sm : kMaxWarpsPerSm / W), fit = (size_t)n_sm * per_sm;
-  *grid = (int)(ctas < tiles ? ctas : tiles);
-  *resident = (int)(fit < (size_t)*grid ? fit : (size_t)*grid);
+  const size_t per = sh.ctas_per_sm < kMaxWarpsPerSm / W ? sh.ctas_per_sm : kMaxWarpsPerSm / W;
+  const size_t ctas = (size_t)n_sm * per, fit = (size_t)n_sm * per_sm, tiles = (size_t)n_feds * p->segs_per_fed;
+  // few tiles: their events are shared out, down to kTileChunk at a time
+  uint32_t chunks = 1;
+  while (tiles * chunks < 2 * fit && (n_events + 2 * chunks - 1) / (2 * chunks) >= kTileChunk) chunks *= 2;
+  p->chunk = (n_events + chunks - 1) / chunks;
+  const uint32_t passes = (p->chunk + W * 32 - 1) / (W * 32);  // at most 32 events, a lane each, per warp and pass
+  p->per_warp = (p->chunk + W * passes - 1) / (W * passes);
+  const size_t items = tiles * ((n_events + p->chunk - 1) / p->chunk);
+  p->grid = (int)(ctas < items ? ctas : items);
+  p->resident = (int)(fit < (size_t)p->grid ? fit : (size_t)p->grid);
   return cudaSuccess;
 }
 
-// Batches of at least this many events without amplitudes take k_stream: a tile is
-// 24 KB and an event's gathers of the same channels about 4 KB.
-constexpr uint32_t kStreamEvents = 8;
-bool use_stream(uint32_t n_events, bool amps) { return !amps && n_events >= kStreamEvents; }
-
-template <int W, int U>
-cudaError_t launch_stream_t(const uint8_t* raw, uint32_t n_events, uint32_t n_feds, const uint64_t* clu_off,
-                            uint64_t out_cap, sst_event_status* status, const KParams& kp, const Scratch& s,
-                            const Shape& sh, int n_sm, cudaStream_t st) {
-  int grid = 0, resident = 0;
-  size_t sm = 0;
-  cudaError_t e = stream_grid<W, U>(sh, n_feds, n_sm, &grid, &resident, &sm);
+cudaError_t plan_batch(const Shape& sh, uint32_t n_events, uint32_t n_feds, bool amps, int n_sm, Plan* p) {
+  const size_t records = (size_t)n_events * n_feds;
+  const bool one_wave = (size_t)n_feds * kFe <= (size_t)n_sm * 4;  // the tiles fit the GPU at once
+  const bool tiles = n_events >= kTileEvents || one_wave || records > kTileRecords;
+  if (records < (one_wave ? kEventRecords : amps ? kEventRecordsAmps : kEventRecordsWide) &&
+      (one_wave || !tiles)) {
+    p->kind = Plan::kFeds;
+    p->grid = (int)records;
+    p->block = ev::kThreads;
+    p->smem = sizeof(ev::Shm<kEvTile, true>);
+    return cudaSuccess;
+  }
+  if (tiles) {
+    p->kind = Plan::kTiles;
+    auto* f = sh.block == 128 ? (sh.units == 1 ? plan_tiles<4, 1> : plan_tiles<4, 2>)
+                              : (sh.units == 1 ? plan_tiles<8, 1> : plan_tiles<8, 2>);
+    return f(sh, n_events, n_feds, n_sm, p);
+  }
+  p->kind = Plan::kUnits;
+  p->block = kFedWarps * 32;
+  p->smem = kFedWarps * sizeof(FedWarp);
+  int per_sm = 0;
+  cudaError_t e = prepare((const void*)k_stream_fed<false>, p->block, p->smem, &per_sm);
   if (e) return e;
-  const KParams kps = with_spill(kp, s);
-  if ((size_t)grid * W > s.spill_warps) return cudaErrorInvalidConfiguration;
-  // events per warp and pass over the tile (at most 32, one lane each): all warps of the CTA busy
-  const uint32_t passes = (n_events + W * 32 - 1) / (W * 32);
-  const uint32_t per_warp = (n_events + W * passes - 1) / (W * passes);
-  return launch_pdl(k_stream<W, U>, (unsigned)grid, (unsigned)(W * 32), sm, st, raw, (const uint64_t*)s.fed_off,
-                    n_events, n_feds, clu_off, out_cap, status, kps, s.stage, s.ev_alloc, s.fed_cnt, s.fed_start,
-                    s.tickets, (const uint2*)s.unit_desc, per_warp, (uint32_t)resident);
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const size_t per = sh.ctas_per_sm < per_sm ? sh.ctas_per_sm : per_sm, ctas = (size_t)n_sm * per;
+  // FE units per warp: few enough that every warp has an item, but no fewer than half a
+  // FED's (a quarter's channels leave lanes idle) once that makes a wave, and a whole FED's
+  // when halves make more than two (6 events: 77 with halves, 86 with whole FEDs)
+  p->units = 1;
+  while (p->units < kFe / 2 && records * (kFe / p->units) > ctas * kFedWarps) p->units *= 2;
+  if (records * 2 > 2 * ctas * kFedWarps) p->units = kFe;
+  const size_t need = (records * (kFe / p->units) + kFedWarps - 1) / kFedWarps;
+  p->grid = (int)(ctas < need ? ctas : need);
+  p->resident = p->grid;
+  return cudaSuccess;
 }
 
-cudaError_t launch_stream(const uint8_t* raw, uint32_t n_events, uint32_t n_feds, const uint64_t* clu_off,
-                          uint64_t out_cap, sst_event_status* status, const KParams& kp, const Scratch& s,
-                          const Shape& sh, int n_sm, cudaStream_t st) {
-  auto* f = sh.block == 128 ? (sh.units == 1 ? launch_stream_t<4, 1> : launch_stream_t<4, 2>)
-                            : (sh.units == 1 ? launch_stream_t<8, 1> : launch_stream_t<8, 2>);
-  return f(raw, n_events, n_feds, clu_off, out_cap, status, kp, s, sh, n_sm, st);
+template <bool AMP, int W, int U>
+cudaError_t launch_tiles(const Plan& p, const uint8_t* raw, uint32_t n_events, uint32_t n_feds,
+                         const uint64_t* clu_off, uint64_t out_cap, sst_event_status* status, const KParams& kp,
+                         const Scratch& s, const cs::Amps& am, cudaStream_t st) {
+  int per_sm = 0;
+  cudaError_t e = prepare((const void*)k_stream<AMP, W, U>, p.block, p.smem, &per_sm);
+  if (e) return e;
+  return launch_pdl(k_stream<AMP, W, U>, (unsigned)p.grid, (unsigned)p.block, p.smem, st, raw,
+                    (const uint64_t*)s.fed_off, n_events, n_feds, clu_off, out_cap, status, kp, s.stage, s.ev_alloc,
+                    s.fed_cnt, s.fed_start, s.tickets, (const uint2*)s.unit_desc, p.chunk, p.per_warp,
+                    (uint32_t)p.resident, am);
+}
+
+template <bool AMP>
+cudaError_t launch_stream(const Plan& p, const Shape& sh, const uint8_t* raw, uint32_t n_events, uint32_t n_feds,
+                          const uint64_t* clu_off, uint64_t out_cap, sst_event_status* status, const KParams& kp,
+                          const Scratch& s, const cs::Amps& am, cudaStream_t st) {
+  if ((size_t)p.grid * (p.block / 32) > s.spill_warps) return cudaErrorInvalidConfiguration;
+  const KParams kps = with_spill(kp, s);
+  if (p.kind == Plan::kTiles) {
+    auto* f = sh.block == 128 ? (sh.units == 1 ? launch_tiles<AMP, 4, 1> : launch_tiles<AMP, 4, 2>)
+                              : (sh.units == 1 ? launch_tiles<AMP, 8, 1> : launch_tiles<AMP, 8, 2>);
+    return f(p, raw, n_events, n_feds, clu_off, out_cap, status, kps, s, am, st);
+  }
+  int per_sm = 0;
+  cudaError_t e = prepare((const void*)k_stream_fed<AMP>, p.block, p.smem, &per_sm);
+  if (e) return e;
+  return launch_pdl(k_stream_fed<AMP>, (unsigned)p.grid, (unsigned)p.block, p.smem, st, raw,
+                    (const uint64_t*)s.fed_off, n_events, n_feds, clu_off, out_cap, status, kps, s.stage, s.ev_alloc,
+                    s.fed_cnt, s.fed_start, s.tickets, (const uint2*)s.unit_desc, p.units, am);
 }
 
 // k_stream's per-event cluster order and the copy into the caller's SoA.  chans:
 // channels per segment.
 cudaError_t launch_order(const uint64_t* clu_off, uint32_t n_events, uint32_t n_segs, const sst_clusters& out,
                          sst_event_status* status, const Scratch& s, uint64_t* pack_off, uint32_t chans,
-                         cudaStream_t st) {
+                         const cs::Amps& am, cudaStream_t st) {
   cudaError_t e;
   if (pack_off) {
     k_clu_scan<<<n_events, 1024, 0, st>>>(s.fed_cnt, n_segs, status, pack_off, s.tickets + 1);
     if ((e = cudaGetLastError())) return e;
   }
-  // 128 segments per CTA; 16 when that would give a small grid (few events or FEDs), so
-  // that enough CTAs share the copy
-  const uint32_t cpe128 = (n_segs + 127) / 128;
-  const bool wide = (uint64_t)n_events * cpe128 >= 256;
-  const uint32_t cpe = wide ? cpe128 : (n_segs + 15) / 16;
-  return launch_pdl(wide ? k_order<128> : k_order<16>, (unsigned)((uint64_t)n_events * cpe), 256u, 0, st,
+  // 128 segments per CTA; 32 or 16 when that would give a small grid, so that enough
+  // CTAs share the copy
+  const uint64_t all = (uint64_t)n_events * n_segs;
+  const uint32_t per = all >= 128 * 1000 ? 128u : all >= 32 * 500 ? 32u : 16u;
+  const uint32_t cpe = (n_segs + per - 1) / per;
+  auto* k = am.bytes ? (per == 128 ? k_order<128, true> : per == 32 ? k_order<32, true> : k_order<16, true>)
+                     : (per == 128 ? k_order<128, false> : per == 32 ? k_order<32, false> : k_order<16, false>);
+  return launch_pdl(k, (unsigned)((uint64_t)n_events * cpe), 256u, 0, st,
                     (const uint2*)s.stage, clu_off, (const uint64_t*)pack_off, (const uint32_t*)s.fed_cnt,
-                    (const uint32_t*)s.fed_start, n_segs, cpe, out, status, chans);
+                    (const uint32_t*)s.fed_start, n_segs, cpe, out, status, chans, am);
 }
 
 }  // namespace
@@ -1047,18 +1251,14 @@ bool shape_valid(const Shape& s) {
 
 cudaError_t batch_launch_info(const Shape& sh, uint32_t n_events, uint32_t n_feds, int n_sm, int* grid, size_t* smem,
                               int* block, int* items_per_fed) {
-  if (use_stream(n_events, false)) {
-    int resident = 0;
-    *block = sh.block;
-    *items_per_fed = kFe / sh.units;
-    auto* f = sh.block == 128 ? (sh.units == 1 ? stream_grid<4, 1> : stream_grid<4, 2>)
-                              : (sh.units == 1 ? stream_grid<8, 1> : stream_grid<8, 2>);
-    return f(sh, n_feds, n_sm, grid, &resident, smem);
-  }
-  *grid = (int)(n_events * n_feds);
-  *block = ev::kThreads;
-  *smem = sizeof(ev::Shm<kEvTile, true>);
-  *items_per_fed = 1;
+  Plan p;
+  const bool amps = false;
+  const cudaError_t e = plan_batch(sh, n_events, n_feds, amps, n_sm, &p);
+  if (e) return e;
+  *grid = p.grid;
+  *block = p.block;
+  *smem = p.smem;
+  *items_per_fed = p.kind == Plan::kTiles ? kFe / sh.units : p.kind == Plan::kUnits ? (int)(kFe / p.units) : 1;
   return cudaSuccess;
 }
 
@@ -1077,7 +1277,7 @@ cudaError_t launch_cluster(const sst_digis& in, uint32_t n_feds, const sst_clust
   const size_t sm = sizeof(ev::Shm<kEvTile, true>);
   auto* k = out.amp ? k_cluster<true> : k_cluster<false>;
   return launch_feds((const void*)k, sm, s.look, 1, n_feds, s.lb_spin_limit, st, [&](ev::Shared& sh) {
-    return launch_pdl(k, n_feds, (unsigned)ev::kThreads, sm, st, in, kp, out, sh);
+    return launch_pdl(k, n_feds, (unsigned)ev::kThreads, sm, st, in, with_spill(kp, s), out, sh);
   });
 }
 
@@ -1085,23 +1285,29 @@ cudaError_t launch_batch(const uint8_t* raw, const uint64_t* event_off, const ui
                          uint32_t n_feds, const uint64_t* clu_off, const sst_clusters& out, sst_event_status* status,
                          const KParams& kp, Scratch& s, const Shape& sh, int n_sm, cudaStream_t st,
                          uint64_t* pack_off, cudaEvent_t ev_begin, cudaEvent_t ev_end, const uint64_t* event_end) {
-  cudaError_t e;
-  const bool stream = use_stream(n_events, out.amp != nullptr);
-  if (stream) {
-    const uint32_t cpe = (n_feds + kFedScanThreads - 1) / kFedScanThreads;
-    k_fed_scan<<<(unsigned)((uint64_t)n_events * cpe), kFedScanThreads, 0, st>>>(
-        event_off, event_end, fed_len, n_feds, cpe, s.fed_off, status, s.ev_alloc, s.tickets, raw, s.unit_desc);
-    if ((e = cudaGetLastError())) return e;
+  Plan p;
+  const bool amps = out.amp != nullptr;
+  cudaError_t e = plan_batch(sh, n_events, n_feds, amps, n_sm, &p);
+  if (e) return e;
+  if (p.kind == Plan::kFeds) {
+    if (ev_begin && (e = cudaEventRecord(ev_begin, st))) return e;
+    e = launch_event(raw, event_off, event_end, fed_len, n_events, n_feds, clu_off, out, status, kp, s, st, pack_off);
+    if (e) return e;
+    return ev_end ? cudaEventRecord(ev_end, st) : cudaSuccess;
   }
+  const uint32_t cpe = (n_feds + kFedScanThreads - 1) / kFedScanThreads;
+  k_fed_scan<<<(unsigned)((uint64_t)n_events * cpe), kFedScanThreads, 0, st>>>(
+      event_off, event_end, fed_len, n_feds, cpe, s.fed_off, status, s.ev_alloc, s.tickets, raw, s.unit_desc,
+      out.amp ? s.amp_alloc : nullptr);
+  if ((e = cudaGetLastError())) return e;
   if (ev_begin && (e = cudaEventRecord(ev_begin, st))) return e;
-  e = stream ? launch_stream(raw, n_events, n_feds, clu_off, out.capacity, status, kp, s, sh, n_sm, st)
-             : launch_event(raw, event_off, event_end, fed_len, n_events, n_feds, clu_off, out, status, kp, s, st,
-                            pack_off);
+  const cs::Amps am = amp_args(out, s);
+  e = (out.amp ? launch_stream<true> : launch_stream<false>)(p, sh, raw, n_events, n_feds, clu_off, out.capacity,
+                                                             status, kp, s, am, st);
   if (e) return e;
   if (ev_end && (e = cudaEventRecord(ev_end, st))) return e;
-  if (!stream) return cudaSuccess;
-  const uint32_t per_fed = kFe * (256 / sh.block);
-  return launch_order(clu_off, n_events, n_feds * per_fed, out, status, s, pack_off, (uint32_t)kCh / per_fed, st);
+  return launch_order(clu_off, n_events, n_feds * p.segs_per_fed, out, status, s, pack_off,
+                      (uint32_t)kCh / p.segs_per_fed, am, st);
 }
 
 cudaError_t rebase_amp_first(uint32_t* amp_first, const uint64_t* count, uint32_t base, int n_sm, cudaStream_t st) {

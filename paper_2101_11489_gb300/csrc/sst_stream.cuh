@@ -59,14 +59,21 @@ static_assert(layout_ok<1>() && layout_ok<2>(), "per-warp shared memory layout")
 // CTA of an SM: 226 against 185 us (64 full-detector events).
 // Record: {first strip | last + 1 << 8 | task << 17; raw ADC | charge << 16;
 // noise^2, then place among the task's kept clusters; moment}.
+// Clusters with amplitudes: `from` says where a record's first digi is (Walk::from); 128
+// words after its kSpillRecords are free for per-task values.
 struct List {
   uint4* rec;
+  uint32_t* from;
   uint32_t n;
   // Appends r of every lane with `emit` (all lanes call).
-  __device__ __forceinline__ void append(bool emit, uint4 r) {
+  template <bool AMP>
+  __device__ __forceinline__ void append(bool emit, uint4 r, uint32_t at) {
     const unsigned b = __ballot_sync(0xffffffffu, emit);
     const uint32_t i = n + __popc(b & ((1u << (threadIdx.x & 31)) - 1u));
-    if (emit && i < kSpillRecords) rec[i] = r;
+    if (emit && i < kSpillRecords) {
+      rec[i] = r;
+      if (AMP) from[i] = at;
+    }
     n += __popc(b);
   }
 };
@@ -115,9 +122,10 @@ struct Walk {
   float n2;            // sum of noise^2, strip by strip
   uint32_t seeded;     // it has a seed
   uint32_t digis;      // digis read
+  uint32_t from;       // amplitudes: byte after the candidate's first digi (16 bits) | strip past its run << 16
   __device__ __forceinline__ void begin(uint32_t pos) {
     p = pos;
-    strip = strip_end = 0;
+    strip = strip_end = from = 0;
     first = sums = moment = seeded = digis = 0;
     last1 = 0u - 4096u;  // the first active strip starts a candidate, whatever its linking limit
     n2 = 0.f;
@@ -137,118 +145,239 @@ struct Walk {
 //
 // The step is straight-line predicated code, written as PTX because the compiler's
 // own version of the same step branches around its parts (88 instructions a step
-// against about 63, 12 of them only when some lane ends a seeded candidate).  How
-// many lanes still walk is looked at every second step.
+// against about 65, 12 of them only when some lane ends a seeded candidate).  A digi is
+// fetched (header, ADC, calibration entry) one step before it is used, so that the
+// loads' latency is covered by the step between; on return the digi fetched last is
+// given back.  How many lanes still walk is looked at every second step.
 //   end2  the record's end - 2 (0: the lane has no record);  cal: its channel's
-//   calibration entries (shared);  m0, m1: its APVs' multipliers;  task17: its
-//   task << 17;  list.n: on return with the records appended.
+//   calibration entries (DIRECT: in global memory, else shared);  m0, m1: its APVs'
+//   multipliers;  task17: its task << 17;  list.n: on return with the records appended.
 
-// Run header, when one comes next: `ok` when its bytes end within the record, its
-// strips within the channel, its width is not 0 and it starts after the run before it.
-#define CS_HEADER                               \
-  "setp.eq.u32 hdr, %1, %2;\n"                  \
-  "@hdr ld.shared.u8 b0, [%0];\n"               \
-  "@hdr ld.shared.u8 b1, [%0+1];\n"             \
-  "add.u32 e, %0, b1;\n"                        \
-  "add.u32 u, b0, b1;\n"                        \
-  "setp.le.and.u32 ok, e, %12, hdr;\n"          \
-  "setp.le.and.u32 ok, u, 256, ok;\n"           \
-  "setp.lt.and.u32 ok, b0, u, ok;\n"            \
-  "setp.ge.and.u32 ok, b0, %1, ok;\n"           \
-  "not.pred alive, hdr;\n"                      \
-  "or.pred alive, alive, ok;\n"
-// The rest of a step.  First the digi and its strip's calibration entry; whether it is
-// active, a seed, not linked to the active strip before it; the seeded candidates
-// that end here go to the list; the gain-corrected charge (adc x multiplier, half up,
-// capped at 254, saturation codes kept); the open candidate.
-#define CS_DIGI(NEXT)                                   \
-  "@ok mov.u32 %1, b0;\n"                               \
-  "@ok mov.u32 %2, u;\n"                                \
-  "@ok add.u32 %0, %0, 2;\n"                            \
-  "ld.shared.u8 a, [%0];\n"                             \
-  "mad.lo.u32 ad, %1, 8, %13;\n"                        \
-  "ld.shared.v2.u32 {c, nq}, [ad];\n"                   \
-  "@alive add.u32 %0, %0, 1;\n"                         \
-  "@alive add.u32 %9, %9, 1;\n"                         \
-  "and.b32 lo, c, 255;\n"                               \
-  "setp.gt.and.u32 act, a, lo, alive;\n"                \
-  "bfe.u32 hi, c, 8, 8;\n"                              \
-  "setp.gt.and.u32 seed, a, hi, act;\n"                 \
-  "shr.u32 gap, c, 16;\n"                               \
-  "sub.u32 d, %1, %4;\n"                                \
-  "setp.ge.and.u32 start, d, gap, act;\n"               \
-  "and.pred emit, start, seeded;\n"                     \
-  "vote.sync.ballot.b32 bal, emit, 0xffffffff;\n"       \
-  "setp.eq.u32 t, bal, 0;\n"                            \
-  "@t bra.uni " NEXT ";\n"                              \
-  "and.b32 i, bal, %16;\n"                              \
-  "popc.b32 i, i;\n"                                    \
-  "add.u32 i, i, %10;\n"                                \
-  "popc.b32 d, bal;\n"                                  \
-  "add.u32 %10, %10, d;\n"                              \
-  "mad.lo.u32 x, %4, 256, %3;\n"                        \
-  "mov.b32 d, %7;\n"                                    \
-  "mad.wide.u32 g, i, 16, %18;\n"                       \
-  "@emit st.global.v4.u32 [g], {x, %5, d, %6};\n"       \
-  NEXT ":\n"                                            \
-  "setp.lt.u32 t, %1, 128;\n"                           \
-  "selp.u32 m, %14, %15, t;\n"                          \
-  "mad.lo.u32 q, a, m, %19;\n"                          \
-  "shr.u32 q, q, %20;\n"                                \
-  "min.u32 q, q, 254;\n"                                \
-  "setp.ge.u32 t, a, 254;\n"                            \
-  "selp.u32 q, a, q, t;\n"                              \
-  "@start add.u32 %3, %1, %21;\n"                       \
-  "@start mov.u32 %5, 0;\n"                             \
-  "@start mov.u32 %6, 0;\n"                             \
-  "@start mov.f32 %7, 0f00000000;\n"                    \
-  "not.pred t, start;\n"                                \
-  "and.pred t, t, seeded;\n"                            \
-  "or.pred seeded, t, seed;\n"                          \
-  "mov.b32 nz, nq;\n"                                   \
-  "@act mad.lo.u32 %5, q, 65536, %5;\n"                 \
-  "@act add.u32 %5, %5, a;\n"                           \
-  "@act mad.lo.u32 %6, %1, q, %6;\n"                    \
-  "@act add.rn.f32 %7, %7, nz;\n"                       \
-  "@alive add.u32 %1, %1, 1;\n"                         \
-  "@act mov.u32 %4, %1;\n"
+// Fetches the next digi of a lane that was (WAS) and is (AL) still walking: strip S, ADC A, calibration
+// entry {C, N}.  A run header, when one comes next, is `ok` when its bytes end within the
+// record, its strips within the channel, its width is not 0 and it starts after the run
+// before it.
+  #define CS_FETCH(S, A, C, N, F, AL, WAS, END2, ENTRY, ON_FETCH) \
+  "setp.eq.and.u32 hdr, %1, %2, " WAS ";\n" \
+  "@hdr ld.shared.u8 b0, [%0];\n" \
+  "@hdr ld.shared.u8 b1, [%0+1];\n" \
+  "add.u32 e, %0, b1;\n" \
+  "add.u32 u, b0, b1;\n" \
+  "setp.le.and.u32 ok, e, %" END2 ", hdr;\n" \
+  "setp.le.and.u32 ok, u, 256, ok;\n" \
+  "setp.lt.and.u32 ok, b0, u, ok;\n" \
+  "setp.ge.and.u32 ok, b0, %1, ok;\n" \
+  "not.pred " AL ", hdr;\n" \
+  "and.pred " AL ", " AL ", " WAS ";\n" \
+  "or.pred " AL ", " AL ", ok;\n" \
+  "@ok mov.u32 %1, b0;\n" \
+  "@ok mov.u32 %2, u;\n" \
+  "@ok add.u32 %0, %0, 2;\n" \
+  "mov.u32 " S ", %1;\n" \
+  "@" AL " ld.shared.u8 " A ", [%0];\n" \
+  ENTRY(S, C, N, AL) \
+  "@" AL " add.u32 %0, %0, 1;\n" \
+  "@" AL " add.u32 %1, " S ", 1;\n" \
+  ON_FETCH(F)
+// Uses a fetched digi: whether it is active, a seed, not linked to the active strip before
+// it; the seeded candidates that end here go to the list; the gain-corrected charge (adc
+// x multiplier, half up, capped at 254, saturation codes kept); the open candidate.
+// Operands 0 - 11 are the walk's state, the arguments the numbers of the others;
+// ON_FETCH, ON_EMIT and ON_START add what clusters with amplitudes need.
+  #define CS_USE(S, A, C, N, F, AL, NEXT, M0, M1, LT, REC, HALF, SHIFT, T17, ON_EMIT, ON_START) \
+  "@" AL " add.u32 %9, %9, 1;\n" \
+  "and.b32 lo, " C ", 255;\n" \
+  "setp.gt.and.u32 act, " A ", lo, " AL ";\n" \
+  "bfe.u32 hi, " C ", 8, 8;\n" \
+  "setp.gt.and.u32 seed, " A ", hi, act;\n" \
+  "shr.u32 gap, " C ", 16;\n" \
+  "sub.u32 d, " S ", %4;\n" \
+  "setp.ge.and.u32 start, d, gap, act;\n" \
+  "and.pred emit, start, seeded;\n" \
+  "vote.sync.ballot.b32 bal, emit, 0xffffffff;\n" \
+  "setp.eq.u32 t, bal, 0;\n" \
+  "@t bra.uni " NEXT ";\n" \
+  "and.b32 i, bal, %" LT ";\n" \
+  "popc.b32 i, i;\n" \
+  "add.u32 i, i, %10;\n" \
+  "popc.b32 d, bal;\n" \
+  "add.u32 %10, %10, d;\n" \
+  "mad.lo.u32 x, %4, 256, %3;\n" \
+  "mov.b32 d, %7;\n" \
+  "mad.wide.u32 g, i, 16, %" REC ";\n" \
+  "@emit st.global.v4.u32 [g], {x, %5, d, %6};\n" \
+  ON_EMIT \
+  NEXT ":\n" \
+  "setp.lt.u32 t, " S ", 128;\n" \
+  "selp.u32 m, %" M0 ", %" M1 ", t;\n" \
+  "mad.lo.u32 q, " A ", m, %" HALF ";\n" \
+  "shr.u32 q, q, %" SHIFT ";\n" \
+  "min.u32 q, q, 254;\n" \
+  "setp.ge.u32 t, " A ", 254;\n" \
+  "selp.u32 q, " A ", q, t;\n" \
+  "@start add.u32 %3, " S ", %" T17 ";\n" \
+  ON_START(F) \
+  "@start mov.u32 %5, 0;\n" \
+  "@start mov.u32 %6, 0;\n" \
+  "@start mov.f32 %7, 0f00000000;\n" \
+  "not.pred t, start;\n" \
+  "and.pred t, t, seeded;\n" \
+  "or.pred seeded, t, seed;\n" \
+  "mov.b32 nz, " N ";\n" \
+  "@act mad.lo.u32 %5, q, 65536, %5;\n" \
+  "@act add.u32 %5, %5, " A ";\n" \
+  "@act mad.lo.u32 %6, " S ", q, %6;\n" \
+  "@act add.rn.f32 %7, %7, nz;\n" \
+  "@act add.u32 %4, " S ", 1;\n"
+  #define CS_WALK(E2, ENTRY, M0, M1, LT, FEW, REC, HALF, SHIFT, T17, ON_FETCH, ON_EMIT, ON_START) \
+  "{\n" \
+  ".reg .pred hdr, ok, alive0, alive1, act, seed, start, emit, seeded, t;\n" \
+  ".reg .u32 b0, b1, e, u, ad, lo, hi, gap, d, bal, i, x, m, q;\n" \
+  ".reg .u32 s0, a0, c0, n0, f0, s1, a1, c1, n1, f1;\n" \
+  ".reg .f32 nz;\n" \
+  ".reg .u64 g;\n" \
+  "setp.ne.u32 seeded, %8, 0;\n" \
+  "setp.ne.u32 alive1, %" E2 ", 0;\n" \
+  "mov.u32 a0, 0;\n" \
+  "mov.u32 c0, 0;\n" \
+  "mov.u32 n0, 0;\n" \
+  "mov.u32 a1, 0;\n" \
+  "mov.u32 c1, 0;\n" \
+  "mov.u32 n1, 0;\n" \
+  "mov.u32 b0, 0;\n" \
+  "mov.u32 b1, 0;\n" \
+  CS_FETCH("s0", "a0", "c0", "n0", "f0", "alive0", "alive1", E2, ENTRY, ON_FETCH) \
+  "STEP:\n" \
+  "vote.sync.ballot.b32 bal, alive0, 0xffffffff;\n" \
+  "popc.b32 i, bal;\n" \
+  "setp.le.u32 t, i, %" FEW ";\n" \
+  "@t bra.uni DONE;\n" \
+  CS_FETCH("s1", "a1", "c1", "n1", "f1", "alive1", "alive0", E2, ENTRY, ON_FETCH) \
+  CS_USE("s0", "a0", "c0", "n0", "f0", "alive0", "NEXT0", M0, M1, LT, REC, HALF, SHIFT, T17, ON_EMIT, ON_START) \
+  CS_FETCH("s0", "a0", "c0", "n0", "f0", "alive0", "alive1", E2, ENTRY, ON_FETCH) \
+  CS_USE("s1", "a1", "c1", "n1", "f1", "alive1", "NEXT1", M0, M1, LT, REC, HALF, SHIFT, T17, ON_EMIT, ON_START) \
+  "bra.uni STEP;\n" \
+  "DONE:\n" \
+  "@alive0 sub.u32 %0, %0, 1;\n" \
+  "@alive0 sub.u32 %1, %1, 1;\n" \
+  "selp.u32 %8, 1, 0, seeded;\n" \
+  "selp.u32 %11, 1, 0, alive0;\n" \
+  "}\n"
+// The same with entries two steps ahead, for those in global memory: a step of the warps
+// of a scheduler takes about 400 cycles, an entry from L2 more.  The two digis fetched
+// last are used, not given back.
+  #define CS_WALK_AHEAD(E2, ENTRY, M0, M1, LT, FEW, REC, HALF, SHIFT, T17, ON_FETCH, ON_EMIT, ON_START) \
+  "{\n" \
+  ".reg .pred hdr, ok, alive0, alive1, alive2, act, seed, start, emit, seeded, t;\n" \
+  ".reg .u32 b0, b1, e, u, ad, lo, hi, gap, d, bal, i, x, m, q;\n" \
+  ".reg .u32 s0, a0, c0, n0, f0, s1, a1, c1, n1, f1, s2, a2, c2, n2, f2;\n" \
+  ".reg .f32 nz;\n" \
+  ".reg .u64 g;\n" \
+  "setp.ne.u32 seeded, %8, 0;\n" \
+  "setp.ne.u32 alive2, %" E2 ", 0;\n" \
+  "mov.u32 a0, 0;\n" \
+  "mov.u32 c0, 0;\n" \
+  "mov.u32 n0, 0;\n" \
+  "mov.u32 a1, 0;\n" \
+  "mov.u32 c1, 0;\n" \
+  "mov.u32 n1, 0;\n" \
+  "mov.u32 a2, 0;\n" \
+  "mov.u32 c2, 0;\n" \
+  "mov.u32 n2, 0;\n" \
+  "mov.u32 b0, 0;\n" \
+  "mov.u32 b1, 0;\n" \
+  CS_FETCH("s0", "a0", "c0", "n0", "f0", "alive0", "alive2", E2, ENTRY, ON_FETCH) \
+  CS_FETCH("s1", "a1", "c1", "n1", "f1", "alive1", "alive0", E2, ENTRY, ON_FETCH) \
+  "STEP:\n" \
+  "vote.sync.ballot.b32 bal, alive0, 0xffffffff;\n" \
+  "popc.b32 i, bal;\n" \
+  "setp.le.u32 t, i, %" FEW ";\n" \
+  "@t bra.uni DONE;\n" \
+  CS_FETCH("s2", "a2", "c2", "n2", "f2", "alive2", "alive1", E2, ENTRY, ON_FETCH) \
+  CS_USE("s0", "a0", "c0", "n0", "f0", "alive0", "NEXT0", M0, M1, LT, REC, HALF, SHIFT, T17, ON_EMIT, ON_START) \
+  CS_FETCH("s0", "a0", "c0", "n0", "f0", "alive0", "alive2", E2, ENTRY, ON_FETCH) \
+  CS_USE("s1", "a1", "c1", "n1", "f1", "alive1", "NEXT1", M0, M1, LT, REC, HALF, SHIFT, T17, ON_EMIT, ON_START) \
+  CS_FETCH("s1", "a1", "c1", "n1", "f1", "alive1", "alive0", E2, ENTRY, ON_FETCH) \
+  CS_USE("s2", "a2", "c2", "n2", "f2", "alive2", "NEXT2", M0, M1, LT, REC, HALF, SHIFT, T17, ON_EMIT, ON_START) \
+  "bra.uni STEP;\n" \
+  "DONE:\n" \
+  CS_USE("s0", "a0", "c0", "n0", "f0", "alive0", "NEXT3", M0, M1, LT, REC, HALF, SHIFT, T17, ON_EMIT, ON_START) \
+  CS_USE("s1", "a1", "c1", "n1", "f1", "alive1", "NEXT4", M0, M1, LT, REC, HALF, SHIFT, T17, ON_EMIT, ON_START) \
+  "selp.u32 %8, 1, 0, seeded;\n" \
+  "selp.u32 %11, 1, 0, alive1;\n" \
+  "}\n"
+#define CS_NOTHING(F)
+#define CS_FROM_FETCH(F) "mad.lo.u32 " F ", %2, 65536, %0;\n"
+#define CS_FROM_START(F) "@start mov.u32 %12, " F ";\n"
+#define CS_ENTRY13S(S, C, N, AL) "mad.lo.u32 ad, " S ", 8, %13;\n" "@" AL " ld.shared.v2.u32 {" C ", " N "}, [ad];\n"
+#define CS_ENTRY13D(S, C, N, AL) "mad.wide.u32 g, " S ", 8, %13;\n" "@" AL " ld.global.nc.v2.u32 {" C ", " N "}, [g];\n"
+#define CS_ENTRY14S(S, C, N, AL) "mad.lo.u32 ad, " S ", 8, %14;\n" "@" AL " ld.shared.v2.u32 {" C ", " N "}, [ad];\n"
+#define CS_ENTRY14D(S, C, N, AL) "mad.wide.u32 g, " S ", 8, %14;\n" "@" AL " ld.global.nc.v2.u32 {" C ", " N "}, [g];\n"
 
-__device__ __forceinline__ bool walk_staged(Walk& k, uint32_t end2, uint32_t cal, int32_t m0, int32_t m1,
+template <bool AMP, bool DIRECT>
+__device__ __forceinline__ bool walk_staged(Walk& k, uint32_t end2, const uint2* cal, int32_t m0, int32_t m1,
                                             uint32_t task17, uint32_t few, List& list) {
   const uint32_t lt = (1u << (threadIdx.x & 31)) - 1u;
   uint32_t walking;
-  asm volatile(
-      "{\n"
-      ".reg .pred hdr, ok, alive, act, seed, start, emit, seeded, t;\n"
-      ".reg .u32 b0, b1, e, u, a, ad, c, nq, lo, hi, gap, d, bal, i, x, m, q;\n"
-      ".reg .f32 nz;\n"
-      ".reg .u64 g;\n"
-      "setp.ne.u32 seeded, %8, 0;\n"
-      "mov.u32 b0, 0;\n"
-      "mov.u32 b1, 0;\n"
-      "STEP:\n" CS_HEADER
-      "vote.sync.ballot.b32 bal, alive, 0xffffffff;\n"
-      "popc.b32 i, bal;\n"
-      "setp.le.u32 t, i, %17;\n"
-      "@t bra.uni DONE;\n" CS_DIGI("NEXT0") CS_HEADER CS_DIGI("NEXT1")
-      "bra.uni STEP;\n"
-      "DONE:\n"
-      "selp.u32 %8, 1, 0, seeded;\n"
-      "selp.u32 %11, 1, 0, alive;\n"
-      "}\n"
-      : "+r"(k.p), "+r"(k.strip), "+r"(k.strip_end), "+r"(k.first), "+r"(k.last1), "+r"(k.sums), "+r"(k.moment),
-        "+f"(k.n2), "+r"(k.seeded), "+r"(k.digis), "+r"(list.n), "=r"(walking)
-      : "r"(end2), "r"(cal), "r"(m0), "r"(m1), "r"(lt), "r"(few), "l"(list.rec), "n"(1 << (kMulShift - 1)),
-        "n"(kMulShift), "r"(task17)
-      : "memory");
+  if (AMP && DIRECT) {
+    asm volatile(CS_WALK_AHEAD("13", CS_ENTRY14D, "15", "16", "17", "18", "19", "20", "21", "22",
+                         CS_FROM_FETCH,
+                         "mad.wide.u32 g, i, 4, %23;\n"
+                         "@emit st.global.u32 [g], %12;\n",
+                         CS_FROM_START)
+                 : "+r"(k.p), "+r"(k.strip), "+r"(k.strip_end), "+r"(k.first), "+r"(k.last1), "+r"(k.sums),
+                   "+r"(k.moment), "+f"(k.n2), "+r"(k.seeded), "+r"(k.digis), "+r"(list.n), "=r"(walking),
+                   "+r"(k.from)
+                 : "r"(end2), "l"(cal), "r"(m0), "r"(m1), "r"(lt), "r"(few), "l"(list.rec),
+                   "n"(1 << (kMulShift - 1)), "n"(kMulShift), "r"(task17), "l"(list.from)
+                 : "memory");
+  } else if (AMP) {
+    asm volatile(CS_WALK("13", CS_ENTRY14S, "15", "16", "17", "18", "19", "20", "21", "22",
+                         CS_FROM_FETCH,
+                         "mad.wide.u32 g, i, 4, %23;\n"
+                         "@emit st.global.u32 [g], %12;\n",
+                         CS_FROM_START)
+                 : "+r"(k.p), "+r"(k.strip), "+r"(k.strip_end), "+r"(k.first), "+r"(k.last1), "+r"(k.sums),
+                   "+r"(k.moment), "+f"(k.n2), "+r"(k.seeded), "+r"(k.digis), "+r"(list.n), "=r"(walking),
+                   "+r"(k.from)
+                 : "r"(end2), "r"((uint32_t)__cvta_generic_to_shared(cal)), "r"(m0), "r"(m1), "r"(lt), "r"(few), "l"(list.rec),
+                   "n"(1 << (kMulShift - 1)), "n"(kMulShift), "r"(task17), "l"(list.from)
+                 : "memory");
+  } else if (DIRECT) {
+    asm volatile(CS_WALK_AHEAD("12", CS_ENTRY13D, "14", "15", "16", "17", "18", "19", "20", "21",
+                         CS_NOTHING, "", CS_NOTHING)
+                 : "+r"(k.p), "+r"(k.strip), "+r"(k.strip_end), "+r"(k.first), "+r"(k.last1), "+r"(k.sums),
+                   "+r"(k.moment), "+f"(k.n2), "+r"(k.seeded), "+r"(k.digis), "+r"(list.n), "=r"(walking)
+                 : "r"(end2), "l"(cal), "r"(m0), "r"(m1), "r"(lt), "r"(few), "l"(list.rec),
+                   "n"(1 << (kMulShift - 1)), "n"(kMulShift), "r"(task17)
+                 : "memory");
+  } else {
+    asm volatile(CS_WALK("12", CS_ENTRY13S, "14", "15", "16", "17", "18", "19", "20", "21",
+                         CS_NOTHING, "", CS_NOTHING)
+                 : "+r"(k.p), "+r"(k.strip), "+r"(k.strip_end), "+r"(k.first), "+r"(k.last1), "+r"(k.sums),
+                   "+r"(k.moment), "+f"(k.n2), "+r"(k.seeded), "+r"(k.digis), "+r"(list.n), "=r"(walking)
+                 : "r"(end2), "r"((uint32_t)__cvta_generic_to_shared(cal)), "r"(m0), "r"(m1), "r"(lt), "r"(few), "l"(list.rec),
+                   "n"(1 << (kMulShift - 1)), "n"(kMulShift), "r"(task17)
+                 : "memory");
+  }
   return walking != 0;
 }
-#undef CS_HEADER
-#undef CS_DIGI
+#undef CS_WALK
+#undef CS_WALK_AHEAD
+#undef CS_FETCH
+#undef CS_USE
+#undef CS_NOTHING
+#undef CS_FROM_FETCH
+#undef CS_FROM_START
+#undef CS_ENTRY13S
+#undef CS_ENTRY13D
+#undef CS_ENTRY14S
+#undef CS_ENTRY14D
 
 // The same walk for any record: read in place from anywhere (a unit larger than the
 // staging buffer), APVs without a multiplier dividing.  One channel per lane to the
 // record's end (`end` == p: none).
+template <bool AMP>
 __device__ void walk_any(Walk& k, const uint8_t* src, uint32_t end, const uint2* cal, int32_t m0, int32_t m1,
                          uint32_t task17, List& list) {
   for (;;) {
@@ -277,11 +406,12 @@ __device__ void walk_any(Walk& k, const uint8_t* src, uint32_t end, const uint2*
     }
     const bool act = a > (c.x & 255u), seed = a > ((c.x >> 8) & 255u);  // a lane that has stopped: 0, never active
     const bool start = act && s - k.last1 >= (c.x >> 16);
-    list.append(start && k.seeded, k.record());
+    list.append<AMP>(start && k.seeded, k.record(), k.from);
     if (act) {
       const uint32_t q = charge(a, s < (uint32_t)kApv ? m0 : m1);
       if (start) {
         k.first = s + task17;
+        k.from = (k.strip_end << 16) + k.p;
         k.sums = k.moment = k.seeded = 0;
         k.n2 = 0.f;
       }
@@ -305,16 +435,66 @@ __device__ __forceinline__ uint32_t stop_status(const Walk& k, uint32_t end, Rd 
                                               : (uint32_t)SST_CH_TRUNC;
 }
 
+// A record's strips [lo, hi], widened over up to max_adj adjacent bad strips of module
+// det at either end.
+__device__ __forceinline__ void record_strips(uint4 r, const KParams& kp, uint32_t det, int* lo, int* hi) {
+  *lo = (int)(r.x & 255u);
+  *hi = (int)((r.x >> 8) & 511u) - 1;
+  if (kp.max_adj > 0) {
+    const uint32_t* m = kp.badmask + (size_t)det * kMaskWords;
+    for (int k = 0; k < kp.max_adj && *lo > 0 && bit(m, *lo - 1); k++) --*lo;
+    for (int k = 0; k < kp.max_adj && *hi + 1 < kStrips && bit(m, *hi + 1); k++) ++*hi;
+  }
+}
+
+// Amplitude staging of a launch (rec null: no amplitudes).
+struct Amps {
+  uint32_t* spill = nullptr;      // per warp of the grid, kAmpSpill words (List::from)
+  uint8_t* bytes = nullptr;       // staged amplitudes, sliced per event like the output
+  uint32_t* first = nullptr;      // per staged cluster: its first amplitude within its segment
+  const uint64_t* off = nullptr;  // [n_events + 1] event slices
+  uint64_t cap = 0;               // bytes of staging and of output
+  uint32_t* alloc = nullptr;      // allocation counter per event
+  uint32_t* seg_cnt = nullptr;    // per segment: amplitudes stored (0 when they did not fit)
+  uint32_t* seg_start = nullptr;  // per segment: offset in the event's slice, or kNoAmp
+};
+// Event e's slice [a, b) of the amplitude arrays.
+__device__ __forceinline__ void amp_slice(const uint64_t* off, uint64_t cap, uint32_t e, uint32_t* a, uint32_t* b) {
+  uint64_t lo = off[e], hi = off[e + 1] < cap ? off[e + 1] : cap;  // cap is below 2^32
+  if (lo > hi) lo = hi;
+  *a = (uint32_t)lo;
+  *b = (uint32_t)hi;
+}
+
+// The channels of a warp's tasks.  Tile: every slot has the same C channels (of many
+// events), in shared memory.  DIRECT: the slots are FE units of one FED, one after the
+// other, in global memory.
+template <int C, bool DIRECT>
+struct Channels {
+  static constexpr bool kDirect = DIRECT;
+  const uint2* cal;  // calibration entries of the first channel
+  const int2* mul;   // APV multipliers, two per channel
+  uint32_t ch0;      // module id of the first channel
+  // channel of task t, slots counted from slot `done`
+  __device__ __forceinline__ uint32_t of(uint32_t t, int done) const {
+    return DIRECT ? (uint32_t)done * C + t : t % C;
+  }
+};
+
 // Cluster threshold of every record and the kept ones' places within their
 // channel: record i's z becomes the number of kept records of its channel before
 // it, or kNotKept; w.kept counts them.  A channel's records are in strip order.
-template <class W>
-__device__ __forceinline__ void rank_records(W& w, const List& list, float t_cluster) {
+// AMP: the strips of those before are added to z at bit 8, and w.task (free by now) sums
+// each channel's.
+template <bool AMP, class W, class Chans>
+__device__ __forceinline__ void rank_records(W& w, const List& list, const KParams& kp, const Chans& chans, int done) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   for (int i = lane; i < W::kTasks / 4; i += 32) reinterpret_cast<uint32_t*>(w.kept)[i] = 0;
+  if (AMP)
+    for (int i = lane; i < W::kTasks; i += 32) w.task[i] = 0;
   __syncwarp();
-  const Threshold thr(t_cluster);
+  const Threshold thr(kp.t_cluster);
   const uint4 none = make_uint4(0u, 0u, 0x7f800000u, 0u);
   uint4 ahead = (uint32_t)lane < list.n ? list.rec[lane] : none;
   for (uint32_t i = lane; i - lane < list.n; i += 32) {
@@ -323,10 +503,24 @@ __device__ __forceinline__ void rank_records(W& w, const List& list, float t_clu
     const bool pass = thr.pass(r.y & 0xFFFFu, __uint_as_float(r.z));
     const uint32_t t = r.x >> 17;
     const unsigned same = __match_any_sync(0xffffffffu, pass ? t : 128u);
-    const uint32_t rank = (pass ? (uint32_t)w.kept[t] : 0u) + __popc(same & lt);
-    __syncwarp();
+    uint32_t rank = (pass ? (uint32_t)w.kept[t] : 0u) + __popc(same & lt), z = rank;
+    if (AMP) {
+      int lo = 0, hi = -1;
+      if (pass) record_strips(r, kp, chans.ch0 + chans.of(t, done), &lo, &hi);
+      const uint32_t wd = (uint32_t)(hi - lo + 1);
+      uint32_t before = pass ? w.task[t] : 0u;
+      for (unsigned m = pass ? same & lt : 0u; __any_sync(0xffffffffu, m != 0); m &= m - 1u) {
+        const uint32_t v = __shfl_sync(0xffffffffu, wd, m ? __ffs(m) - 1 : 0);
+        if (m) before += v;
+      }
+      z |= before << 8;
+      __syncwarp();
+      if (pass && (same >> lane) == 1u) w.task[t] = before + wd;
+    } else {
+      __syncwarp();
+    }
     if (pass && (same >> lane) == 1u) w.kept[t] = (uint8_t)(rank + 1u);  // the channel's last record here
-    if (i < list.n) list.rec[i].z = pass ? rank : kNotKept;
+    if (i < list.n) list.rec[i].z = pass ? z : kNotKept;
     __syncwarp();
   }
 }
@@ -352,15 +546,67 @@ __device__ __forceinline__ void write_records(const W& w, const List& list, cons
     const uint32_t t = r.x >> 17, slot = t / C;
     const uint32_t pos = w.task[t] + r.z;
     if (pos >= w.slot.room[slot]) continue;
-    int lo = (int)(r.x & 255u), hi = (int)((r.x >> 8) & 511u) - 1;
-    if (kp.max_adj > 0) {
-      const uint32_t* m = kp.badmask + (size_t)det(t) * kMaskWords;
-      for (int k = 0; k < kp.max_adj && lo > 0 && bit(m, lo - 1); k++) lo--;
-      for (int k = 0; k < kp.max_adj && hi + 1 < kStrips && bit(m, hi + 1); k++) hi++;
-    }
+    int lo, hi;
+    record_strips(r, kp, det(t), &lo, &hi);
     const uint32_t q = r.y >> 16;
     stage[w.base[slot] + pos] =
         staged_cluster((uint32_t)lo, (uint32_t)(hi - lo + 1), q, r.w - (uint32_t)lo * q, t - slot * C);
+  }
+}
+
+// write_records for clusters with amplitudes.  `rel` (per task): the strips of the slot's
+// channels before it; w.slot.nbad: where the slot's amplitudes are staged, or kNoAmp.  A
+// cluster's amplitudes: 0 for every strip but its active digis, whose charges are formed
+// again from the record's bytes (rd; `shift` makes an index of a Walk::from byte) and
+// the calibration entries.
+template <int C, class W, class Chans, typename Rd>
+__device__ __forceinline__ void write_amplitudes(const W& w, const List& list, const KParams& kp, uint2* stage,
+                                                 const Amps& am, const uint32_t* rel, const Chans& chans, int done,
+                                                 uint32_t shift, Rd rd) {
+  const int lane = threadIdx.x & 31;
+  uint4 ahead = make_uint4(0u, 0u, kNotKept, 0u);
+  uint32_t from_ahead = 0;
+  if ((uint32_t)lane < list.n) {
+    ahead = list.rec[lane];
+    from_ahead = list.from[lane];
+  }
+  for (uint32_t i = lane; i < list.n; i += 32) {
+    const uint4 r = ahead;
+    const uint32_t from = from_ahead;
+    if (i + 32 < list.n) {
+      ahead = list.rec[i + 32];
+      from_ahead = list.from[i + 32];
+    }
+    if (r.z == kNotKept) continue;
+    const uint32_t t = r.x >> 17, slot = t / C, c = chans.of(t, done);
+    const uint32_t pos = w.task[t] + (r.z & 255u), first = rel[t] + (r.z >> 8);
+    int lo, hi;
+    record_strips(r, kp, chans.ch0 + c, &lo, &hi);
+    const uint32_t q = r.y >> 16;
+    if (pos < w.slot.room[slot]) {
+      stage[w.base[slot] + pos] =
+          staged_cluster((uint32_t)lo, (uint32_t)(hi - lo + 1), q, r.w - (uint32_t)lo * q, t - slot * C);
+      am.first[w.base[slot] + pos] = first;
+    }
+    if (w.slot.nbad[slot] == kNoAmp) continue;
+    uint8_t* d = am.bytes + (size_t)w.slot.nbad[slot] + first;
+    uint32_t p = ((from + shift) & 0xFFFFu) - 1u, run_end = from >> 16, next = r.x & 255u;  // next: strip of the digi at p
+    const uint32_t last1 = (r.x >> 8) & 511u;
+    const uint2* cal = chans.cal + c * kStrips;
+    const int2 mul = chans.mul[c];
+    for (uint32_t st = (uint32_t)lo; st <= (uint32_t)hi; st++) {
+      uint32_t v = 0;
+      if (st == next && st < last1) {
+        const uint32_t a = rd(p++);
+        if (a > (cal[st].x & 255u)) v = charge(a, st < (uint32_t)kApv ? mul.x : mul.y);
+        if (++next == run_end && next < last1) {
+          next = rd(p);
+          run_end = next + rd(p + 1);
+          p += 2;
+        }
+      }
+      *d++ = (uint8_t)v;
+    }
   }
 }
 
@@ -434,15 +680,14 @@ __device__ __forceinline__ bool walk_lengths(uint32_t p, uint32_t len, Rd rd, Pu
 
 // Unpacks and clusters n <= 32 slots (lane s < n holds slot s's FE unit in `me`, its event
 // in `e`, its segment index in `seg`): channels c0 .. c0 + C - 1 of each unit.
-// cal: the calibration entries of the C channels, in shared memory; mul: their
-// APVs' multipliers (two per channel), any_div: one of them is missing; ch0: the
-// module id of the first.
-// before_rank() runs between the walk and the rest.
-template <int C, class W, typename Hook>
+// any_div: an APV of theirs has no multiplier.  before_rank() runs between the walk and
+// the rest.
+template <bool AMP, int C, class W, class Chans, typename Hook>
 __device__ void process_slots(W& w, int n, int c0, const SlotSrc& me, uint32_t e, size_t seg, const KParams& kp,
                               const uint64_t* __restrict__ clu_off, uint64_t out_cap, sst_event_status* status,
                               uint2* stage, uint32_t* ev_alloc, uint32_t* seg_cnt, uint32_t* seg_start, uint4* spill,
-                              const uint2* cal, const int2* mul, bool any_div, uint32_t ch0, Hook before_rank) {
+                              const Chans& chans, bool any_div, const Amps& am,
+                              uint32_t* amp_spill, Hook before_rank) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   constexpr int kL = C / 3;  // lanes per slot when a lane sums three channels
@@ -525,7 +770,7 @@ __device__ void process_slots(W& w, int n, int c0, const SlotSrc& me, uint32_t e
       w.slot.nbad[lane - done] = st ? (uint32_t)C : 0u;
     }
     __syncwarp();
-    List list{spill, 0u};
+    List list{spill, amp_spill, 0u};
     // A channel found corrupt (its lane calls with err): its status, and its records,
     // among those from `from` on, are dropped.
     auto corrupt = [&](uint32_t t, uint32_t err) {
@@ -538,11 +783,39 @@ __device__ void process_slots(W& w, int n, int c0, const SlotSrc& me, uint32_t e
       }
       __syncwarp();
     };
-    if (staged && !any_div) {
-      const uint32_t buf0 = (uint32_t)__cvta_generic_to_shared(w.buf), cal0 = (uint32_t)__cvta_generic_to_shared(cal);
-      int next = 0;                       // channels taken
+    // The same at src, byte by byte, for any record and any APV.
+    auto walk_in_place = [&](int t0, int t1, const uint8_t* src) {
+      for (int r0 = t0; r0 < t1; r0 += 32) {
+        uint32_t t = 0, tk = 0;
+        if (r0 + lane < t1) {
+          t = w.order[r0 + lane];
+          tk = w.task[t];
+        }
+        const uint32_t pos = tk & 0xFFFFu, len = tk >> 16;
+        const bool has = len >= 3u, code = has && src[pos + 2] == SST_ZS_CODE;
+        const uint32_t c = chans.of(t, done);
+        const int2 mm = chans.mul[c];
+        Walk k;
+        k.begin(pos + 3u);
+        const uint32_t rec_end = code ? pos + len : 0u;
+        walk_any<AMP>(k, src, rec_end, chans.cal + c * kStrips, mm.x, mm.y, t << 17, list);
+        const uint32_t err = !has ? 0u
+                             : !code ? (uint32_t)SST_CH_BAD_CODE
+                             : k.p != rec_end ? stop_status(k, rec_end, [&](uint32_t i) { return (uint32_t)src[i]; })
+                                              : 0u;
+        list.append<AMP>(has && !err && k.seeded, k.record(), k.from);
+        if (has && !err) atomicAdd(&w.slot.digis[t / C], k.digis);
+        if (__any_sync(0xffffffffu, err != 0u)) corrupt(t, err);
+      }
+    };
+    const uint32_t buf0 = (uint32_t)__cvta_generic_to_shared(w.buf);
+    // Walks channels order[t0] .. order[t1 - 1], whose records are in the buffer `shift`
+    // bytes before their positions.
+    auto walk_fast = [&](int t0, int t1, uint32_t shift) {
+      int next = t0;                      // channels taken
       bool walking = false, has = false;  // the lane has a channel record: task t, bytes up to rec_end
-      uint32_t t = 0, rec_end = 0, cal_a = 0;
+      uint32_t t = 0, rec_end = 0;
+      const uint2* cal = chans.cal;
       int2 mm = make_int2(0, 0);
       Walk k;
       k.begin(buf0);
@@ -551,7 +824,7 @@ __device__ void process_slots(W& w, int n, int c0, const SlotSrc& me, uint32_t e
         const bool ended = has && !walking;
         const bool bad = ended && k.p != rec_end;
         if (ended && !bad) atomicAdd(&w.slot.digis[t / C], k.digis);
-        list.append(ended && !bad && k.seeded, k.record());
+        list.append<AMP>(ended && !bad && k.seeded, k.record(), k.from);
         if (__any_sync(0xffffffffu, bad))
           corrupt(t, !bad ? 0u
                      : rec_end == 0u
@@ -561,51 +834,68 @@ __device__ void process_slots(W& w, int n, int c0, const SlotSrc& me, uint32_t e
         const unsigned idle = __ballot_sync(0xffffffffu, !walking);
         if (!walking) {
           const int i = next + __popc(idle & lt);
-          has = i < n_task;
-          uint32_t tk = 0;
+          has = i < t1;
+          uint32_t tk = shift;
           if (has) {
             t = w.order[i];
             tk = w.task[t];
           }
-          const uint32_t pos = tk & 0xFFFFu, len = tk >> 16, c = t % C;
+          const uint32_t pos = (tk & 0xFFFFu) - shift, len = tk >> 16, c = chans.of(t, done);
           has = len >= 3u;
-          cal_a = cal0 + c * (uint32_t)(kStrips * sizeof(uint2));
-          mm = mul[c];
+          cal = chans.cal + c * kStrips;
+          mm = chans.mul[c];
           k.begin(buf0 + pos + 3u);
           rec_end = has && w.buf[pos + 2u] == SST_ZS_CODE ? buf0 + pos + len : 0u;  // 0: stops at once
         }
         next += __popc(idle);
         if (!__any_sync(0xffffffffu, has)) break;
-        walking = walk_staged(k, rec_end ? rec_end - 2u : 0u, cal_a, mm.x, mm.y, t << 17,
-                              next < n_task ? (uint32_t)kRefill : 0u, list);
+        walking = walk_staged<AMP, Chans::kDirect>(k, rec_end ? rec_end - 2u : 0u, cal, mm.x, mm.y, t << 17,
+                              next < t1 ? (uint32_t)kRefill : 0u, list);
+      }
+    };
+    if (staged && !any_div) {
+      walk_fast(0, n_task, 0);
+    } else if (!any_div) {
+      // one FE unit larger than the buffer: as many of its channels at a time as fit
+      if (lane < C) w.order[lane] = (uint8_t)lane;
+      __syncwarp();
+      for (int c = 0; c < C;) {
+        const uint32_t p0 = (w.task[c] & 0xFFFFu) & ~7u;
+        uint32_t end = p0;
+        int c1 = c;
+        while (c1 < C && (w.task[c1] & 0xFFFFu) + (w.task[c1] >> 16) - p0 <= (uint32_t)W::kBuf) {
+          end = max(end, (w.task[c1] & 0xFFFFu) + (w.task[c1] >> 16));
+          c1++;
+        }
+        if (c1 == c) {  // a record longer than the buffer (no valid one is)
+          walk_in_place(c, c + 1, src0);
+          c1 = c + 1;
+        } else {
+          const uint8_t* g = src0 + p0;
+          if ((reinterpret_cast<uintptr_t>(g) & 7u) == 0) {
+            for (uint32_t i = lane; i < (end - p0 + 7u) / 8u; i += 32)
+              asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(buf0 + 8 * i), "l"(g + 8 * i) : "memory");
+          } else {
+            for (uint32_t i = lane; i < end - p0; i += 32) w.buf[i] = __ldg(g + i);
+          }
+          asm volatile("cp.async.wait_all;" ::: "memory");
+          __syncwarp();
+          const uint32_t n0 = list.n;
+          walk_fast(c, c1, p0);
+          __syncwarp();
+          if (AMP)  // bytes of the unit, not of the buffer
+            for (uint32_t i = n0 + lane; i < list.n; i += 32)
+              list.from[i] = (list.from[i] & 0xFFFF0000u) | ((list.from[i] - buf0 + p0) & 0xFFFFu);
+          __syncwarp();
+        }
+        c = c1;
       }
     } else {
-      const uint8_t* src = staged ? w.buf : src0;
-      for (int r0 = 0; r0 < n_task; r0 += 32) {
-        uint32_t t = 0, tk = 0;
-        if (r0 + lane < n_task) {
-          t = w.order[r0 + lane];
-          tk = w.task[t];
-        }
-        const uint32_t pos = tk & 0xFFFFu, len = tk >> 16;
-        const bool has = len >= 3u, code = has && src[pos + 2] == SST_ZS_CODE;
-        const int2 mm = mul[t % C];
-        Walk k;
-        k.begin(pos + 3u);
-        const uint32_t rec_end = code ? pos + len : 0u;
-        walk_any(k, src, rec_end, cal + (t % C) * kStrips, mm.x, mm.y, t << 17, list);
-        const uint32_t err = !has ? 0u
-                             : !code ? (uint32_t)SST_CH_BAD_CODE
-                             : k.p != rec_end ? stop_status(k, rec_end, [&](uint32_t i) { return (uint32_t)src[i]; })
-                                              : 0u;
-        list.append(has && !err && k.seeded, k.record());
-        if (has && !err) atomicAdd(&w.slot.digis[t / C], k.digis);
-        if (__any_sync(0xffffffffu, err != 0u)) corrupt(t, err);
-      }
+      walk_in_place(0, n_task, staged ? w.buf : src0);
     }
     __syncwarp();
     if (done + m >= n) before_rank();
-    rank_records(w, list, kp.t_cluster);
+    rank_records<AMP>(w, list, kp, chans, done);
     // places: each lane sums three channels, kL lanes make a slot
     const bool sums3 = 3 * lane < W::kTasks;
     const uint32_t k0 = sums3 ? w.kept[3 * lane] : 0u, k1 = sums3 ? w.kept[3 * lane + 1] : 0u;
@@ -617,13 +907,39 @@ __device__ void process_slots(W& w, int n, int c0, const SlotSrc& me, uint32_t e
       if ((lane & (kL - 1)) >= d) incl += y;
     }
     const uint32_t found = __shfl_sync(0xffffffffu, incl, (kL * (lane - done) + kL - 1) & 31);  // of my slot
+    // the strips of their kept clusters, the same way
+    uint32_t a0 = 0, a1 = 0, asum = 0, aincl = 0, strips = 0;
+    if (AMP) {
+      if (sums3) {
+        a0 = w.task[3 * lane];
+        a1 = w.task[3 * lane + 1];
+        asum = a0 + a1 + w.task[3 * lane + 2];
+      }
+      aincl = asum;
+#pragma unroll
+      for (int d = 1; d < kL; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, aincl, d, kL);
+        if ((lane & (kL - 1)) >= d) aincl += y;
+      }
+      strips = __shfl_sync(0xffffffffu, aincl, (kL * (lane - done) + kL - 1) & 31);
+    }
     uint32_t start = 0;
     if (mine) {
+      const uint32_t astart = AMP && strips ? atomicAdd(am.alloc + e, strips) : 0u;
       start = found ? atomicAdd(ev_alloc + e, found) : 0u;
       const uint32_t fits = start < room ? (found < room - start ? found : room - start) : 0u;
       uint32_t fl = w.slot.flags[lane - done];
       if (fits < found) fl |= SST_EV_CLUSTER_CAPACITY;
       const uint32_t nb = w.slot.nbad[lane - done], nd = w.slot.digis[lane - done];
+      if (AMP) {
+        uint32_t lo, hi;
+        amp_slice(am.off, am.cap, e, &lo, &hi);
+        const bool ok = (uint64_t)astart + strips <= hi - lo;
+        if (!ok) fl |= SST_EV_AMP_CAPACITY;
+        am.seg_cnt[seg] = ok ? strips : 0u;
+        am.seg_start[seg] = ok ? astart : kNoAmp;
+        w.slot.nbad[lane - done] = ok ? lo + astart : kNoAmp;
+      }
       if (fl) atomicOr(&status[e].flags, fl);
       if (nb) atomicAdd(&status[e].n_bad_channels, nb);
       if (nd) atomicAdd(&status[e].n_digi, nd);
@@ -631,13 +947,26 @@ __device__ void process_slots(W& w, int n, int c0, const SlotSrc& me, uint32_t e
       seg_start[seg] = start;
     }
     const uint32_t place = __shfl_sync(0xffffffffu, start, (done + lane / kL) & 31) + incl - sum;
+    uint32_t* rel = list.from + kSpillRecords;
     if (sums3) {
       w.task[3 * lane] = place;
       w.task[3 * lane + 1] = place + k0;
       w.task[3 * lane + 2] = place + k0 + k1;
+      if (AMP) {
+        rel[3 * lane] = aincl - asum;
+        rel[3 * lane + 1] = aincl - asum + a0;
+        rel[3 * lane + 2] = aincl - asum + a0 + a1;
+      }
     }
     __syncwarp();
-    write_records<C>(w, list, kp, stage, [&](uint32_t tt) { return ch0 + tt % C; });
+    if (AMP) {
+      // (the fast walk's bytes are counted by shared address, of which 16 bits are enough)
+      write_amplitudes<C>(w, list, kp, stage, am, rel, chans, done,
+                          staged && !any_div ? 0u - (uint32_t)__cvta_generic_to_shared(w.buf) : 0u,
+                          [&](uint32_t i) { return staged ? (uint32_t)w.buf[i] : (uint32_t)src0[i]; });
+    } else {
+      write_records<C>(w, list, kp, stage, [&](uint32_t tt) { return chans.ch0 + chans.of(tt, done); });
+    }
     __syncwarp();
     done += m;
   }
