@@ -1097,18 +1097,20 @@ cudaError_t launch_event(const uint8_t* raw, const uint64_t* event_off, const ui
   });
 }
 
-// Which kernel a batch takes, by its events and its FED records (events x FEDs).
-// Measured on full-detector events (440 FEDs) unless noted, us a batch:
+// Which kernel a batch takes, by its events, FEDs and FED records (events x FEDs).  Times
+// in us a batch; "skewed": the FEDs' densities differ up to a hundredfold either way.
 //   k_event (a CTA per record, one launch) has the shortest critical path but the least
-//   throughput: 1 event 28 (k_stream_fed 31), 2 events 50 (41); 120 FEDs x 4 events 25
-//   (27); with amplitudes, whose second launch is the longer one, 2 events 57 (54), 200
-//   FEDs x 6 events 58 (63);
+//   throughput, and a long FED holds it up most: 440 FEDs x 1 event 28 (k_stream_fed 31),
+//   x 2 50 (41); with amplitudes x 2 57 (54), x 3 skewed 436 (k_stream_fed from here on).
 //   k_stream pays for its tiles: while they all fit the GPU at once (up to 76 FEDs) it is
-//   the fastest of the three from 4 events on (61 FEDs x 4: 20, 23 and 23; x 37: 37, 51
-//   and 64); beyond, from 12 events on (8 events 104, k_stream_fed 91; 16: 118 and 130).
-constexpr uint32_t kEventRecords = 240, kEventRecordsWide = 700, kEventRecordsAmps = 1600;
-constexpr uint32_t kTileEvents = 12, kTileRecords = 3600;
-constexpr uint32_t kTileChunk = 32;
+//   the fastest from 100 records on (13 FEDs x 17 events 18.6 against k_event's 22.5,
+//   skewed 37 against 112; 61 x 2 17.7 and 20.6), but a single FED has 8 tiles (1 x 120:
+//   24 and 18); beyond, from 1,500 records of 10 events and more on (200 x 10 54,
+//   k_stream_fed 59; 120 x 13 43 and 45; 100 x 12 40 and 36; 440 x 8 103 and 86), or of
+//   16 events, or 3,600 records.
+constexpr uint32_t kEventRecords = 100, kEventRecordsOneFed = 240, kEventRecordsWide = 700, kEventRecordsAmps = 850;
+constexpr uint32_t kTileEvents = 10, kTileEventsFew = 16, kTileRecordsFew = 1500, kTileRecords = 3600;
+constexpr uint32_t kTileChunk = 32, kTileChunkMin = 8;
 
 // How a batch is launched.
 struct Plan {
@@ -1131,9 +1133,13 @@ cudaError_t plan_tiles(const Shape& sh, uint32_t n_events, uint32_t n_feds, int 
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const size_t per = sh.ctas_per_sm < kMaxWarpsPerSm / W ? sh.ctas_per_sm : kMaxWarpsPerSm / W;
   const size_t ctas = (size_t)n_sm * per, fit = (size_t)n_sm * per_sm, tiles = (size_t)n_feds * p->segs_per_fed;
-  // few tiles: their events are shared out, down to kTileChunk at a time
+  // Few tiles: their events are shared out, down to kTileChunk at a time for a second
+  // wave and to kTileChunkMin while that is one wave at most (2 FEDs x 147 events: 45 us
+  // with chunks of 37, 33 of 19, 27 of 10; but 3 FEDs x 256: 35 with 384 items, 46 with 768).
   uint32_t chunks = 1;
-  while (tiles * chunks < 2 * fit && (n_events + 2 * chunks - 1) / (2 * chunks) >= kTileChunk) chunks *= 2;
+  auto halves = [&] { return (n_events + 2 * chunks - 1) / (2 * chunks); };  // events of a chunk with twice as many
+  while ((tiles * chunks < 2 * fit && halves() >= kTileChunk) || (2 * tiles * chunks <= fit && halves() >= kTileChunkMin))
+    chunks *= 2;
   p->chunk = (n_events + chunks - 1) / chunks;
   const uint32_t passes = (p->chunk + W * 32 - 1) / (W * 32);  // at most 32 events, a lane each, per warp and pass
   p->per_warp = (p->chunk + W * passes - 1) / (W * passes);
@@ -1146,8 +1152,10 @@ cudaError_t plan_tiles(const Shape& sh, uint32_t n_events, uint32_t n_feds, int 
 cudaError_t plan_batch(const Shape& sh, uint32_t n_events, uint32_t n_feds, bool amps, int n_sm, Plan* p) {
   const size_t records = (size_t)n_events * n_feds;
   const bool one_wave = (size_t)n_feds * kFe <= (size_t)n_sm * 4;  // the tiles fit the GPU at once
-  const bool tiles = n_events >= kTileEvents || one_wave || records > kTileRecords;
-  if (records < (one_wave ? kEventRecords : amps ? kEventRecordsAmps : kEventRecordsWide) &&
+  const bool tiles = one_wave || records > kTileRecords ||
+                     n_events >= (records < kTileRecordsFew ? kTileEventsFew : kTileEvents);
+  if (records < (one_wave ? n_feds > 1 ? kEventRecords : kEventRecordsOneFed
+                 : amps ? kEventRecordsAmps : kEventRecordsWide) &&
       (one_wave || !tiles)) {
     p->kind = Plan::kFeds;
     p->grid = (int)records;
@@ -1169,12 +1177,13 @@ cudaError_t plan_batch(const Shape& sh, uint32_t n_events, uint32_t n_feds, bool
   if (e) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const size_t per = sh.ctas_per_sm < per_sm ? sh.ctas_per_sm : per_sm, ctas = (size_t)n_sm * per;
-  // FE units per warp: few enough that every warp has an item, but no fewer than half a
-  // FED's (a quarter's channels leave lanes idle) once that makes a wave, and a whole FED's
-  // when halves make more than two (6 events: 77 with halves, 86 with whole FEDs)
+  // FE units per warp: as few as give every warp one item, half a FED's at most (48
+  // channels); two (24 channels, evener shares) where halves fill more than two thirds of
+  // a wave: 440 FEDs x 3 events 56.6 with halves, 57.3 with quarters, but 256 and 161
+  // when the FEDs' densities differ a hundredfold; 440 x 5 77 and 69; 150 x 8 36 and 42
   p->units = 1;
   while (p->units < kFe / 2 && records * (kFe / p->units) > ctas * kFedWarps) p->units *= 2;
-  if (records * 2 > 2 * ctas * kFedWarps) p->units = kFe;
+  if (records * 3 > ctas * kFedWarps) p->units = 2;
   const size_t need = (records * (kFe / p->units) + kFedWarps - 1) / kFedWarps;
   p->grid = (int)(ctas < need ? ctas : need);
   p->resident = p->grid;

@@ -98,7 +98,7 @@ def test_per_event(small):
 
 
 @pytest.mark.parametrize("amps", [False, True])
-@pytest.mark.parametrize("n_events", [1, 3, 59, 60])  # 236 FED records: a CTA each; 240: channel streams
+@pytest.mark.parametrize("n_events", [1, 3, 24, 25, 60])  # 96 FED records: a CTA each; 100: channel streams
 def test_few_events(small, n_events, amps):
     g, pats = small
     pats = list(pats.values())
@@ -109,9 +109,11 @@ def test_few_events(small, n_events, amps):
 
 
 @pytest.mark.parametrize("n_feds,n_events,amps", [
-    (77, 9, False), (77, 10, False), (77, 11, False), (77, 12, False),  # 693 | 770 records, 11 | 12 events
-    (145, 11, True), (146, 11, True), (146, 12, True),                  # 1,595 | 1,606 records
-    (360, 10, False), (361, 10, True),                                  # 3,600 | 3,610 records
+    (1, 239, False), (1, 240, False), (1, 99, True), (2, 49, True), (2, 50, True),
+    (77, 9, False), (77, 10, False), (77, 15, False), (77, 16, False),  # 693 | 770 records, 15 | 16 events
+    (150, 9, False), (150, 10, False), (149, 10, False),                # 9 | 10 events, 1,500 | 1,490 records
+    (77, 11, True), (86, 10, True), (150, 10, True),                    # 847 | 860 records
+    (400, 9, False), (401, 9, True),                                    # 3,600 | 3,609 records
 ])
 def test_choice_of_kernel(n_feds, n_events, amps):
     calib = eg.make_calibration(n_feds, 17, 0.02)
