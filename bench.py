@@ -352,7 +352,7 @@ def measured_peaks():
 def kernel_traffic():
     """DRAM bytes per launch of the batched kernel from the committed ncu summary,
     or None when the kernel source has changed since it was captured."""
-    p = os.path.join(ROOT, "profiles", "k_batch_traffic.json")
+    p = os.path.join(ROOT, "profiles", "k_stream_traffic.json")
     if not os.path.exists(p):
         return None
     d = json.load(open(p))
@@ -364,7 +364,7 @@ def kernel_traffic():
 def kernel_source_sha256():
     """SHA-256 over the sources the batched kernel is compiled from, in this order."""
     h = hashlib.sha256()
-    for f in ("sst_kernels.cu", "sst_fe.cuh", "sst_internal.h"):
+    for f in ("sst_kernels.cu", "sst_stream.cuh", "sst_internal.h"):
         h.update(open(os.path.join(ROOT, "paper_2101_11489_gb300", "csrc", f), "rb").read())
     return h.hexdigest()
 
@@ -384,15 +384,14 @@ def algorithmic_bytes(events, n_digi, n_clusters):
 def kernel_bytes(events, n_digi, n_clusters):
     """Bytes the batched kernel's own dataflow touches per launch (a finer model
     than algorithmic_bytes, for comparison with the measured DRAM traffic): the
-    payload; the per-strip calibration word and noise^2 of every recorded strip (4
-    + 4 B); the APV multipliers (8 B per channel); the FE-unit descriptors the
-    prologue wrote (8 B per unit) and the FED lengths and offsets (4 + 8 B per
-    FED); the staged cluster records (16 B per cluster); the event status.  The
-    bad-strip masks are read only when clusters are widened over bad strips, which
-    the default parameters do not."""
+    payload; the calibration entry of every recorded strip (8 B); the APV
+    multipliers (8 B per channel); the FE-unit descriptors the prologue wrote (8 B
+    per unit) and the FED lengths and offsets (4 + 8 B per FED); the staged cluster
+    records (8 B per cluster); the event status.  The bad-strip masks are read only
+    when clusters are widened over bad strips, which the default parameters do not."""
     payload = sum(int(e[0].size) for e in events)
     n_feds = sum(int(e[1].size) for e in events)
-    return (payload + 8 * n_digi + n_feds * 96 * 8 + n_feds * 8 * 8 + 12 * n_feds + 16 * n_clusters
+    return (payload + 8 * n_digi + n_feds * 96 * 8 + n_feds * 8 * 8 + 12 * n_feds + 8 * n_clusters
             + 16 * len(events))
 
 
@@ -742,7 +741,7 @@ def main():
             "gpu_launches": 3 * args.steps,
             "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                          "frac": round(achieved / peak, 4), "traffic": traffic,
-                         "kernel": "k_batch", "kernels_per_step": 3, "kernel_ms": round(k_ms, 4), "algorithmic_bytes": int(b_alg),
+                         "kernel": "k_stream", "kernels_per_step": 3, "kernel_ms": round(k_ms, 4), "algorithmic_bytes": int(b_alg),
                          "bytes_definition": "payload + 4 B noise and a bad-strip bit per recorded strip + APV "
                                              "gains + fed_len/fed_off + 16 B per cluster + 16 B status per event",
                          "traffic_model": {"bytes": int(b_kern), "achieved": round(b_kern / (k_ms / 1e3) / 1e9, 1),
@@ -898,11 +897,11 @@ def run_single(args, rank, world, local, wid):
             "graph": {"value": round(world * 1e3 / g_ms, 1), "unit": "events/s", "ms_per_step": round(g_ms, 4),
                       "steps": g_steps, "what": "the same launch sequence captured once as a CUDA graph and "
                                                 "replayed (median step)"},
-            "gpu_launches": 5 * args.steps,
+            "gpu_launches": 2 * args.steps,
             "roofline": {"bound": "hbm", "achieved": round(b_alg / (mean_ms / 1e3) / 1e9, 1), "peak": peak,
                          "unit": "GB/s", "frac": round(b_alg / (mean_ms / 1e3) / 1e9 / peak, 4), "traffic": None,
-                         "kernel": "the per-event launch sequence (k_fed_scan, k_unpack, k_cluster, k_order and a "
-                                   "memset): launch- and latency-bound at one event per launch",
+                         "kernel": "the per-event launch sequence (k_unpack, k_cluster): launch- and latency-bound "
+                                   "at one event per launch",
                          "algorithmic_bytes": int(b_alg), "peak_kind": peak_kind},
             "cpu_baseline": cpu, "clocks": clk,
         }), flush=True)

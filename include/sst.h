@@ -237,8 +237,8 @@ sst_status sst_cluster(sst_ctx* ctx, const sst_digis* in, uint32_t n_feds, const
  * cudaMalloc synchronise the device under a real-time pipeline).  It needs no
  * context: it unpacks exactly as sst_unpack does (same arguments, same outputs,
  * same status semantics), on the current CUDA device, with its scratch in a fixed
- * device array of the library (SST_NOALLOC_MAX_FEDS look-back states and FED
- * offsets, about 16 KiB per device, held until the process exits).  It calls no
+ * device array of the library (two sets of SST_NOALLOC_MAX_FEDS look-back states,
+ * about 16 KiB per device, held until the process exits).  It calls no
  * cudaMalloc, cudaFree or allocating routine.
  *   - n_feds > SST_NOALLOC_MAX_FEDS returns SST_ERR_TOO_LARGE; a null pointer, a
  *     misaligned raw buffer or n_feds == 0 returns SST_ERR_INVALID_ARG; a CUDA
@@ -248,19 +248,20 @@ sst_status sst_cluster(sst_ctx* ctx, const sst_digis* in, uint32_t n_feds, const
  *     stream.
  *   - All calls on a device share the one array: calls whose work overlaps on the
  *     GPU (different streams, not ordered) race and give wrong results.  Every call
- *     clears what must start at zero on its own stream before its kernels run. */
+ *     finds its set cleared: by the call before, or, once a call was captured into a
+ *     graph, by itself on its own stream before its kernel runs. */
 #define SST_NOALLOC_MAX_FEDS 1024u
 sst_status sst_unpack_noalloc(const uint8_t* raw, uint64_t raw_bytes, const uint32_t* fed_len, uint32_t n_feds,
                               const sst_digis* out, void* stream);
 
 /* ---- batched path (section 3: many events concurrently on one GPU) -------------- */
 
-/* Unpacks and clusters n_events events in one persistent launch; digis stay on
- * chip.  Each warp takes two adjacent FE units at a time; their clusters are
- * staged (context scratch of out->capacity records), then ordered and copied per
- * event by one more kernel (two with amplitudes).  The launch sequence allocates nothing once the context
- * has run one batch of this size, so it can be captured in a CUDA graph.  All
- * pointers are device memory:
+/* Unpacks and clusters n_events events; digis stay on chip.  The smallest batches
+ * take one launch, a block per FED record.  In larger ones a lane reads a channel
+ * record; the clusters are staged (context scratch of out->capacity records), then
+ * ordered and copied per event by one more kernel (two with amplitudes).  The
+ * launch sequence allocates nothing once the context has run one batch of this
+ * size, so it can be captured in a CUDA graph.  All pointers are device memory:
  *   raw        events back to back; event e occupies [event_off[e], event_off[e+1]),
  *              every event_off[e] a multiple of 16
  *   event_off  [n_events + 1] uint64
@@ -351,7 +352,7 @@ sst_status sst_local_x(sst_ctx* ctx, const uint32_t* det, const float* barycente
 typedef struct {
   uint32_t block;             /* batched kernel: threads per CTA, 128 or 256 */
   uint32_t ctas_per_sm;       /* batched kernel: persistent CTAs per SM, 1..8 (clamped to what fits) */
-  uint32_t units_per_warp;    /* batched kernel: FE units per warp work item, 1 or 2 (12 or 24 channels) */
+  uint32_t units_per_warp;    /* batched kernel: 1 or 2: a warp stages up to 4 or 8 FE units' records at once */
   uint32_t host_chunk_events; /* sst_batch_host: events per pipeline chunk (the batch depth of each
                                  launch), 0..4096; 0 = automatic (a quarter of the batch, at most 32) */
   uint32_t tile_digis;        /* per-event unpack (sst_unpack): digis per on-chip tile, 1024, 2048 or 4096 */
@@ -363,8 +364,8 @@ sst_status sst_set_tune(sst_ctx* ctx, const sst_tune* t);
 sst_status sst_get_tune(const sst_ctx* ctx, sst_tune* t);
 
 /* Times every candidate shape of the batched kernel on the given batch (same
- * arguments as sst_batch; the outputs are overwritten): block 128 / 256 x work
- * items of 1 / 2 FE units x 2..8 CTAs per SM (shapes that cannot be resident, or
+ * arguments as sst_batch; the outputs are overwritten): block 128 / 256 x
+ * units_per_warp 1 / 2 x 2..8 CTAs per SM (shapes that cannot be resident, or
  * that the occupancy clamps to a shape already timed, are skipped).  Each shape
  * runs one untimed and two timed launch sequences.  Keeps the fastest in the
  * context and returns it in *best with its time per launch sequence in *best_us.

@@ -2,15 +2,15 @@
 // three-threshold clustering (arXiv 2101.11489, section 2), per event and batched
 // (section 3).
 //
-// Batches of many events (k_stream, sst_stream.cuh): one lane per channel record, the
-// calibration entries of one FE unit in shared memory while all events' records of it
-// pass.  The FED headers are checked by a prologue (k_fed_scan), which hands every FE
+// Batches (k_stream, sst_stream.cuh): one lane per channel record, the calibration
+// entries of one FE unit in shared memory while all events' records of it pass; where
+// the events are too few for that, each warp reads them from global memory
+// (k_stream_fed).  The FED headers are checked by a prologue (k_fed_scan), which hands every FE
 // unit its byte range; the kept clusters are staged per FE unit and event and put in
 // order by k_order.  Placing them with a look-back over the units before instead
 // would make every warp wait for units that other CTAs take at the same time.
 //
-// Single events, batches of few, and clusters with amplitudes (k_unpack, k_cluster,
-// k_event, sst_event.cuh): one CTA per FED, which finds its record, and with a
+// Single events and the smallest batches (k_unpack, k_cluster, k_event, sst_event.cuh): one CTA per FED, which finds its record, and with a
 // look-back over the FEDs before it its place in the output, by itself; one launch
 // per call.
 //
