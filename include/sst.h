@@ -27,6 +27,9 @@
  * synchronises the device, so make one warm-up call before capturing a stream
  * into a CUDA graph.  Contexts are independent; one context must not be used from
  * two host threads at once, except sst_submit / sst_poll, which are thread safe.
+ * Calls of one context on different streams are ordered by the caller; only
+ * sst_unpack of one event may overlap sst_cluster of another (each has scratch of
+ * its own).
  */
 #ifndef SST_H
 #define SST_H

@@ -41,8 +41,7 @@ static cudaError_t grow(T*& p, size_t& cap, size_t need) {
   return e;
 }
 
-// Two cleared sets of shared state for `events` events of `feds` FEDs in all.
-static cudaError_t grow_look(LookState& l, size_t events, size_t feds) {
+cudaError_t ensure_look(LookState& l, size_t events, size_t feds) {
   const size_t words = LookState::words_for(events, 1) + feds + 3 * (feds / 1024 + 1);
   if (words <= l.cap) return cudaSuccess;
   const bool replayed = l.replayed;
@@ -79,7 +78,7 @@ cudaError_t ensure_scratch(Scratch& s, size_t items, size_t events, size_t stage
     }
     if ((e = grow(s.ev_alloc, s.ev_cap, events))) return e;
     if ((e = grow(s.stage, s.stage_cap, stage_records))) return e;
-    if ((e = grow_look(s.look, s.ev_cap, s.items_cap / kFe))) return e;
+    if ((e = ensure_look(s.look, s.ev_cap, s.items_cap / kFe))) return e;
   }
   return cudaSuccess;
 }
@@ -117,7 +116,8 @@ cudaError_t ensure_amp_scratch(Scratch& s, size_t amp_bytes) {
 }
 
 void free_scratch(Scratch& s) {
-  if (s.look.words) cudaFree(s.look.words);
+  for (LookState* l : {&s.look, &s.look_unpack, &s.look_cluster})
+    if (l->words) cudaFree(l->words);
   if (s.fed_off) cudaFree(s.fed_off);
   if (s.fed_cnt) cudaFree(s.fed_cnt);
   if (s.fed_start) cudaFree(s.fed_start);
@@ -157,6 +157,8 @@ sst_status sst_create(sst_ctx** out, int device, uint32_t n_feds) {
   c->shape = default_shape();
   DeviceGuard g(device);
   cudaError_t e = cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, device);
+  if (e == cudaSuccess) e = ensure_look(c->scratch.look_unpack, 1, n_feds);
+  if (e == cudaSuccess) e = ensure_look(c->scratch.look_cluster, 1, n_feds);
   if (e == cudaSuccess) e = ensure_scratch(c->scratch, (size_t)n_feds * kFe, 1, 1);
   // (its one size: launches captured into a graph keep its address)
   if (e == cudaSuccess) e = ensure_spill(c->scratch, (size_t)c->n_sm * kMaxWarpsPerSm);

@@ -65,7 +65,8 @@ struct LookState {
 // stream): the state shared by the CTAs of the one-CTA-per-FED kernels, work tickets,
 // and the many-event kernel's FED offsets, cluster bookkeeping and staging buffer.
 struct Scratch {
-  LookState look;
+  LookState look;                       // k_event's
+  LookState look_unpack, look_cluster;  // the per-event calls', which may overlap on two streams (contexts only)
   uint64_t* fed_off = nullptr;       // absolute byte offset per (event, FED)
   uint32_t* fed_cnt = nullptr;       // clusters found per segment (event, FE unit or half of one)
   uint32_t* fed_start = nullptr;     // staging offset per segment, within its event's slice
@@ -163,6 +164,8 @@ sst_status set_err(sst_ctx* c, sst_status code, const std::string& msg);
 sst_status cuda_err(sst_ctx* c, cudaError_t e, const char* where);
 KParams kparams(const sst_ctx* c);
 cudaError_t ensure_scratch(Scratch& s, size_t items, size_t events, size_t stage_records);
+// Two cleared sets of shared state for `events` events of `feds` FEDs in all; grows only.
+cudaError_t ensure_look(LookState& l, size_t events, size_t feds);
 // Candidate lists for `warps` warps of k_stream; grows only.
 cudaError_t ensure_spill(Scratch& s, size_t warps);
 // What k_stream needs for amplitudes beside the above (after ensure_scratch and

@@ -1078,7 +1078,7 @@ template <int TILE>
 cudaError_t launch_unpack_t(const uint8_t* raw, uint64_t raw_bytes, const uint32_t* fed_len, uint32_t n_feds,
                             const sst_digis& out, Scratch& s, const Shape& shape, cudaStream_t st) {
   const size_t sm = sizeof(ev::Shm<TILE, false>);
-  return launch_feds((const void*)k_unpack<TILE>, sm, s.look, 1, n_feds, s.lb_spin_limit, st, [&](ev::Shared& sh) {
+  return launch_feds((const void*)k_unpack<TILE>, sm, s.look_unpack, 1, n_feds, s.lb_spin_limit, st, [&](ev::Shared& sh) {
     sh.withhold = s.lb_withhold;
     return launch_pdl(k_unpack<TILE>, n_feds, (unsigned)ev::kThreads, sm, st, raw, raw_bytes, fed_len, out, sh,
                       shape.lanes);
@@ -1285,7 +1285,7 @@ cudaError_t launch_cluster(const sst_digis& in, uint32_t n_feds, const sst_clust
                            Scratch& s, cudaStream_t st) {
   const size_t sm = sizeof(ev::Shm<kEvTile, true>);
   auto* k = out.amp ? k_cluster<true> : k_cluster<false>;
-  return launch_feds((const void*)k, sm, s.look, 1, n_feds, s.lb_spin_limit, st, [&](ev::Shared& sh) {
+  return launch_feds((const void*)k, sm, s.look_cluster, 1, n_feds, s.lb_spin_limit, st, [&](ev::Shared& sh) {
     return launch_pdl(k, n_feds, (unsigned)ev::kThreads, sm, st, in, with_spill(kp, s), out, sh);
   });
 }

@@ -25,7 +25,7 @@ constexpr size_t kWords = sst::LookState::words_for(1, kMaxFeds);
 static __device__ __align__(256) unsigned long long g_scratch[2 * kWords];
 
 std::mutex g_mu;
-sst::Scratch g_state[kMaxDevices];  // per device; look.words is g_scratch's address there, once known
+sst::Scratch g_state[kMaxDevices];  // per device; look_unpack.words is g_scratch's address there, once known
 
 // Finds g_scratch's address on the current device (on the first call for that device).
 cudaError_t find_scratch(sst::LookState& l) {
@@ -51,7 +51,7 @@ extern "C" sst_status sst_unpack_noalloc(const uint8_t* raw, uint64_t raw_bytes,
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return SST_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_mu);
   sst::Scratch& s = g_state[dev];
-  if (find_scratch(s.look) != cudaSuccess) return SST_ERR_CUDA;
+  if (find_scratch(s.look_unpack) != cudaSuccess) return SST_ERR_CUDA;
   const cudaError_t e = sst::launch_unpack(raw, raw_bytes, fed_len, n_feds, *out, s, sst::default_shape(),
                                            static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? SST_OK : SST_ERR_CUDA;
