@@ -25,11 +25,12 @@
  * owns its device calibration tables and its internal scratch (look-back flags,
  * work tickets), which it sizes on first use; a call that has to grow scratch
  * synchronises the device, so make one warm-up call before capturing a stream
- * into a CUDA graph.  Contexts are independent; one context must not be used from
- * two host threads at once, except sst_submit / sst_poll, which are thread safe.
- * Calls of one context on different streams are ordered by the caller; only
- * sst_unpack of one event may overlap sst_cluster of another (each has scratch of
- * its own).
+ * into a CUDA graph.  Growing scratch also ends the batched graphs captured before
+ * (their launches keep the old buffers); those of the per-event calls stay valid.
+ * Contexts are independent; one context must not be used from two host threads at
+ * once, except sst_submit / sst_poll, which are thread safe.  Calls of one context
+ * on different streams are ordered by the caller; only sst_unpack of one event may
+ * overlap sst_cluster of another (each has scratch of its own).
  */
 #ifndef SST_H
 #define SST_H
@@ -240,8 +241,8 @@ sst_status sst_cluster(sst_ctx* ctx, const sst_digis* in, uint32_t n_feds, const
  * cudaMalloc synchronise the device under a real-time pipeline).  It needs no
  * context: it unpacks exactly as sst_unpack does (same arguments, same outputs,
  * same status semantics), on the current CUDA device, with its scratch in a fixed
- * device array of the library (two sets of SST_NOALLOC_MAX_FEDS look-back states,
- * about 16 KiB per device, held until the process exits).  It calls no
+ * device array of the library (SST_NOALLOC_MAX_FEDS look-back states and the work
+ * tickets, about 16 KiB per device, held until the process exits).  It calls no
  * cudaMalloc, cudaFree or allocating routine.
  *   - n_feds > SST_NOALLOC_MAX_FEDS returns SST_ERR_TOO_LARGE; a null pointer, a
  *     misaligned raw buffer or n_feds == 0 returns SST_ERR_INVALID_ARG; a CUDA
@@ -250,9 +251,8 @@ sst_status sst_cluster(sst_ctx* ctx, const sst_digis* in, uint32_t n_feds, const
  *     device (cudaGetSymbolAddress); make that first call before capturing any
  *     stream.
  *   - All calls on a device share the one array: calls whose work overlaps on the
- *     GPU (different streams, not ordered) race and give wrong results.  Every call
- *     finds its set cleared: by the call before, or, once a call was captured into a
- *     graph, by itself on its own stream before its kernel runs. */
+ *     GPU (different streams, not ordered) race and give wrong results.  A call
+ *     depends on nothing that an earlier one left there. */
 #define SST_NOALLOC_MAX_FEDS 1024u
 sst_status sst_unpack_noalloc(const uint8_t* raw, uint64_t raw_bytes, const uint32_t* fed_len, uint32_t n_feds,
                               const sst_digis* out, void* stream);

@@ -41,18 +41,20 @@ static cudaError_t grow(T*& p, size_t& cap, size_t need) {
   return e;
 }
 
-cudaError_t ensure_look(LookState& l, size_t events, size_t feds) {
-  const size_t words = LookState::words_for(events, 1) + feds + 3 * (feds / 1024 + 1);
-  if (words <= l.cap) return cudaSuccess;
-  const bool replayed = l.replayed;
-  if (l.words) cudaFree(l.words);
-  l = LookState{};
-  cudaError_t e = cudaMalloc(&l.words, 2 * words * sizeof(*l.words));
-  if (!e) e = cudaMemset(l.words, 0, 2 * words * sizeof(*l.words));
+cudaError_t ensure_look(LookState& l, size_t events, size_t items) {
+  if (l.words) return cudaSuccess;
+  const size_t bytes = LookState::words_for(events, items) * sizeof(*l.words);
+  unsigned long long* p = nullptr;
+  cudaError_t e = cudaMalloc(&p, bytes);
+  if (!e) e = cudaMemset(p, 0, bytes);
   if (!e) e = cudaDeviceSynchronize();  // cleared for every stream
-  if (e) return e;
-  l.cap = words;
-  l.replayed = replayed;
+  if (e) {
+    cudaFree(p);
+    return e;
+  }
+  l.words = p;
+  l.events = events;
+  l.items = items;
   return cudaSuccess;
 }
 
@@ -62,6 +64,7 @@ cudaError_t ensure_scratch(Scratch& s, size_t items, size_t events, size_t stage
     if ((e = cudaMalloc(&s.tickets, 16 * sizeof(uint32_t)))) return e;
     if ((e = cudaMemset(s.tickets, 0, 16 * sizeof(uint32_t)))) return e;
   }
+  if ((e = ensure_look(s.look_event, kEventRecordsMost, kEventRecordsMost))) return e;
   items = items ? items : 1;
   events = events ? events : 1;
   stage_records = stage_records ? stage_records : 1;
@@ -78,7 +81,6 @@ cudaError_t ensure_scratch(Scratch& s, size_t items, size_t events, size_t stage
     }
     if ((e = grow(s.ev_alloc, s.ev_cap, events))) return e;
     if ((e = grow(s.stage, s.stage_cap, stage_records))) return e;
-    if ((e = ensure_look(s.look, s.ev_cap, s.items_cap / kFe))) return e;
   }
   return cudaSuccess;
 }
@@ -116,7 +118,7 @@ cudaError_t ensure_amp_scratch(Scratch& s, size_t amp_bytes) {
 }
 
 void free_scratch(Scratch& s) {
-  for (LookState* l : {&s.look, &s.look_unpack, &s.look_cluster})
+  for (LookState* l : {&s.look_unpack, &s.look_cluster, &s.look_event})
     if (l->words) cudaFree(l->words);
   if (s.fed_off) cudaFree(s.fed_off);
   if (s.fed_cnt) cudaFree(s.fed_cnt);

@@ -6,7 +6,7 @@
 // steps of one FED, so every step is spread over the CTA's threads and everything
 // around the step is kept short: no prologue (a CTA sums the FED lengths before its
 // own), no ordering pass (a CTA sums the counts that the FEDs before it publish) and
-// no clearing between launches (each clears what the launch before it used).  An event
+// no clearing between launches (what a launch reads carries its tag).  An event
 // of 440 FEDs took 48 us in four launches and a memset, a warp per FE unit; it takes 35
 // in two (8 FEDs: 29 and 17; the allocation-free unpack of 440 FEDs: 22 and 12.5).
 //
@@ -21,15 +21,17 @@ constexpr int kFedBuf = 8192;      // bytes of FED record staged on chip (larger
 constexpr int kRunSlots = (kFedBuf + 2) / 3;  // a run header takes at least 3 bytes with its ADC
 constexpr uint32_t kFedClusters = kCh * kStrips / 2;  // most clusters of a FED
 constexpr uint32_t kLbBlock = 1024;  // FEDs whose counts a CTA sums one by one
-constexpr unsigned long long kSet = 1ull << 63;
+constexpr uint32_t kNoStatus = 0xFFFFFFFFu;
+static_assert(kLbBlock == 1024 && LookState::kTags == 1024, "sizes of the shared state (LookState)");
 
-// State shared by the CTAs of a launch, zero when it starts.
+// State shared by the CTAs of a launch.
 struct Shared {
-  uint32_t* ticket;         // next item
-  uint32_t* acc;            // [events][2]: flags, bad channels
-  unsigned long long* lb;   // [n_items] counts, then [2 * (n_items / kLbBlock + 1)] prefixes (below)
-  unsigned long long* clear;  // the state of the launch before, to be zeroed for the next one
-  uint32_t n_clear;         // its words
+  uint32_t* ticket;         // next item; zero when the launch starts
+  unsigned long long* lb;   // [n_items] what the items published (Counts::word)
+  unsigned long long* pre;  // [n_items / kLbBlock + 1][4] sums (look_back)
+  uint32_t* late;           // [events] the launch's tag once a wait for the event's place has run out
+  uint32_t* st;             // [n_items] channel statuses | bad channels << 8, where the count says so
+  uint32_t tag;             // the launch's: 1 .. LookState::kTags - 1
   uint32_t n_items;         // events x FEDs
   uint32_t n_feds;
   uint32_t spin_limit;      // polls before a wait gives up
@@ -72,7 +74,6 @@ template <class S, typename Meanwhile>
 __device__ __forceinline__ uint32_t take_item(S& s, const Shared& sh, Meanwhile meanwhile) {
   uint32_t t = 0;
   if (threadIdx.x == 0) t = atomicAdd(sh.ticket, 1u);
-  for (uint32_t i = blockIdx.x * kThreads + threadIdx.x; i < sh.n_clear; i += gridDim.x * kThreads) sh.clear[i] = 0;
   meanwhile();
   if (threadIdx.x == 0) s.scal[kIdx] = t;
   __syncthreads();
@@ -122,41 +123,61 @@ __device__ __forceinline__ uint32_t block_scan(S& s, uint32_t v, uint32_t* total
   return warps_before(s, __shfl_sync(0xffffffffu, x, 31), total) + x - v;
 }
 
-// What a FED publishes: clusters (below 2^15), digis (below 2^16) and the strips of its
-// clusters (below 2^30), in one word with kSet.  Its channel statuses go to the event's
-// words first, so that whoever has read the count sees them too.
+// What a FED publishes in one word: clusters (at most 96 x 256), digis (the same), the
+// strips of its clusters (at most 256 each), whether it has channel statuses and the
+// launch's tag.  The statuses, which few FEDs have, are in a word of their own, written
+// before.
 struct Counts {
   unsigned long long clusters = 0, digis = 0, amps = 0;
-  __device__ __forceinline__ unsigned long long word() const { return kSet | (amps << 32) | (digis << 16) | clusters; }
+  uint32_t flags = 0, bad = 0;  // OR of the channel statuses, bad channels
+  static constexpr unsigned long long kStatus = 1ull << 53;
+  static constexpr int kTagAt = 54;
+  __device__ __forceinline__ unsigned long long word(uint32_t tag) const {
+    return ((unsigned long long)tag << kTagAt) | (bad ? kStatus : 0ull) | (amps << 30) | (digis << 15) | clusters;
+  }
   __device__ __forceinline__ void add(unsigned long long w) {
-    clusters += w & 0xFFFFull;
-    digis += (w >> 16) & 0xFFFFull;
-    amps += (w >> 32) & 0x3FFFFFFFull;
+    clusters += w & 0x7FFFull;
+    digis += (w >> 15) & 0x7FFFull;
+    amps += (w >> 30) & 0x7FFFFFull;
   }
 };
-__device__ __forceinline__ void publish(const Shared& sh, uint32_t idx, uint32_t e, const Counts& c, uint32_t flags,
-                                        uint32_t nbad) {
-  if (flags) atomicOr(sh.acc + 2 * (size_t)e, flags);
-  if (nbad) atomicAdd(sh.acc + 2 * (size_t)e + 1, nbad);
-  if ((int64_t)idx != (int64_t)sh.withhold) st_release(sh.lb + idx, c.word());
+static_assert(kCh * kStrips < 1 << 15 && kCh * kStrips * kStrips < 1 << 23 && LookState::kTags <= 1 << 10,
+              "fields of a count's word");
+__device__ __forceinline__ void publish(const Shared& sh, uint32_t idx, const Counts& c) {
+  if (c.bad) sh.st[idx] = c.flags | (c.bad << 8);
+  if ((int64_t)idx != (int64_t)sh.withhold) st_release(sh.lb + idx, c.word(sh.tag));
+}
+
+// OR over the CTA's threads (all call; two barriers).
+template <class S>
+__device__ __forceinline__ uint32_t block_or(S& s, uint32_t v) {
+  v = __reduce_or_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) s.sum[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = __reduce_or_sync(0xffffffffu, threadIdx.x % 32 < kWarps ? s.sum[threadIdx.x % 32] : 0u);
+  __syncthreads();
+  return v;
 }
 
 // What the items lo .. idx - 1 published, summed (all threads call).  The counts of
 // up to kLbBlock items are read at once, a few by each thread, so that a CTA waits for
 // the slowest of them and not for a chain; further back, the last item of every
-// kLbBlock (last_of_block) publishes the sums up to and including itself, with its own
-// counts.  A wait gives up after spin_limit polls: *timed_out is set and the sums are
-// partial.
+// kLbBlock publishes the sums up to and including itself, with its own counts `own`.
+// st_from: the first item whose statuses are wanted (kNoStatus: none).  A wait gives up
+// after spin_limit polls: *timed_out is set and the sums are partial.
 template <bool AMP, class S>
-__device__ __forceinline__ Counts look_back(S& s, const Shared& sh, uint32_t idx, uint32_t lo, const Counts& own,
-                                            bool last_of_block, bool* timed_out) {
+__device__ __forceinline__ Counts look_back(S& s, const Shared& sh, uint32_t idx, uint32_t lo, uint32_t st_from,
+                                            const Counts& own, bool* timed_out) {
   const uint32_t w0 = idx & ~(kLbBlock - 1u), from = w0 > lo ? w0 : lo;
+  const bool last_of_block = lo == 0 && (idx & (kLbBlock - 1u)) == kLbBlock - 1u;
+  if (last_of_block) st_from = 0;
+  constexpr unsigned long long kSums = (1ull << Counts::kTagAt) - 1u;
   Counts c;
   bool to = false;
   auto poll = [&](const unsigned long long* p) -> unsigned long long {
     unsigned long long v = ld_acquire(p);
     unsigned ns = 32;
-    for (uint32_t k = 0; !(v & kSet); v = ld_acquire(p)) {
+    for (uint32_t k = 0; (uint32_t)(v >> Counts::kTagAt) != sh.tag; v = ld_acquire(p)) {
       if (to || ++k > sh.spin_limit) {
         to = true;
         return 0ull;
@@ -166,13 +187,26 @@ __device__ __forceinline__ Counts look_back(S& s, const Shared& sh, uint32_t idx
     }
     return v;
   };
-  for (uint32_t i = from + threadIdx.x; i < idx; i += kThreads) c.add(poll(sh.lb + i));
+  for (uint32_t i = from + threadIdx.x; i < idx; i += kThreads) {
+    const unsigned long long w = poll(sh.lb + i);
+    c.add(w);
+    if ((w & Counts::kStatus) && i >= st_from) {
+      const uint32_t st = __ldcg(sh.st + i);
+      c.flags |= st & 255u;
+      c.bad += st >> 8;
+    }
+  }
   if (from > lo && threadIdx.x == 0) {  // the sums up to item from - 1
-    const unsigned long long* pre = sh.lb + sh.n_items + 3 * (size_t)(from / kLbBlock - 1);
-    c.clusters += poll(pre) & ~kSet;
+    const unsigned long long* pre = sh.pre + 4 * (size_t)(from / kLbBlock - 1);
+    c.clusters += poll(pre) & kSums;
     if (!to) {
       c.digis += __ldcg(pre + 1);
       c.amps += __ldcg(pre + 2);
+      if (st_from != kNoStatus) {
+        const unsigned long long st = __ldcg(pre + 3);
+        c.flags |= (uint32_t)(st >> 32);
+        c.bad += (uint32_t)st;
+      }
     }
   }
   // clusters and digis in one sum (each below 2^32 within one block of items)
@@ -185,31 +219,35 @@ __device__ __forceinline__ Counts look_back(S& s, const Shared& sh, uint32_t idx
     c.digis = block_sum(s, c.digis);
     if (AMP) c.amps = block_sum(s, c.amps);
   }
+  if (st_from != kNoStatus && __syncthreads_or(c.bad != 0)) {
+    c.flags = block_or(s, c.flags);
+    c.bad = (uint32_t)block_sum(s, c.bad);
+  }
   to = __syncthreads_or(to);
   if (threadIdx.x == 0 && last_of_block && (int64_t)idx != (int64_t)sh.withhold) {
-    unsigned long long* pre = sh.lb + sh.n_items + 3 * (size_t)(idx / kLbBlock);
+    unsigned long long* pre = sh.pre + 4 * (size_t)(idx / kLbBlock);
     pre[1] = c.digis + own.digis;
     pre[2] = c.amps + own.amps;
+    pre[3] = ((unsigned long long)(c.flags | own.flags) << 32) | (c.bad + own.bad);
     __threadfence();
-    st_release(pre, kSet | (c.clusters + own.clusters));
+    st_release(pre, ((unsigned long long)sh.tag << Counts::kTagAt) | (c.clusters + own.clusters));
   }
   *timed_out = to;
   return c;
 }
 
 // An event's flags, written by its last FED's CTA (which has seen every FED's count,
-// and with it the statuses): `flags` and what the event's word holds.  A CTA whose wait
-// ran out adds SST_EV_TIMEOUT to the word and then to the flags; with the word read
-// after the flags are written, one of the two is seen.
+// and with it the statuses), and SST_EV_TIMEOUT when a wait for the event's place ran
+// out.  A CTA whose wait did marks the event's word and then adds the flag; with the word
+// read after the flags are written, one of the two is seen.
 __device__ __forceinline__ void write_flags(const Shared& sh, uint32_t e, uint32_t flags, sst_event_status* st) {
   volatile uint32_t* f = &st->flags;
   *f = flags;
   __threadfence();
-  const uint32_t w = atomicOr(sh.acc + 2 * (size_t)e, 0u);
-  if (w) atomicOr(&st->flags, w);
+  if (atomicOr(sh.late + e, 0u) == sh.tag) atomicOr(&st->flags, SST_EV_TIMEOUT);
 }
 __device__ __forceinline__ void flag_timeout(const Shared& sh, uint32_t e, sst_event_status* st) {
-  atomicOr(sh.acc + 2 * (size_t)e, SST_EV_TIMEOUT);
+  atomicExch(sh.late + e, sh.tag);
   __threadfence();
   atomicOr(&st->flags, SST_EV_TIMEOUT);
 }

@@ -47,26 +47,31 @@ struct Shape {
   int units = 2;       // batched kernel: FE units per warp work item (1 or 2)
 };
 
-// The shared state of the one-CTA-per-FED kernels (ev::Shared): two sets of words,
-// used in turn, each zero when a launch takes it.
+// What the CTAs of a one-CTA-per-FED launch share (ev::Shared).  Every word that a launch
+// reads carries the launch's tag, and every tag has a ticket counter of its own, so that
+// no launch depends on what the one before it left or cleared: 0 marks cleared words,
+// ordinary launches take 1 .. kTags - 2 in turn, launches captured into a graph (whose
+// replays are not seen on the host) the last, and clear the state themselves, ahead.
+// Each kind of launch has a state of its own: an unpacking and a clustering call of one
+// context may overlap on two streams.  Allocated once, so that captured launches keep it.
 struct LookState {
-  unsigned long long* words = nullptr;  // [2 * cap]
-  size_t cap = 0;                       // words of a set
-  size_t used[2] = {0, 0};              // words the last launch on the set may have written, not yet cleared
-  uint32_t next = 0;                    // the next launch's set
-  bool replayed = false;                // a launch was captured into a graph (shared_state)
-  // a ticket, two words of 32 bits per event, a count per (event, FED) and three sums per 1024 of them
-  static constexpr size_t words_for(size_t events, size_t feds) {
-    return 1 + events + events * feds + 3 * (events * feds / 1024 + 1);
+  static constexpr uint32_t kTags = 1024;
+  unsigned long long* words = nullptr;
+  size_t events = 0, items = 0;  // most events, and FED records over all of them
+  uint32_t launches = 1;         // counts ordinary launches (atomically); the first finds cleared words
+  // tickets, a count per FED record, four sums per 1024 of them, a word of 32 bits per event and per record
+  static constexpr size_t words_for(size_t events, size_t items) {
+    return kTags / 2 + items + 4 * (items / 1024 + 1) + (events + 1) / 2 + (items + 1) / 2;
   }
 };
+constexpr uint32_t kEventRecordsMost = 850;  // FED records of a batch that k_event takes: fewer than this
 
 // Device scratch for one stream of work, owned by a context (or by one server
 // stream): the state shared by the CTAs of the one-CTA-per-FED kernels, work tickets,
 // and the many-event kernel's FED offsets, cluster bookkeeping and staging buffer.
 struct Scratch {
-  LookState look;                       // k_event's
-  LookState look_unpack, look_cluster;  // the per-event calls', which may overlap on two streams (contexts only)
+  LookState look_unpack, look_cluster;  // the per-event calls' (contexts only)
+  LookState look_event;                 // k_event's
   uint64_t* fed_off = nullptr;       // absolute byte offset per (event, FED)
   uint32_t* fed_cnt = nullptr;       // clusters found per segment (event, FE unit or half of one)
   uint32_t* fed_start = nullptr;     // staging offset per segment, within its event's slice
@@ -164,8 +169,8 @@ sst_status set_err(sst_ctx* c, sst_status code, const std::string& msg);
 sst_status cuda_err(sst_ctx* c, cudaError_t e, const char* where);
 KParams kparams(const sst_ctx* c);
 cudaError_t ensure_scratch(Scratch& s, size_t items, size_t events, size_t stage_records);
-// Two cleared sets of shared state for `events` events of `feds` FEDs in all; grows only.
-cudaError_t ensure_look(LookState& l, size_t events, size_t feds);
+// Memory for launches of up to `events` events of `items` FED records in all, once.
+cudaError_t ensure_look(LookState& l, size_t events, size_t items);
 // Candidate lists for `warps` warps of k_stream; grows only.
 cudaError_t ensure_spill(Scratch& s, size_t warps);
 // What k_stream needs for amplitudes beside the above (after ensure_scratch and

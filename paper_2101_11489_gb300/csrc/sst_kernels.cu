@@ -592,14 +592,16 @@ __global__ void __launch_bounds__(ev::kThreads) k_unpack(const uint8_t* __restri
   const uint32_t total = staged ? ev::parse_record<true>(s, src, len, f, ok) : ev::parse_record<false>(s, src, len, f, ok);
   ev::Counts own;
   own.digis = total;
-  if (tid == 0) ev::publish(sh, f, 0, own, s.scal[ev::kFlags], s.scal[ev::kBad]);
+  own.flags = s.scal[ev::kFlags];
+  own.bad = s.scal[ev::kBad];
+  if (tid == 0) ev::publish(sh, f, own);
   const bool single = total <= (uint32_t)TILE;
   if (single) {  // while the FEDs before this one publish
     if (staged) ev::emit_slots(s, len);
     else ev::emit_channels(s, src, 0, kCh, lanes);
   }
-  const uint64_t base =
-      ev::look_back<false>(s, sh, f, 0, own, (f & (ev::kLbBlock - 1u)) == ev::kLbBlock - 1u, &timed_out).digis;
+  const ev::Counts before = ev::look_back<false>(s, sh, f, 0, f == sh.n_feds - 1 ? 0u : ev::kNoStatus, own, &timed_out);
+  const uint64_t base = before.digis;
   const uint64_t cap = out.capacity;
   for (int c = tid; c <= kCh; c += ev::kThreads) {
     if (c == kCh && f != sh.n_feds - 1) continue;
@@ -627,8 +629,10 @@ __global__ void __launch_bounds__(ev::kThreads) k_unpack(const uint8_t* __restri
     const uint64_t all = base + total;
     out.status->n_digi = (uint32_t)(all < cap ? all : cap);
     out.status->n_clusters = 0;
-    out.status->n_bad_channels = __ldcg(sh.acc + 1);
-    ev::write_flags(sh, 0, (size_ok ? 0u : SST_EV_SIZE) | (all > cap ? SST_EV_DIGI_CAPACITY : 0u), out.status);
+    out.status->n_bad_channels = before.bad + own.bad;
+    ev::write_flags(sh, 0,
+                    before.flags | own.flags | (size_ok ? 0u : SST_EV_SIZE) | (all > cap ? SST_EV_DIGI_CAPACITY : 0u),
+                    out.status);
   }
 }
 
@@ -716,8 +720,8 @@ __global__ void __launch_bounds__(ev::kThreads) k_cluster(sst_digis in, KParams 
         ev::Counts own;
         own.clusters = n;
         own.amps = a;
-        if (tid == 0) ev::publish(sh, f, 0, own, 0, 0);
-        return before = ev::look_back<AMP>(s, sh, f, 0, own, (f & (ev::kLbBlock - 1u)) == ev::kLbBlock - 1u, &timed_out);
+        if (tid == 0) ev::publish(sh, f, own);
+        return before = ev::look_back<AMP>(s, sh, f, 0, ev::kNoStatus, own, &timed_out);
       },
       o, out, fed_spill(kp), &amps);
   if (tid != 0) return;
@@ -802,12 +806,14 @@ __global__ void __launch_bounds__(ev::kThreads) k_event(const uint8_t* __restric
         own.clusters = n;
         own.digis = total;
         own.amps = a;
-        if (tid == 0) ev::publish(sh, idx, e, own, s.scal[ev::kFlags], s.scal[ev::kBad]);
-        before = ev::look_back<AMP>(s, sh, idx, from, own, (idx & (ev::kLbBlock - 1u)) == ev::kLbBlock - 1u, &timed_out);
+        own.flags = s.scal[ev::kFlags];
+        own.bad = s.scal[ev::kBad];
+        if (tid == 0) ev::publish(sh, idx, own);
+        before = ev::look_back<AMP>(s, sh, idx, from, f == n_feds - 1 ? lo : ev::kNoStatus, own, &timed_out);
         // the clusters, digis and amplitudes before the event's first, which `before` includes
         if (pack_off && e > 0 && (AMP || f == n_feds - 1)) {
           bool to;
-          const ev::Counts start = ev::look_back<AMP>(s, sh, lo, 0, ev::Counts{}, false, &to);
+          const ev::Counts start = ev::look_back<AMP>(s, sh, lo, 0, ev::kNoStatus, ev::Counts{}, &to);
           before.digis -= start.digis;
           before.amps -= start.amps;
           first = start.clusters;
@@ -826,9 +832,9 @@ __global__ void __launch_bounds__(ev::kThreads) k_event(const uint8_t* __restric
     sst_event_status* st = status + e;
     st->n_digi = (uint32_t)(before.digis + total);
     st->n_clusters = (uint32_t)(place(all) - place(first));
-    st->n_bad_channels = __ldcg(sh.acc + 2 * (size_t)e + 1);
+    st->n_bad_channels = before.bad + s.scal[ev::kBad];
     ev::write_flags(sh, e,
-                    (size_ok ? 0u : SST_EV_SIZE) | (all > o.room ? SST_EV_CLUSTER_CAPACITY : 0u) |
+                    before.flags | s.scal[ev::kFlags] | (size_ok ? 0u : SST_EV_SIZE) | (all > o.room ? SST_EV_CLUSTER_CAPACITY : 0u) |
                         (AMP && before.amps + amps > o.a_room ? SST_EV_AMP_CAPACITY : 0u),
                     st);
   }
@@ -1029,33 +1035,37 @@ cs::Amps amp_args(const sst_clusters& out, const Scratch& s) {
   return a;
 }
 
-// The shared state of a launch of one CTA per FED of n_events events: one of the two
-// sets of l in turn, cleared by the launch before (which had the other).  A launch
-// that a graph may replay has the same set every time, and the replays are not seen
-// here: from the first capture on, every launch clears its set itself, ahead.
+// The shared state of a launch of one CTA per FED of n_events events, under the next tag
+// of l (the last for a launch that a graph may replay).  The state is cleared before a
+// captured launch and when half of the tags have gone round: a word keeps its tag at most
+// that long, and work that wrongly overlapped a clearing is cleared away by the next one
+// before its tag is due again.
 cudaError_t shared_state(LookState& l, uint32_t n_events, uint32_t n_feds, uint32_t spin_limit, cudaStream_t st,
                          ev::Shared* sh) {
-  const size_t words = LookState::words_for(n_events, n_feds);
-  if (words > l.cap) return cudaErrorInvalidValue;
+  const size_t items = (size_t)n_events * n_feds;
+  if (!l.words || n_events > l.events || items > l.items) return cudaErrorInvalidValue;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaError_t e = cudaStreamIsCapturing(st, &cs);
   if (e) return e;
-  if (cs != cudaStreamCaptureStatusNone) l.replayed = true;
-  unsigned long long* set = l.words + l.next * l.cap;
-  unsigned long long* other = l.words + (l.next ^ 1u) * l.cap;
-  if (l.replayed && (e = cudaMemsetAsync(set, 0, words * sizeof(*set), st))) return e;
-  sh->ticket = reinterpret_cast<uint32_t*>(set);
-  sh->acc = reinterpret_cast<uint32_t*>(set + 1);
-  sh->lb = set + 1 + (size_t)n_events;
-  sh->clear = other;
-  sh->n_clear = (uint32_t)l.used[l.next ^ 1u];
-  sh->n_items = n_events * n_feds;
+  constexpr uint32_t kTurn = LookState::kTags - 2;
+  uint32_t tag = LookState::kTags - 1;
+  bool clear = true;
+  if (cs == cudaStreamCaptureStatusNone) {
+    const uint32_t n = __atomic_fetch_add(&l.launches, 1u, __ATOMIC_RELAXED) % kTurn;  // (0 when the count wraps, too)
+    tag = n + 1;
+    clear = n % (kTurn / 2) == 0;
+  }
+  if (clear && (e = cudaMemsetAsync(l.words, 0, LookState::words_for(l.events, l.items) * sizeof(*l.words), st))) return e;
+  sh->ticket = reinterpret_cast<uint32_t*>(l.words) + tag;
+  sh->lb = l.words + LookState::kTags / 2;
+  sh->pre = sh->lb + l.items;
+  sh->late = reinterpret_cast<uint32_t*>(sh->pre + 4 * (l.items / 1024 + 1));
+  sh->st = sh->late + (l.events + 1) / 2 * 2;
+  sh->n_items = (uint32_t)items;
   sh->n_feds = n_feds;
+  sh->tag = tag;
   sh->spin_limit = spin_limit ? spin_limit : kLbSpinLimit;
   sh->withhold = -1;
-  l.used[l.next] = words;
-  l.used[l.next ^ 1u] = 0;
-  l.next ^= 1u;
   return cudaSuccess;
 }
 
@@ -1068,10 +1078,7 @@ cudaError_t launch_feds(const void* fn, size_t smem, LookState& l, uint32_t n_ev
   ev::Shared sh;
   cudaError_t e = prepare(fn, ev::kThreads, smem, &per_sm);
   if (!e) e = shared_state(l, n_events, n_feds, spin_limit, st, &sh);
-  if (e) return e;
-  e = bind(sh);
-  if (e) l.replayed = true;  // the other set was not cleared
-  return e;
+  return e ? e : bind(sh);
 }
 
 template <int TILE>
@@ -1091,7 +1098,7 @@ cudaError_t launch_event(const uint8_t* raw, const uint64_t* event_off, const ui
                          cudaStream_t st, uint64_t* pack_off) {
   const size_t sm = sizeof(ev::Shm<kEvTile, true>);
   auto* k = out.amp ? k_event<true> : k_event<false>;
-  return launch_feds((const void*)k, sm, s.look, n_events, n_feds, s.lb_spin_limit, st, [&](ev::Shared& sh) {
+  return launch_feds((const void*)k, sm, s.look_event, n_events, n_feds, s.lb_spin_limit, st, [&](ev::Shared& sh) {
     return launch_pdl(k, n_events * n_feds, (unsigned)ev::kThreads, sm, st, raw, event_off, event_end, fed_len,
                       n_events, clu_off, out, status, with_spill(kp, s), pack_off, sh);
   });
@@ -1109,6 +1116,10 @@ cudaError_t launch_event(const uint8_t* raw, const uint64_t* event_off, const ui
 //   k_stream_fed 59; 120 x 13 43 and 45; 100 x 12 40 and 36; 440 x 8 103 and 86), or of
 //   16 events, or 3,600 records.
 constexpr uint32_t kEventRecords = 100, kEventRecordsOneFed = 240, kEventRecordsWide = 700, kEventRecordsAmps = 850;
+static_assert(kEventRecords <= kEventRecordsMost && kEventRecordsOneFed <= kEventRecordsMost &&
+                  kEventRecordsWide <= kEventRecordsMost && kEventRecordsAmps <= kEventRecordsMost &&
+                  kEventRecordsMost <= ev::kLbBlock,
+              "k_event's shared state has room for the records it takes, in one look-back block");
 constexpr uint32_t kTileEvents = 10, kTileEventsFew = 16, kTileRecordsFew = 1500, kTileRecords = 3600;
 constexpr uint32_t kTileChunk = 32, kTileChunkMin = 8;
 

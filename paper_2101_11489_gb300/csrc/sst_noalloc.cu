@@ -20,21 +20,22 @@ namespace {
 constexpr uint32_t kMaxFeds = SST_NOALLOC_MAX_FEDS;
 constexpr int kMaxDevices = 64;
 
-// The launches' shared state: two sets (sst::LookState), about 16 KiB.
-constexpr size_t kWords = sst::LookState::words_for(1, kMaxFeds);
-static __device__ __align__(256) unsigned long long g_scratch[2 * kWords];
+// The launches' shared state (sst::LookState), about 16 KiB.
+static __device__ __align__(256) unsigned long long g_scratch[sst::LookState::words_for(1, kMaxFeds)];
 
-std::mutex g_mu;
+std::mutex g_mu;                    // held while a device's address is looked up
 sst::Scratch g_state[kMaxDevices];  // per device; look_unpack.words is g_scratch's address there, once known
 
 // Finds g_scratch's address on the current device (on the first call for that device).
 cudaError_t find_scratch(sst::LookState& l) {
+  std::lock_guard<std::mutex> lock(g_mu);
   if (l.words) return cudaSuccess;
   void* p = nullptr;
   const cudaError_t e = cudaGetSymbolAddress(&p, g_scratch);
   if (e != cudaSuccess) return e;
   l.words = static_cast<unsigned long long*>(p);
-  l.cap = kWords;
+  l.events = 1;
+  l.items = kMaxFeds;
   return cudaSuccess;
 }
 
@@ -49,7 +50,6 @@ extern "C" sst_status sst_unpack_noalloc(const uint8_t* raw, uint64_t raw_bytes,
   if (n_feds > kMaxFeds) return SST_ERR_TOO_LARGE;
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return SST_ERR_CUDA;
-  std::lock_guard<std::mutex> lock(g_mu);
   sst::Scratch& s = g_state[dev];
   if (find_scratch(s.look_unpack) != cudaSuccess) return SST_ERR_CUDA;
   const cudaError_t e = sst::launch_unpack(raw, raw_bytes, fed_len, n_feds, *out, s, sst::default_shape(),

@@ -1,6 +1,7 @@
 """The state that the CTAs of a one-CTA-per-FED launch share, against the oracle where it
 can go wrong: the unpacking of one event beside the clustering of the one before on another
-stream.
+stream, more launches than the state has tags, and captured launches replayed after the
+context has grown.
 """
 import numpy as np
 import pytest
@@ -16,6 +17,7 @@ import paper_2101_11489_gb300 as sst  # noqa: E402
 from _gpu_util import Gpu, assert_clusters_equal, assert_digis_equal  # noqa: E402
 
 N_FEDS = 60
+LAUNCHES = 2100  # twice round the 1,022 tags
 
 
 def device(e):
@@ -59,3 +61,73 @@ def test_unpacking_beside_clustering(gt, amps):
         assert dh["flags"] == ost["flags"] and dh["n_clusters"] == ost["n_clusters"]
         assert_digis_equal(dh, od)
         assert_clusters_equal(c[i].to_host(0, dh["n_clusters"]), oc)
+
+
+@pytest.mark.parametrize("call", ["unpack", "noalloc", "batch"])
+def test_more_launches_than_tags(gt, call):
+    w, calib, g = gt
+    sizes = (N_FEDS, 7, 33)
+    evs = [eg.make_event(w, calib, 20 + k, n_feds=n) for k, n in enumerate(sizes)]
+    dev = [device(e) for e in evs]
+    bad = torch.zeros((), dtype=torch.int64, device="cuda")
+    outs = []
+    for e, n, (raw, fl) in zip(evs, sizes, dev):
+        od, oc, ost = g.oracle(e.raw, e.fed_len, n)
+        if call == "batch":
+            c = sst.ClusterBuffers.alloc(e.nbytes // 2 + 1)
+            st = torch.zeros(4, dtype=torch.int32, device="cuda")
+            off = torch.tensor([0, e.nbytes], dtype=torch.int64, device="cuda")
+            room = torch.tensor([0, e.nbytes // 2 + 1], dtype=torch.int64, device="cuda")
+            status = torch.tensor([ost[k] for k in ("n_digi", "n_clusters", "flags", "n_bad_channels")],
+                                  dtype=torch.int32, device="cuda")
+            crec = c.record()
+            outs.append((lambda raw=raw, fl=fl, n=n, st=st, off=off, room=room, crec=crec:
+                         sst.sst_batch(g.ctx, raw, off, fl, 1, n, room, crec, st),
+                         [(c.det, oc["det"].astype(np.int32)), (c.charge, oc["charge"].astype(np.int32)),
+                          (st, status.cpu().numpy())], c))
+        else:
+            d = sst.DigiBuffers.alloc(e.nbytes, n)
+            drec = d.record()
+            f = ((lambda raw=raw, fl=fl, n=n, drec=drec: sst.sst_unpack(g.ctx, raw, fl, n, drec)) if call == "unpack" else
+                 (lambda raw=raw, fl=fl, n=n, drec=drec: sst.sst_unpack_noalloc(raw, fl, n, drec)))
+            outs.append((f, [(d.strip, od["strip"].astype(np.int32)), (d.adc, od["adc"]),
+                             (d.chan_off, od["chan_off"].astype(np.int32))], d))
+    outs = [(f, [(t.view(torch.int32) if t.dtype == torch.uint32 else t, torch.from_numpy(np.ascontiguousarray(v)).cuda())
+                 for t, v in pairs], keep) for f, pairs, keep in outs]
+    for i in range(LAUNCHES):
+        f, pairs, _ = outs[(i * i + i // 3) % 3]
+        f()
+        for t, v in pairs:
+            bad += (t[:v.numel()] != v).sum()
+            t[:v.numel()] = -1 if t.dtype != torch.uint8 else 255
+    torch.cuda.synchronize()
+    assert int(bad) == 0
+
+
+def test_replays_after_the_context_has_grown(gt):
+    w, calib, g = gt
+    e = eg.make_event(w, calib, 31, n_feds=N_FEDS)
+    od, oc, _ = g.oracle(e.raw, e.fed_len, N_FEDS)
+    raw, fl = device(e)
+    d, c = sst.DigiBuffers.alloc(e.nbytes, N_FEDS), sst.ClusterBuffers.alloc(e.nbytes // 2 + 1)
+    drec, crec = d.record(), c.record()
+
+    def launch():
+        sst.sst_unpack(g.ctx, raw, fl, N_FEDS, drec)
+        sst.sst_cluster(g.ctx, drec, N_FEDS, crec)
+
+    launch()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        launch()
+    for n in (2, 9, 40):  # batches that grow the context's scratch
+        for st, cl in g.batch([(e.raw, e.fed_len)] * n):
+            assert_clusters_equal(cl, oc)
+        for t in (d.strip, c.det):
+            t.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        dh = d.to_host()
+        assert_digis_equal(dh, od)
+        assert_clusters_equal(c.to_host(0, dh["n_clusters"]), oc)
