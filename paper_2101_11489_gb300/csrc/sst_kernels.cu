@@ -4,9 +4,9 @@
 //
 // Batches (k_stream, sst_stream.cuh): one lane per channel record, the calibration
 // entries of one FE unit in shared memory while all events' records of it pass; where
-// the events are too few for that, each warp reads them from global memory
-// (k_stream_fed).  The FED headers are checked by a prologue (k_fed_scan), which hands every FE
-// unit its byte range; the kept clusters are staged per FE unit and event and put in
+// the events are too few for that, or their records are read in place from host memory,
+// each warp reads them from global memory (k_stream_fed).  The FED headers are checked by
+// a prologue (k_fed_scan), which hands every FE unit its byte range; the kept clusters are staged per FE unit and event and put in
 // order by k_order.  Placing them with a look-back over the units before instead
 // would make every warp wait for units that other CTAs take at the same time.
 //
@@ -323,12 +323,14 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_stream(const uint8_t* __rest
 // memory, digi by digi.  The tile of k_stream would cost more than these gathers (24 KB
 // against about 4 KB per FE unit and event), and its warps would each have only a few
 // channels.  FED-major order, so that the warps at work read the same FEDs' entries.
+// LINK: the records are read in place from host memory; else the bytes of a warp's next
+// item are fetched to L2 while it works.
 constexpr int kFedWarps = 8;
 struct FedWarp {
   cs::WarpT<2> w;
   int2 mul[kCh];  // the units' APV multipliers
 };
-template <bool AMP>
+template <bool AMP, bool LINK>
 __global__ void __launch_bounds__(kFedWarps * 32, 3) k_stream_fed(
     const uint8_t* __restrict__ raw, const uint64_t* __restrict__ fed_off, uint32_t n_events, uint32_t n_feds,
     const uint64_t* __restrict__ clu_off, uint64_t out_cap, sst_event_status* status, KParams kp, uint2* stage,
@@ -370,11 +372,13 @@ __global__ void __launch_bounds__(kFedWarps * 32, 3) k_stream_fed(
     div = __any_sync(0xffffffffu, div);
     next = __shfl_sync(0xffffffffu, next, 0);
     const cs::SlotSrc src2 = src_of(next);
-    const cs::Channels<kChPerFe, true> chans{kp.calq + (size_t)ch0 * kStrips, w.mul, ch0};
+    const cs::Channels<kChPerFe, true, LINK> chans{kp.calq + (size_t)ch0 * kStrips, w.mul, ch0};
     cs::process_slots<AMP, kChPerFe>(w.w, (int)units, 0, src, e,
                                      ((size_t)e * n_feds + f) * kFe + u + (lane < (int)units ? lane : 0), kp, clu_off,
                                      out_cap, status, stage, ev_alloc, seg_cnt, seg_start, spill, chans, div, am,
-                                     amp_spill, [&] { prefetch_slots(src2); });
+                                     amp_spill, [&] {
+                                       if (!LINK) prefetch_slots(src2);
+                                     });
     src = src2;
     t = next;
   }
@@ -1115,6 +1119,12 @@ cudaError_t launch_event(const uint8_t* raw, const uint64_t* event_off, const ui
 //   24 and 18); beyond, from 1,500 records of 10 events and more on (200 x 10 54,
 //   k_stream_fed 59; 120 x 13 43 and 45; 100 x 12 40 and 36; 440 x 8 103 and 86), or of
 //   16 events, or 3,600 records.
+// A batch read in place from pinned host memory is bound by the link, which a warp's
+// contiguous piece of four FE units (1.4 KB) loads better than the tiles' single units:
+// 440 FEDs x 16 | 32 | 64 | 128 events 153 | 253 | 448 | 853 us with k_stream_fed, 150 | 267
+// | 500 | 965 with k_stream (two units: 147 | 249 | 450 | 866); served, 87 | 93 | 101 | 104 k
+// events/s against 79 | 80 | 84 | 87 k (two units: 87 | 90 | 98 | 99 k).  Fetching ahead to
+// L2 does not pay there (k_stream without it: 83 | 84 | 88 | 90 k).
 constexpr uint32_t kEventRecords = 100, kEventRecordsOneFed = 240, kEventRecordsWide = 700, kEventRecordsAmps = 850;
 static_assert(kEventRecords <= kEventRecordsMost && kEventRecordsOneFed <= kEventRecordsMost &&
                   kEventRecordsWide <= kEventRecordsMost && kEventRecordsAmps <= kEventRecordsMost &&
@@ -1130,6 +1140,7 @@ struct Plan {
   size_t smem = 0;
   uint32_t segs_per_fed = kFe;     // segments of the staging buffer per FED and event
   uint32_t units = 0;              // kUnits: FE units per warp
+  bool link = false;               // kUnits: the records are read in place from host memory
   uint32_t chunk = 0, per_warp = 0;  // kTiles: events per item, and per warp of it
 };
 
@@ -1160,7 +1171,8 @@ cudaError_t plan_tiles(const Shape& sh, uint32_t n_events, uint32_t n_feds, int 
   return cudaSuccess;
 }
 
-cudaError_t plan_batch(const Shape& sh, uint32_t n_events, uint32_t n_feds, bool amps, int n_sm, Plan* p) {
+cudaError_t plan_batch(const Shape& sh, uint32_t n_events, uint32_t n_feds, bool amps, bool in_place, int n_sm,
+                       Plan* p) {
   const size_t records = (size_t)n_events * n_feds;
   const bool one_wave = (size_t)n_feds * kFe <= (size_t)n_sm * 4;  // the tiles fit the GPU at once
   const bool tiles = one_wave || records > kTileRecords ||
@@ -1174,17 +1186,18 @@ cudaError_t plan_batch(const Shape& sh, uint32_t n_events, uint32_t n_feds, bool
     p->smem = sizeof(ev::Shm<kEvTile, true>);
     return cudaSuccess;
   }
-  if (tiles) {
+  if (tiles && !in_place) {
     p->kind = Plan::kTiles;
     auto* f = sh.block == 128 ? (sh.units == 1 ? plan_tiles<4, 1> : plan_tiles<4, 2>)
                               : (sh.units == 1 ? plan_tiles<8, 1> : plan_tiles<8, 2>);
     return f(sh, n_events, n_feds, n_sm, p);
   }
   p->kind = Plan::kUnits;
+  p->link = in_place;
   p->block = kFedWarps * 32;
   p->smem = kFedWarps * sizeof(FedWarp);
   int per_sm = 0;
-  cudaError_t e = prepare((const void*)k_stream_fed<false>, p->block, p->smem, &per_sm);
+  cudaError_t e = prepare((const void*)k_stream_fed<false, false>, p->block, p->smem, &per_sm);
   if (e) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const size_t per = sh.ctas_per_sm < per_sm ? sh.ctas_per_sm : per_sm, ctas = (size_t)n_sm * per;
@@ -1194,7 +1207,7 @@ cudaError_t plan_batch(const Shape& sh, uint32_t n_events, uint32_t n_feds, bool
   // when the FEDs' densities differ a hundredfold; 440 x 5 77 and 69; 150 x 8 36 and 42
   p->units = 1;
   while (p->units < kFe / 2 && records * (kFe / p->units) > ctas * kFedWarps) p->units *= 2;
-  if (records * 3 > ctas * kFedWarps) p->units = 2;
+  if (records * 3 > ctas * kFedWarps) p->units = in_place ? 4 : 2;
   const size_t need = (records * (kFe / p->units) + kFedWarps - 1) / kFedWarps;
   p->grid = (int)(ctas < need ? ctas : need);
   p->resident = p->grid;
@@ -1226,9 +1239,10 @@ cudaError_t launch_stream(const Plan& p, const Shape& sh, const uint8_t* raw, ui
     return f(p, raw, n_events, n_feds, clu_off, out_cap, status, kps, s, am, st);
   }
   int per_sm = 0;
-  cudaError_t e = prepare((const void*)k_stream_fed<AMP>, p.block, p.smem, &per_sm);
+  auto* k = !AMP && p.link ? k_stream_fed<false, true> : k_stream_fed<AMP, false>;
+  cudaError_t e = prepare((const void*)k, p.block, p.smem, &per_sm);
   if (e) return e;
-  return launch_pdl(k_stream_fed<AMP>, (unsigned)p.grid, (unsigned)p.block, p.smem, st, raw,
+  return launch_pdl(k, (unsigned)p.grid, (unsigned)p.block, p.smem, st, raw,
                     (const uint64_t*)s.fed_off, n_events, n_feds, clu_off, out_cap, status, kps, s.stage, s.ev_alloc,
                     s.fed_cnt, s.fed_start, s.tickets, (const uint2*)s.unit_desc, p.units, am);
 }
@@ -1273,7 +1287,7 @@ cudaError_t batch_launch_info(const Shape& sh, uint32_t n_events, uint32_t n_fed
                               int* block, int* items_per_fed) {
   Plan p;
   const bool amps = false;
-  const cudaError_t e = plan_batch(sh, n_events, n_feds, amps, n_sm, &p);
+  const cudaError_t e = plan_batch(sh, n_events, n_feds, amps, false, n_sm, &p);
   if (e) return e;
   *grid = p.grid;
   *block = p.block;
@@ -1307,7 +1321,7 @@ cudaError_t launch_batch(const uint8_t* raw, const uint64_t* event_off, const ui
                          uint64_t* pack_off, cudaEvent_t ev_begin, cudaEvent_t ev_end, const uint64_t* event_end) {
   Plan p;
   const bool amps = out.amp != nullptr;
-  cudaError_t e = plan_batch(sh, n_events, n_feds, amps, n_sm, &p);
+  cudaError_t e = plan_batch(sh, n_events, n_feds, amps, event_end != nullptr, n_sm, &p);
   if (e) return e;
   if (p.kind == Plan::kFeds) {
     if (ev_begin && (e = cudaEventRecord(ev_begin, st))) return e;
