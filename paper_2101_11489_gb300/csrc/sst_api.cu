@@ -79,7 +79,9 @@ cudaError_t ensure_scratch(Scratch& s, size_t items, size_t events, size_t stage
       if ((e = grow(s.unit_desc, c4, items))) return e;
       s.items_cap = items;
     }
-    if ((e = grow(s.ev_alloc, s.ev_cap, events))) return e;
+    size_t counters = counters_for(s.ev_cap);
+    if ((e = grow(s.ev_alloc, counters, counters_for(events)))) return e;
+    if (events > s.ev_cap) s.ev_cap = events;
     if ((e = grow(s.stage, s.stage_cap, stage_records))) return e;
   }
   return cudaSuccess;
@@ -112,7 +114,9 @@ cudaError_t ensure_amp_scratch(Scratch& s, size_t amp_bytes) {
   s.amp_items_cap = s.items_cap;
   if ((e = grow(s.amp_spill, c3, s.spill_warps * kAmpSpill))) return e;
   s.amp_spill_warps = s.spill_warps;
-  if ((e = grow(s.amp_alloc, s.amp_ev_cap, s.ev_cap))) return e;
+  size_t counters = counters_for(s.amp_ev_cap);
+  if ((e = grow(s.amp_alloc, counters, counters_for(s.ev_cap)))) return e;
+  s.amp_ev_cap = s.ev_cap;
   if ((e = grow(s.stage_amp, s.stage_amp_cap, s.stage_cap))) return e;
   return grow(s.amp_stage, s.amp_stage_cap, amp_bytes);
 }

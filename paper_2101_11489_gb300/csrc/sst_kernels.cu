@@ -173,8 +173,8 @@ __global__ void k_fed_scan(const uint64_t* __restrict__ event_off, const uint64_
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint64_t ev0 = event_off[e], ev1 = event_end ? event_end[e] : event_off[e + 1];
   if (c == 0 && threadIdx.x == 0) {
-    ev_alloc[e] = 0;
-    if (amp_alloc) amp_alloc[e] = 0;
+    ev_alloc[counter_at(e)] = 0;
+    if (amp_alloc) amp_alloc[counter_at(e)] = 0;
   }
   if (e == 0 && c == 0 && threadIdx.x < 2) tickets[threadIdx.x] = 0;
   const uint32_t* len_e = fed_len + (size_t)e * n_feds;

@@ -940,8 +940,8 @@ __device__ void process_slots(W& w, int n, int c0, const SlotSrc& me, uint32_t e
     }
     uint32_t start = 0;
     if (mine) {
-      const uint32_t astart = AMP && strips ? atomicAdd(am.alloc + e, strips) : 0u;
-      start = found ? atomicAdd(ev_alloc + e, found) : 0u;
+      const uint32_t astart = AMP && strips ? atomicAdd(am.alloc + counter_at(e), strips) : 0u;
+      start = found ? atomicAdd(ev_alloc + counter_at(e), found) : 0u;
       const uint32_t fits = start < room ? (found < room - start ? found : room - start) : 0u;
       uint32_t fl = w.slot.flags[lane - done];
       if (fits < found) fl |= SST_EV_CLUSTER_CAPACITY;
