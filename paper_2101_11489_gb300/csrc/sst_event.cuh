@@ -128,16 +128,18 @@ __device__ __forceinline__ uint32_t block_scan(S& s, uint32_t v, uint32_t* total
 // launch's tag.  The statuses, which few FEDs have, are in a word of their own, written
 // before.
 struct Counts {
-  unsigned long long clusters = 0, digis = 0, amps = 0;
-  uint32_t flags = 0, bad = 0;  // OR of the channel statuses, bad channels
+  uint32_t clusters = 0, digis = 0;  // (sums too: below 2^32 for SST_MAX_FEDS FEDs)
+  uint32_t flags = 0, bad = 0;       // OR of the channel statuses, bad channels
+  unsigned long long amps = 0;
   static constexpr unsigned long long kStatus = 1ull << 53;
   static constexpr int kTagAt = 54;
   __device__ __forceinline__ unsigned long long word(uint32_t tag) const {
-    return ((unsigned long long)tag << kTagAt) | (bad ? kStatus : 0ull) | (amps << 30) | (digis << 15) | clusters;
+    return ((unsigned long long)tag << kTagAt) | (bad ? kStatus : 0ull) | (amps << 30) |
+           ((unsigned long long)digis << 15) | clusters;
   }
   __device__ __forceinline__ void add(unsigned long long w) {
-    clusters += w & 0x7FFFull;
-    digis += (w >> 15) & 0x7FFFull;
+    clusters += (uint32_t)w & 0x7FFFu;
+    digis += (uint32_t)(w >> 15) & 0x7FFFu;
     amps += (w >> 30) & 0x7FFFFFull;
   }
 };
@@ -163,9 +165,9 @@ __device__ __forceinline__ uint32_t block_or(S& s, uint32_t v) {
 // up to kLbBlock items are read at once, a few by each thread, so that a CTA waits for
 // the slowest of them and not for a chain; further back, the last item of every
 // kLbBlock publishes the sums up to and including itself, with its own counts `own`.
-// st_from: the first item whose statuses are wanted (kNoStatus: none).  A wait gives up
-// after spin_limit polls: *timed_out is set and the sums are partial.
-template <bool AMP, class S>
+// STATUS: the items have statuses, wanted from item st_from on (kNoStatus: none).  A wait
+// gives up after spin_limit polls: *timed_out is set and the sums are partial.
+template <bool AMP, bool STATUS, class S>
 __device__ __forceinline__ Counts look_back(S& s, const Shared& sh, uint32_t idx, uint32_t lo, uint32_t st_from,
                                             const Counts& own, bool* timed_out) {
   const uint32_t w0 = idx & ~(kLbBlock - 1u), from = w0 > lo ? w0 : lo;
@@ -190,7 +192,7 @@ __device__ __forceinline__ Counts look_back(S& s, const Shared& sh, uint32_t idx
   for (uint32_t i = from + threadIdx.x; i < idx; i += kThreads) {
     const unsigned long long w = poll(sh.lb + i);
     c.add(w);
-    if ((w & Counts::kStatus) && i >= st_from) {
+    if (STATUS && (w & Counts::kStatus) && i >= st_from) {
       const uint32_t st = __ldcg(sh.st + i);
       c.flags |= st & 255u;
       c.bad += st >> 8;
@@ -198,11 +200,11 @@ __device__ __forceinline__ Counts look_back(S& s, const Shared& sh, uint32_t idx
   }
   if (from > lo && threadIdx.x == 0) {  // the sums up to item from - 1
     const unsigned long long* pre = sh.pre + 4 * (size_t)(from / kLbBlock - 1);
-    c.clusters += poll(pre) & kSums;
+    c.clusters += (uint32_t)(poll(pre) & kSums);
     if (!to) {
-      c.digis += __ldcg(pre + 1);
+      c.digis += (uint32_t)__ldcg(pre + 1);
       c.amps += __ldcg(pre + 2);
-      if (st_from != kNoStatus) {
+      if (STATUS && st_from != kNoStatus) {
         const unsigned long long st = __ldcg(pre + 3);
         c.flags |= (uint32_t)(st >> 32);
         c.bad += (uint32_t)st;
@@ -211,15 +213,15 @@ __device__ __forceinline__ Counts look_back(S& s, const Shared& sh, uint32_t idx
   }
   // clusters and digis in one sum (each below 2^32 within one block of items)
   if (w0 <= lo && !AMP) {
-    const unsigned long long both = block_sum(s, c.clusters | (c.digis << 32));
-    c.clusters = both & 0xFFFFFFFFull;
-    c.digis = both >> 32;
+    const unsigned long long both = block_sum(s, c.clusters | ((unsigned long long)c.digis << 32));
+    c.clusters = (uint32_t)both;
+    c.digis = (uint32_t)(both >> 32);
   } else {
-    c.clusters = block_sum(s, c.clusters);
-    c.digis = block_sum(s, c.digis);
+    c.clusters = (uint32_t)block_sum(s, c.clusters);
+    c.digis = (uint32_t)block_sum(s, c.digis);
     if (AMP) c.amps = block_sum(s, c.amps);
   }
-  if (st_from != kNoStatus && __syncthreads_or(c.bad != 0)) {
+  if (STATUS && st_from != kNoStatus && __syncthreads_or(c.bad != 0)) {
     c.flags = block_or(s, c.flags);
     c.bad = (uint32_t)block_sum(s, c.bad);
   }
