@@ -410,14 +410,15 @@ sst_status sst_profile_enable(sst_ctx* ctx, int enable);
 sst_status sst_profile_read(sst_ctx* ctx, uint64_t* launches, double* total_ms, int reset);
 
 /* ---- failure detection ----------------------------------------------------------
- * The per-event unpacker places each FED's digis after a device-side look-back over
- * the FEDs before it (section 2: the channel map, here built on the device).  Every
- * such wait gives up after a bounded number of polls (about a second by default),
- * flags the event SST_EV_TIMEOUT and lets the kernel finish; the event's output is
- * then invalid, but no access leaves its buffers.  For tests of that path:
- * spin_limit sets the polls (1 .. 2^20; 0 = the default) and withhold_fed >= 0
- * makes the FED of that index never publish its digi count, so that the FEDs after
- * it run out of polls; withhold_fed = -1 restores normal operation.  Nothing faults,
+ * The per-event calls and the smallest batches place each FED's digis or clusters
+ * after a device-side look-back over the FEDs before it (section 2: the channel map,
+ * here built on the device).  Every such wait gives up after a bounded number of
+ * polls (about a second by default), flags the event SST_EV_TIMEOUT and lets the
+ * kernel finish; the event's output is then invalid, but no access leaves its
+ * buffers.  For tests of that path: spin_limit sets the polls (1 .. 2^20; 0 = the
+ * default) and withhold_fed >= 0 makes the FED of that index (of a batch's first
+ * event) never publish its counts, in sst_unpack, sst_cluster and sst_batch, so that
+ * the FEDs after it run out of polls; -1 restores normal operation.  Nothing faults,
  * traps or waits without end.  INVALID_ARG for spin_limit above 2^20 or
  * withhold_fed below -1. */
 sst_status sst_testing_set_wait(sst_ctx* ctx, uint32_t spin_limit, int32_t withhold_fed);

@@ -97,7 +97,7 @@ struct Scratch {
   uint32_t* amp_spill = nullptr;     // per warp that has a spill area, kAmpSpill words
   size_t amp_spill_warps = 0;
   uint32_t lb_spin_limit = 0;        // polls before a look-back wait gives up (0: the default, about a second)
-  int32_t lb_withhold = -1;          // failure tests: the FED that never publishes its count (-1: none)
+  int32_t lb_withhold = -1;          // failure tests: the FED (of a batch's first event) that never publishes its counts (-1: none)
 };
 // Where event e's allocation counter is: up to 1,024 events have a 128-byte line each, so
 // that the warps' additions do not queue at one line of L2, or at two that share a slice.

@@ -1045,7 +1045,7 @@ cs::Amps amp_args(const sst_clusters& out, const Scratch& s) {
 // captured launch and when half of the tags have gone round: a word keeps its tag at most
 // that long, and work that wrongly overlapped a clearing is cleared away by the next one
 // before its tag is due again.
-cudaError_t shared_state(LookState& l, uint32_t n_events, uint32_t n_feds, uint32_t spin_limit, cudaStream_t st,
+cudaError_t shared_state(const Scratch& s, LookState& l, uint32_t n_events, uint32_t n_feds, cudaStream_t st,
                          ev::Shared* sh) {
   const size_t items = (size_t)n_events * n_feds;
   if (!l.words || n_events > l.events || items > l.items) return cudaErrorInvalidValue;
@@ -1069,20 +1069,20 @@ cudaError_t shared_state(LookState& l, uint32_t n_events, uint32_t n_feds, uint3
   sh->n_items = (uint32_t)items;
   sh->n_feds = n_feds;
   sh->tag = tag;
-  sh->spin_limit = spin_limit ? spin_limit : kLbSpinLimit;
-  sh->withhold = -1;
+  sh->spin_limit = s.lb_spin_limit ? s.lb_spin_limit : kLbSpinLimit;
+  sh->withhold = s.lb_withhold;
   return cudaSuccess;
 }
 
 // Launches kernel k of n_events x n_feds CTAs with the shared state as its last or, in
 // k_unpack, last but one argument (bind makes the call).
 template <typename Bind>
-cudaError_t launch_feds(const void* fn, size_t smem, LookState& l, uint32_t n_events, uint32_t n_feds,
-                        uint32_t spin_limit, cudaStream_t st, Bind bind) {
+cudaError_t launch_feds(const void* fn, size_t smem, const Scratch& s, LookState& l, uint32_t n_events,
+                        uint32_t n_feds, cudaStream_t st, Bind bind) {
   int per_sm = 0;
   ev::Shared sh;
   cudaError_t e = prepare(fn, ev::kThreads, smem, &per_sm);
-  if (!e) e = shared_state(l, n_events, n_feds, spin_limit, st, &sh);
+  if (!e) e = shared_state(s, l, n_events, n_feds, st, &sh);
   return e ? e : bind(sh);
 }
 
@@ -1090,8 +1090,7 @@ template <int TILE>
 cudaError_t launch_unpack_t(const uint8_t* raw, uint64_t raw_bytes, const uint32_t* fed_len, uint32_t n_feds,
                             const sst_digis& out, Scratch& s, const Shape& shape, cudaStream_t st) {
   const size_t sm = sizeof(ev::Shm<TILE, false>);
-  return launch_feds((const void*)k_unpack<TILE>, sm, s.look_unpack, 1, n_feds, s.lb_spin_limit, st, [&](ev::Shared& sh) {
-    sh.withhold = s.lb_withhold;
+  return launch_feds((const void*)k_unpack<TILE>, sm, s, s.look_unpack, 1, n_feds, st, [&](ev::Shared& sh) {
     return launch_pdl(k_unpack<TILE>, n_feds, (unsigned)ev::kThreads, sm, st, raw, raw_bytes, fed_len, out, sh,
                       shape.lanes);
   });
@@ -1103,7 +1102,7 @@ cudaError_t launch_event(const uint8_t* raw, const uint64_t* event_off, const ui
                          cudaStream_t st, uint64_t* pack_off) {
   const size_t sm = sizeof(ev::Shm<kEvTile, true>);
   auto* k = out.amp ? k_event<true> : k_event<false>;
-  return launch_feds((const void*)k, sm, s.look_event, n_events, n_feds, s.lb_spin_limit, st, [&](ev::Shared& sh) {
+  return launch_feds((const void*)k, sm, s, s.look_event, n_events, n_feds, st, [&](ev::Shared& sh) {
     return launch_pdl(k, n_events * n_feds, (unsigned)ev::kThreads, sm, st, raw, event_off, event_end, fed_len,
                       n_events, clu_off, out, status, with_spill(kp, s), pack_off, sh);
   });
@@ -1311,7 +1310,7 @@ cudaError_t launch_cluster(const sst_digis& in, uint32_t n_feds, const sst_clust
                            Scratch& s, cudaStream_t st) {
   const size_t sm = sizeof(ev::Shm<kEvTile, true>);
   auto* k = out.amp ? k_cluster<true> : k_cluster<false>;
-  return launch_feds((const void*)k, sm, s.look_cluster, 1, n_feds, s.lb_spin_limit, st, [&](ev::Shared& sh) {
+  return launch_feds((const void*)k, sm, s, s.look_cluster, 1, n_feds, st, [&](ev::Shared& sh) {
     return launch_pdl(k, n_feds, (unsigned)ev::kThreads, sm, st, in, with_spill(kp, s), out, sh);
   });
 }
