@@ -19,7 +19,7 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kFedBuf = 8192;      // bytes of FED record staged on chip (larger ones are read in place)
 constexpr int kRunSlots = (kFedBuf + 2) / 3;  // a run header takes at least 3 bytes with its ADC
-constexpr uint32_t kFedClusters = kCh * kStrips / 2;  // most clusters of a FED
+constexpr uint32_t kFedClusters = kCh * kStrips / 2;  // most clusters of a FED whose strips ascend
 constexpr uint32_t kLbBlock = 1024;  // FEDs whose counts a CTA sums one by one
 constexpr uint32_t kNoStatus = 0xFFFFFFFFu;
 static_assert(kLbBlock == 1024 && LookState::kTags == 1024, "sizes of the shared state (LookState)");
@@ -655,8 +655,9 @@ __device__ __forceinline__ int lanes_for(int n) {
 // Clusters one FED whose `total` digis load(c0, c1) brings into the tile, classified,
 // chunk by chunk, and writes its clusters in order.  A FED of more than one chunk leaves
 // its clusters in `spill` (kFedClusters of them) until it knows their place; with
-// amplitudes, or without a spill area, it goes through the chunks again (17 events of 13
-// FEDs of very different density, from host memory: 863 us twice, 406 once).
+// amplitudes, without a spill area, or with more clusters (digis given in no order may
+// each be one), it goes through the chunks again (17 events of 13 FEDs of very different
+// density, from host memory: 863 us twice, 406 once).
 // place(found, amps) publishes the counts and returns those of the FEDs before.  Returns
 // the clusters found; *amps_found their strips.
 template <bool AMP, int TILE, class S, typename Load, typename Place>
@@ -677,7 +678,7 @@ __device__ __forceinline__ uint32_t cluster_fed(S& s, const KParams& kp, uint32_
     const int c1 = single ? kCh : chunk_end<TILE>(s, c0);
     chunk(c0, c1);
     if (!AMP && !single && spill)
-      for (uint32_t r = threadIdx.x; r < in_tile; r += kThreads) {
+      for (uint32_t r = threadIdx.x; r < in_tile && found + r < kFedClusters; r += kThreads) {
         int lo, hi;
         uint32_t c;
         const uint32_t i = s.list[r];
@@ -704,7 +705,7 @@ __device__ __forceinline__ uint32_t cluster_fed(S& s, const KParams& kp, uint32_
   const unsigned long long n0 = before.clusters, a0 = before.amps;
   const bool amp_fits = !AMP || a0 + amps <= o.a_room;
   *amps_found = amps;
-  if (!AMP && !single && spill) {
+  if (!AMP && !single && spill && found <= kFedClusters) {
     for (uint32_t r = threadIdx.x; r < found && n0 + r < o.room; r += kThreads) {
       const uint2 v = spill[r];
       const uint32_t lo = v.x & 255u, wd = ((v.x >> 8) & 255u) + 1u, q = v.x >> 16;
