@@ -63,7 +63,6 @@ struct __align__(16) Shm {
   __device__ __forceinline__ uint32_t* slots() { return reinterpret_cast<uint32_t*>(region + kFedBuf); }
 };
 constexpr uint32_t kSeed = 1u << 31;
-constexpr uint32_t kNoChannel = 0x7FFFu;  // key of a digi that takes no part
 enum { kIdx = 0, kFlags, kBad };  // scal
 
 // The item this CTA takes, in ticket order: every item before it has then started, so

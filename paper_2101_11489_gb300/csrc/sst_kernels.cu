@@ -680,6 +680,13 @@ __global__ void __launch_bounds__(ev::kThreads, 4) k_cluster(sst_digis in, KPara
   whole = __syncthreads_and(whole);
   const uint32_t g0 = f * (uint32_t)kFedStrips;
   const uint2* cal0 = kp.calq + g0;
+  // the channel whose range holds digi i of the FED
+  auto channel_of = [&](uint32_t i) {
+    uint32_t c = 0;
+    for (uint32_t step = 64; step > 0; step >>= 1)
+      if (c + step < (uint32_t)kCh && s.chan_cnt[c + step] <= i) c += step;
+    return c;
+  };
   auto load = [&](int c0, int c1) {
     const uint32_t base = s.chan_cnt[c0], n = s.chan_cnt[c1] - base;
     constexpr int kU = 4;  // digis in flight per thread
@@ -690,16 +697,17 @@ __global__ void __launch_bounds__(ev::kThreads, 4) k_cluster(sst_digis in, KPara
 #pragma unroll
       for (int u = 0; u < kU; u++) {
         const uint32_t i = i0 + u * ev::kThreads;
-        key[u] = i < n ? __ldg(in.strip + a + i) - g0 : ev::kNoChannel;
+        key[u] = i < n ? __ldg(in.strip + a + i) - g0 : 0xFFFFFFFFu;
         adc[u] = i < n ? __ldg(in.adc + a + i) : 0u;
       }
 #pragma unroll
       for (int u = 0; u < kU; u++) {
         const uint32_t i = base + i0 + u * ev::kThreads, c = key[u] >> 8;
         v[u] = make_uint2(ev::kNeverActive, 0u);
-        // a digi that does not belong to the channel whose range it is in takes no part
+        // a digi that does not belong to the channel whose range it is in takes no part: it
+        // is an inactive digi there
         if (c < (uint32_t)kCh && i >= s.chan_cnt[c] && i < s.chan_cnt[c + 1]) v[u] = __ldg(cal0 + key[u]);
-        else key[u] = ev::kNoChannel;
+        else if (i0 + u * ev::kThreads < n) key[u] = channel_of(i) << 8;
       }
 #pragma unroll
       for (int u = 0; u < kU; u++)
@@ -710,7 +718,7 @@ __global__ void __launch_bounds__(ev::kThreads, 4) k_cluster(sst_digis in, KPara
         const size_t a = (size_t)s.chan_pos[tid] + k;
         const uint32_t key = in.strip[a] - g0;
         const bool mine = (key >> 8) == (uint32_t)tid;
-        ev::classify(s, s.chan_cnt[tid] - base + k, mine ? key : ev::kNoChannel, in.adc[a],
+        ev::classify(s, s.chan_cnt[tid] - base + k, mine ? key : (uint32_t)tid << 8, in.adc[a],
                      mine ? cal0[key] : make_uint2(ev::kNeverActive, 0u));
       }
     __syncthreads();

@@ -1,6 +1,7 @@
 """sst_cluster on digis that sst_unpack does not write: repeated and descending strips (each
 active digi is then its own candidate, up to 256 in a channel), in a FED of many digi
-chunks between two ordinary ones.
+chunks between two ordinary ones; and digis of other channels within a channel's range,
+which take no part.
 """
 import numpy as np
 import pytest
@@ -78,3 +79,20 @@ def test_strips_out_of_order_stay_in_their_fed(g, order, per_channel, amps):
     assert mine.sum() == CH * per_channel  # each digi on its own
     assert np.array_equal(got["det"][mine], CH + np.arange(CH).repeat(per_channel))
     assert np.array_equal(got["first"][mine], np.tile(one, CH)) and np.all(got["width"][mine] == 1)
+
+
+@pytest.mark.parametrize("amps", [False, True])
+@pytest.mark.parametrize("occ", [0.01, 0.3])
+def test_digis_of_other_channels_take_no_part(g, occ, amps):
+    """Strays anywhere in a channel's range, between linked strips too, change nothing."""
+    strip, adc, off = ordinary(5, 4, occ)
+    want = orc.cluster_event({"strip": strip, "adc": adc, "chan_off": off}, 4, g.noise, g.gain, g.bad, orc_params(g.params))
+    rng = np.random.default_rng(6)
+    at = np.sort(rng.integers(0, strip.size + 1, strip.size // 3))
+    chan = np.searchsorted(off, np.minimum(at, strip.size - 1), side="right") - 1  # whose range each stray is in
+    other = (chan + rng.choice([-1, 1, 7, 300, -200], at.size)) % 400  # (past the last channel too)
+    other = np.where(other == chan, chan + 1, other)
+    out_s, out_a = np.insert(strip, at, other * 256 + rng.integers(0, 256, at.size)), np.insert(adc, at, 253)
+    n = np.diff(off) + np.bincount(chan, minlength=off.size - 1)
+    got, _ = cluster(g, out_s, out_a, np.concatenate([[0], np.cumsum(n)]), amps)
+    assert_clusters_equal({k: v for k, v in got.items() if k != "amp_first"}, want)
