@@ -165,10 +165,11 @@ typedef struct {
    * gain-corrected charge when the strip is active, else 0 (a hole, a bad strip
    * inside, a bad strip the cluster was widened over): cluster k's width[k]
    * amplitudes are amp[amp_first[k] ..].  Within an event they follow the
-   * cluster order.  Amplitudes are allocated per work item (one FE unit per
-   * warp in sst_cluster, two in the batched paths); when an item's amplitudes do not
-   * fit, none of them is stored, its clusters get amp_first = 0xFFFFFFFF and the
-   * event SST_EV_AMP_CAPACITY (the clusters themselves are unaffected). */
+   * cluster order.  Where they do not all fit, the event gets SST_EV_AMP_CAPACITY
+   * and the clusters without amplitudes amp_first = 0xFFFFFFFF (they are otherwise
+   * unaffected): in sst_cluster and the smallest batches every cluster past the
+   * capacity, in larger batches all clusters of an FE unit (or half of one) whose
+   * amplitudes, allocated together, do not fit. */
   uint8_t* amp;            /* [amp_capacity] */
   uint32_t* amp_first;     /* [capacity], absolute index into amp */
   const uint64_t* amp_off; /* sst_batch: [n_events + 1] device, sst_batch_host: [n_events + 1]

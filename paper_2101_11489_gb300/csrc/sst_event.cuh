@@ -702,7 +702,6 @@ __device__ __forceinline__ uint32_t cluster_fed(S& s, const KParams& kp, uint32_
   }
   const Counts before = place(found, amps);
   const unsigned long long n0 = before.clusters, a0 = before.amps;
-  const bool amp_fits = !AMP || a0 + amps <= o.a_room;
   *amps_found = amps;
   if (!AMP && !single && spill && found <= kFedClusters) {
     for (uint32_t r = threadIdx.x; r < found && n0 + r < o.room; r += kThreads) {
@@ -735,8 +734,10 @@ __device__ __forceinline__ uint32_t cluster_fed(S& s, const KParams& kp, uint32_
       }
       const uint32_t wd = (uint32_t)(hi - lo + 1);
       uint32_t a_at = 0, a_tot = 0;
+      bool amp_fits = false;
       if (AMP) {
         a_at = block_scan(s, wd, &a_tot);
+        amp_fits = a0 + arun + a_at + wd <= o.a_room;
         if (have && amp_fits) {
           uint8_t* d = out.amp + o.a_off + a0 + arun + a_at;
           for (uint32_t k = 0; k < wd; k++) d[k] = 0;

@@ -1,7 +1,7 @@
 """sst_cluster on digis that sst_unpack does not write: repeated and descending strips (each
 active digi is then its own candidate, up to 256 in a channel), in a FED of many digi
 chunks between two ordinary ones; and digis of other channels within a channel's range,
-which take no part.
+which take no part.  And amplitude capacities at every kind of limit.
 """
 import numpy as np
 import pytest
@@ -96,3 +96,31 @@ def test_digis_of_other_channels_take_no_part(g, occ, amps):
     n = np.diff(off) + np.bincount(chan, minlength=off.size - 1)
     got, _ = cluster(g, out_s, out_a, np.concatenate([[0], np.cumsum(n)]), amps)
     assert_clusters_equal({k: v for k, v in got.items() if k != "amp_first"}, want)
+
+
+@pytest.mark.parametrize("occ", [0.01, 0.3])
+@pytest.mark.parametrize("short", [0, 1, 1000, -1])
+def test_amplitudes_up_to_the_capacity(g, occ, short):
+    """Every cluster whose amplitudes end within the capacity has them, in a single FED too."""
+    for n_feds in (1, 3):
+        strip, adc, off = ordinary(8, n_feds, occ)
+        digis = {"strip": strip, "adc": adc, "chan_off": off}
+        p = orc_params(g.params)
+        want = orc.cluster_event(digis, n_feds, g.noise, g.gain, g.bad, p)
+        first, amp = orc.cluster_amplitudes(digis, want, g.noise, g.gain, g.bad, p)
+        cap = max(amp.size - short, 1) if short >= 0 else 1  # (a capacity of 0 is refused)
+        d = sst.DigiBuffers.alloc(strip.size, n_feds)
+        d.strip.copy_(torch.from_numpy(strip.astype(np.int32)).cuda())
+        d.adc.copy_(torch.from_numpy(adc).cuda())
+        d.chan_off.copy_(torch.from_numpy(off.astype(np.int32)).cuda())
+        d.status.zero_()
+        c = sst.ClusterBuffers.alloc(want["det"].size, amp_capacity=cap)
+        sst.sst_cluster(g.ctx, d.record(), n_feds, c.record())
+        torch.cuda.synchronize()
+        assert int(d.status[2]) == (sst.SST_EV_AMP_CAPACITY if cap < amp.size else 0)
+        got = c.to_host(0, int(d.status[1]))
+        assert_clusters_equal({k: v for k, v in got.items() if k != "amp_first"}, want)
+        fits = first + want["width"] <= cap
+        assert np.array_equal(got["amp_first"], np.where(fits, first, sst.NO_AMP))
+        end = int((first + want["width"])[fits].max(initial=0))
+        assert np.array_equal(c.amplitudes()[:end], amp[:end])
