@@ -99,25 +99,25 @@ cudaError_t ensure_spill(Scratch& s, size_t warps) {
   return cudaSuccess;
 }
 
-bool amp_scratch_fits(const Scratch& s, size_t amp_bytes) {
-  return amp_bytes <= s.amp_stage_cap && s.amp_items_cap >= s.items_cap && s.amp_ev_cap >= s.ev_cap &&
-         s.stage_amp_cap >= s.stage_cap && s.amp_spill_warps >= s.spill_warps;
+bool amp_scratch_fits(const Scratch& s, size_t items, size_t events, size_t stage_records, size_t amp_bytes) {
+  return amp_bytes <= s.amp_stage_cap && items <= s.amp_items_cap && events <= s.amp_ev_cap &&
+         stage_records <= s.stage_amp_cap && s.spill_warps <= s.amp_spill_warps;
 }
 
-cudaError_t ensure_amp_scratch(Scratch& s, size_t amp_bytes) {
-  if (amp_scratch_fits(s, amp_bytes)) return cudaSuccess;
+cudaError_t ensure_amp_scratch(Scratch& s, size_t items, size_t events, size_t stage_records, size_t amp_bytes) {
+  if (amp_scratch_fits(s, items, events, stage_records, amp_bytes)) return cudaSuccess;
   cudaError_t e = cudaDeviceSynchronize();  // growing: wait for all work that may still use the old buffers
   if (e) return e;
   size_t c1 = 2 * s.amp_items_cap, c2 = 2 * s.amp_items_cap, c3 = s.amp_spill_warps * kAmpSpill;
-  if ((e = grow(s.seg_amp_cnt, c1, 2 * s.items_cap))) return e;
-  if ((e = grow(s.seg_amp_start, c2, 2 * s.items_cap))) return e;
-  s.amp_items_cap = s.items_cap;
+  if ((e = grow(s.seg_amp_cnt, c1, 2 * items))) return e;
+  if ((e = grow(s.seg_amp_start, c2, 2 * items))) return e;
+  if (items > s.amp_items_cap) s.amp_items_cap = items;
   if ((e = grow(s.amp_spill, c3, s.spill_warps * kAmpSpill))) return e;
   s.amp_spill_warps = s.spill_warps;
   size_t counters = counters_for(s.amp_ev_cap);
-  if ((e = grow(s.amp_alloc, counters, counters_for(s.ev_cap)))) return e;
-  s.amp_ev_cap = s.ev_cap;
-  if ((e = grow(s.stage_amp, s.stage_amp_cap, s.stage_cap))) return e;
+  if ((e = grow(s.amp_alloc, counters, counters_for(events)))) return e;
+  if (events > s.amp_ev_cap) s.amp_ev_cap = events;
+  if ((e = grow(s.stage_amp, s.stage_amp_cap, stage_records))) return e;
   return grow(s.amp_stage, s.amp_stage_cap, amp_bytes);
 }
 
@@ -309,7 +309,7 @@ sst_status sst_batch(sst_ctx* ctx, const uint8_t* raw, const uint64_t* event_off
   DeviceGuard g(ctx->device);
   const size_t items = (size_t)n_events * n_feds;
   cudaError_t e = ensure_scratch(ctx->scratch, items * kFe, n_events, out->capacity);
-  if (!e && out->amp) e = ensure_amp_scratch(ctx->scratch, out->amp_capacity);
+  if (!e && out->amp) e = ensure_amp_scratch(ctx->scratch, items * kFe, n_events, out->capacity, out->amp_capacity);
   if (e) return cuda_err(ctx, e, "sst_batch scratch");
   cudaEvent_t eb = nullptr, ee = nullptr;
   if (ctx->profiling) {

@@ -434,13 +434,13 @@ cudaError_t prepare_job(sst_host_pipe& p, const HostJob* job) {
   bool fits = p.scratch.items_cap >= (size_t)job->max_e * nf * sst::kFe && p.scratch.ev_cap >= job->max_e &&
               p.scratch.stage_cap >= job->max_clu;
   const uint64_t amp = job->amps ? (job->max_amp ? job->max_amp : 1) : 0;
-  if (amp) fits = fits && sst::amp_scratch_fits(p.scratch, amp);
+  if (amp) fits = fits && sst::amp_scratch_fits(p.scratch, (size_t)job->max_e * nf * sst::kFe, job->max_e, job->max_clu, amp);
   for (const PipeSlot& s : p.slots) fits = fits && slot_fits(s, job->max_e, nf, job->max_bytes, job->max_clu, amp);
   if (fits) return cudaSuccess;
   cudaError_t e = drain(p);
   if (!e) e = sst::ensure_scratch(p.scratch, (size_t)job->max_e * nf * sst::kFe, job->max_e, job->max_clu);
   if (!e) e = sst::ensure_spill(p.scratch, (size_t)p.ctx->n_sm * sst::kMaxWarpsPerSm);
-  if (!e && amp) e = sst::ensure_amp_scratch(p.scratch, amp);
+  if (!e && amp) e = sst::ensure_amp_scratch(p.scratch, (size_t)job->max_e * nf * sst::kFe, job->max_e, job->max_clu, amp);
   for (PipeSlot& s : p.slots)
     if (!e) e = grow_slot(s, job->max_e, nf, job->max_bytes, job->max_clu, amp);
   return e;

@@ -181,10 +181,10 @@ cudaError_t ensure_scratch(Scratch& s, size_t items, size_t events, size_t stage
 cudaError_t ensure_look(LookState& l, size_t events, size_t items);
 // Candidate lists for `warps` warps of k_stream; grows only.
 cudaError_t ensure_spill(Scratch& s, size_t warps);
-// What k_stream needs for amplitudes beside the above (after ensure_scratch and
-// ensure_spill); grows only.
-cudaError_t ensure_amp_scratch(Scratch& s, size_t amp_bytes);
-bool amp_scratch_fits(const Scratch& s, size_t amp_bytes);
+// What k_stream needs for amplitudes beside the above, for a launch of that size (after
+// ensure_spill); grows only, and only when that launch needs it.
+cudaError_t ensure_amp_scratch(Scratch& s, size_t items, size_t events, size_t stage_records, size_t amp_bytes);
+bool amp_scratch_fits(const Scratch& s, size_t items, size_t events, size_t stage_records, size_t amp_bytes);
 void free_scratch(Scratch& s);
 void free_host_pipe(sst_ctx* ctx);
 

@@ -131,3 +131,36 @@ def test_replays_after_the_context_has_grown(gt):
         dh = d.to_host()
         assert_digis_equal(dh, od)
         assert_clusters_equal(c.to_host(0, dh["n_clusters"]), oc)
+
+
+def test_capture_with_amplitudes_after_a_larger_batch_without(gt):
+    """Once a batch with amplitudes has run, one of its size can be captured, whatever larger batches ran since."""
+    w, calib, g = gt
+    evs = [eg.make_event(w, calib, 40 + i, n_feds=N_FEDS) for i in range(2)]
+    sizes = [e.nbytes for e in evs]
+    eoff, coff, aoff = (torch.from_numpy(np.concatenate([[0], np.cumsum(v)]).astype(np.int64)).cuda()
+                        for v in (sizes, [s // 2 + 1 for s in sizes], [4 * s for s in sizes]))
+    raw = torch.from_numpy(np.concatenate([e.raw for e in evs])).cuda()
+    fl = torch.from_numpy(np.concatenate([e.fed_len for e in evs]).view(np.int32)).cuda()
+    cb = sst.ClusterBuffers.alloc(int(coff[-1]), amp_capacity=int(aoff[-1]))
+    cb.amp_off = aoff
+    st = torch.zeros(8, dtype=torch.int32, device="cuda")
+
+    def launch():
+        sst.sst_batch(g.ctx, raw, eoff, fl, 2, N_FEDS, coff, cb.record(), st)
+
+    launch()
+    g.batch([(e.raw, e.fed_len) for e in evs] * 20)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        launch()
+    st.zero_()
+    cb.det.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    for i, e in enumerate(evs):
+        _, oc, ost = g.oracle(e.raw, e.fed_len, N_FEDS)
+        assert int(st[4 * i + 1]) == ost["n_clusters"]
+        got = cb.to_host(int(coff[i]), ost["n_clusters"])
+        assert_clusters_equal({k: got[k] for k in oc}, oc)
