@@ -17,6 +17,7 @@ sst_status set_err(sst_ctx* c, sst_status code, const std::string& msg) {
 
 sst_status cuda_err(sst_ctx* c, cudaError_t e, const char* where) {
   if (e == cudaSuccess) return SST_OK;
+  cudaGetLastError();  // reported here, not again by the next launch
   return set_err(c, SST_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
@@ -73,15 +74,19 @@ cudaError_t ensure_scratch(Scratch& s, size_t items, size_t events, size_t stage
     if ((e = cudaDeviceSynchronize())) return e;
     if (items > s.items_cap) {
       size_t c1 = s.items_cap, c2 = s.items_cap, c3 = s.items_cap, c4 = s.items_cap;
+      s.items_cap = 0;  // a failure below leaves none of them in use
       if ((e = grow(s.fed_off, c1, items))) return e;
       if ((e = grow(s.fed_cnt, c2, 2 * items))) return e;  // two segments per FE unit at most
       if ((e = grow(s.fed_start, c3, 2 * items))) return e;
       if ((e = grow(s.unit_desc, c4, items))) return e;
       s.items_cap = items;
     }
-    size_t counters = counters_for(s.ev_cap);
-    if ((e = grow(s.ev_alloc, counters, counters_for(events)))) return e;
-    if (events > s.ev_cap) s.ev_cap = events;
+    if (events > s.ev_cap) {
+      size_t counters = counters_for(s.ev_cap);
+      s.ev_cap = 0;
+      if ((e = grow(s.ev_alloc, counters, counters_for(events)))) return e;
+      s.ev_cap = events;
+    }
     if ((e = grow(s.stage, s.stage_cap, stage_records))) return e;
   }
   return cudaSuccess;
@@ -108,15 +113,26 @@ cudaError_t ensure_amp_scratch(Scratch& s, size_t items, size_t events, size_t s
   if (amp_scratch_fits(s, items, events, stage_records, amp_bytes)) return cudaSuccess;
   cudaError_t e = cudaDeviceSynchronize();  // growing: wait for all work that may still use the old buffers
   if (e) return e;
-  size_t c1 = 2 * s.amp_items_cap, c2 = 2 * s.amp_items_cap, c3 = s.amp_spill_warps * kAmpSpill;
-  if ((e = grow(s.seg_amp_cnt, c1, 2 * items))) return e;
-  if ((e = grow(s.seg_amp_start, c2, 2 * items))) return e;
-  if (items > s.amp_items_cap) s.amp_items_cap = items;
-  if ((e = grow(s.amp_spill, c3, s.spill_warps * kAmpSpill))) return e;
-  s.amp_spill_warps = s.spill_warps;
-  size_t counters = counters_for(s.amp_ev_cap);
-  if ((e = grow(s.amp_alloc, counters, counters_for(events)))) return e;
-  if (events > s.amp_ev_cap) s.amp_ev_cap = events;
+  // (a failure leaves what is being grown, and only that, without room)
+  if (items > s.amp_items_cap) {
+    size_t c1 = 2 * s.amp_items_cap, c2 = 2 * s.amp_items_cap;
+    s.amp_items_cap = 0;
+    if ((e = grow(s.seg_amp_cnt, c1, 2 * items))) return e;
+    if ((e = grow(s.seg_amp_start, c2, 2 * items))) return e;
+    s.amp_items_cap = items;
+  }
+  if (s.spill_warps > s.amp_spill_warps) {
+    size_t c = s.amp_spill_warps * kAmpSpill;
+    s.amp_spill_warps = 0;
+    if ((e = grow(s.amp_spill, c, s.spill_warps * kAmpSpill))) return e;
+    s.amp_spill_warps = s.spill_warps;
+  }
+  if (events > s.amp_ev_cap) {
+    size_t c = counters_for(s.amp_ev_cap);
+    s.amp_ev_cap = 0;
+    if ((e = grow(s.amp_alloc, c, counters_for(events)))) return e;
+    s.amp_ev_cap = events;
+  }
   if ((e = grow(s.stage_amp, s.stage_amp_cap, stage_records))) return e;
   return grow(s.amp_stage, s.amp_stage_cap, amp_bytes);
 }

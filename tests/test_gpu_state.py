@@ -164,3 +164,30 @@ def test_capture_with_amplitudes_after_a_larger_batch_without(gt):
         assert int(st[4 * i + 1]) == ost["n_clusters"]
         got = cb.to_host(int(coff[i]), ost["n_clusters"])
         assert_clusters_equal({k: got[k] for k in oc}, oc)
+
+
+def test_a_batch_that_does_not_fit_leaves_the_context_usable(gt):
+    """Scratch that could not grow (the GPU's memory is taken) is not used by the next, smaller batch."""
+    w, calib, g = gt
+    e = eg.make_event(w, calib, 50, n_feds=N_FEDS)
+    n = 1 << 18  # needs about 4 GB of bookkeeping
+    off = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    fl = torch.zeros(1, dtype=torch.int32, device="cuda")  # (the call fails before anything is launched)
+    st = torch.zeros(n * 4, dtype=torch.int32, device="cuda")
+    c = sst.ClusterBuffers.alloc(16)
+    for left in (2.5e9, 1.2e9, 3.5e9):  # a different array fails each time
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        taken = torch.empty(torch.cuda.mem_get_info()[0] - int(left), dtype=torch.uint8, device="cuda")
+        try:
+            with pytest.raises(sst.SstError) as err:
+                sst.sst_batch(g.ctx, st.view(torch.uint8), off, fl, n, N_FEDS, off, c.record(), st)
+            assert err.value.code == sst.SST_ERR_CUDA
+        finally:
+            del taken
+            torch.cuda.empty_cache()
+        for k in (1, 30):
+            for got, cl in g.batch([(e.raw, e.fed_len)] * k):
+                _, oc, ost = g.oracle(e.raw, e.fed_len, N_FEDS)
+                assert got == ost
+                assert_clusters_equal(cl, oc)
