@@ -642,8 +642,7 @@ __global__ void __launch_bounds__(ev::kThreads) k_unpack(const uint8_t* __restri
 
 // The CTA's spill area for a FED of several chunks, or null.
 __device__ __forceinline__ uint2* fed_spill(const KParams& kp) {
-  const size_t have = (size_t)kp.spill_warps * kSpillRecords * 2 / ev::kFedClusters;  // in 8-byte records
-  return blockIdx.x < have ? reinterpret_cast<uint2*>(kp.spill) + (size_t)blockIdx.x * ev::kFedClusters : nullptr;
+  return blockIdx.x < kp.fed_spills ? kp.fed_spill + (size_t)blockIdx.x * kFedClusters : nullptr;
 }
 
 // a3 - a6 per event: one CTA per FED over the digi SoA.  (Four CTAs to an SM, 60 registers,
@@ -1007,11 +1006,13 @@ cudaError_t prepare(const void* fn, int block, size_t smem, int* per_sm) {
   return cudaSuccess;
 }
 
-// The kernels' parameters with the stream's spill areas.
+// The kernels' parameters with the stream's spill areas (k_event's FEDs have k_stream's lists).
 KParams with_spill(const KParams& kp, const Scratch& s) {
   KParams k = kp;
   k.spill = s.spill;
   k.spill_warps = (uint32_t)s.spill_warps;
+  k.fed_spill = reinterpret_cast<uint2*>(s.spill);
+  k.fed_spills = (uint32_t)(s.spill_warps * kSpillRecords * 2 / kFedClusters);
   return k;
 }
 
@@ -1319,7 +1320,10 @@ cudaError_t launch_cluster(const sst_digis& in, uint32_t n_feds, const sst_clust
   const size_t sm = sizeof(ev::Shm<kEvTile, true>);
   auto* k = out.amp ? k_cluster<true> : k_cluster<false>;
   return launch_feds((const void*)k, sm, s, s.look_cluster, 1, n_feds, st, [&](ev::Shared& sh) {
-    return launch_pdl(k, n_feds, (unsigned)ev::kThreads, sm, st, in, with_spill(kp, s), out, sh);
+    KParams kps = kp;
+    kps.fed_spill = s.fed_spill;
+    kps.fed_spills = (uint32_t)s.fed_spills;
+    return launch_pdl(k, n_feds, (unsigned)ev::kThreads, sm, st, in, kps, out, sh);
   });
 }
 

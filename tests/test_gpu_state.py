@@ -191,3 +191,18 @@ def test_a_batch_that_does_not_fit_leaves_the_context_usable(gt):
                 _, oc, ost = g.oracle(e.raw, e.fed_len, N_FEDS)
                 assert got == ost
                 assert_clusters_equal(cl, oc)
+
+
+def test_memory_is_taken_by_the_calls_that_need_it():
+    """A context holds megabytes of scratch only once it has clustered or run a batch."""
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    sst.sst_destroy(sst.sst_create(0, 8))  # (the library's own first use)
+    before = free()
+    ctx = sst.sst_create(0, 8)
+    try:
+        assert before - free() <= 8 << 20
+    finally:
+        sst.sst_destroy(ctx)
