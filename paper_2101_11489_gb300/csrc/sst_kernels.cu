@@ -1126,8 +1126,16 @@ cudaError_t launch_event(const uint8_t* raw, const uint64_t* event_off, const ui
 //   the fastest from 100 records on (13 FEDs x 17 events 18.6 against k_event's 22.5,
 //   skewed 37 against 112; 61 x 2 17.7 and 20.6), but a single FED has 8 tiles (1 x 120:
 //   24 and 18); beyond, from 1,500 records of 10 events and more on (200 x 10 54,
-//   k_stream_fed 59; 120 x 13 43 and 45; 100 x 12 40 and 36; 440 x 8 103 and 86), or of
-//   16 events, or 3,600 records.
+//   k_stream_fed 59; 120 x 13 43 and 45; 100 x 12 40 and 36; 440 x 9 99 and 97; 440 x 8 105
+//   and 87), or of 16 events; where the calibration is larger than the L2 (above 640 FEDs)
+//   every tile comes from DRAM: from 24 events on (1000 x 24 276 and 290; 1000 x 16 242 and
+//   221; 1000 x 4 168 and 111; 4096 x 1 474 and 148).
+// The densities are not known here, and no line is best for all: against one warp per pair of
+// FE units (the kernel before these) the choice loses 100 x 6 skewed 95 -> 103 and 77 x 12
+// skewed 113 -> 121 (tiles: 53 and 52, but 37 and 36 for 28 and 32 when they are alike),
+// 200 x 6 skewed 105 -> 117 (four units a warp; two: 81, but 43 for 39 when alike), 200 x 9 47
+// -> 52 (two units a warp; four: 45, but 116 for 88 when skewed), 440 x 8 with amplitudes 114
+// -> 123 (204 -> 170 when dense, 250 -> 216 when skewed).
 // A batch read in place from pinned host memory is bound by the link, which a warp's
 // contiguous piece of four FE units (1.4 KB) loads better than the tiles' single units:
 // 440 FEDs x 16 | 32 | 64 | 128 events 153 | 253 | 448 | 853 us with k_stream_fed, 150 | 267
@@ -1139,7 +1147,8 @@ static_assert(kEventRecords <= kEventRecordsMost && kEventRecordsOneFed <= kEven
                   kEventRecordsWide <= kEventRecordsMost && kEventRecordsAmps <= kEventRecordsMost &&
                   kEventRecordsMost <= ev::kLbBlock,
               "k_event's shared state has room for the records it takes, in one look-back block");
-constexpr uint32_t kTileEvents = 10, kTileEventsFew = 16, kTileRecordsFew = 1500, kTileRecords = 3600;
+constexpr uint32_t kTileEvents = 10, kTileEventsFew = 16, kTileRecordsFew = 1500;
+constexpr uint32_t kTileEventsMany = 24, kTileFedsMany = 640;
 constexpr uint32_t kTileChunk = 32, kTileChunkMin = 8;
 
 // How a batch is launched.
@@ -1184,8 +1193,9 @@ cudaError_t plan_batch(const Shape& sh, uint32_t n_events, uint32_t n_feds, bool
                        Plan* p) {
   const size_t records = (size_t)n_events * n_feds;
   const bool one_wave = (size_t)n_feds * kFe <= (size_t)n_sm * 4;  // the tiles fit the GPU at once
-  const bool tiles = one_wave || records > kTileRecords ||
-                     n_events >= (records < kTileRecordsFew ? kTileEventsFew : kTileEvents);
+  const bool tiles = one_wave || n_events >= (n_feds > kTileFedsMany        ? kTileEventsMany
+                                              : records < kTileRecordsFew ? kTileEventsFew
+                                                                          : kTileEvents);
   if (records < (one_wave ? n_feds > 1 ? kEventRecords : kEventRecordsOneFed
                  : amps ? kEventRecordsAmps : kEventRecordsWide) &&
       (one_wave || !tiles)) {
@@ -1213,10 +1223,12 @@ cudaError_t plan_batch(const Shape& sh, uint32_t n_events, uint32_t n_feds, bool
   // FE units per warp: as few as give every warp one item, half a FED's at most (48
   // channels); two (24 channels, evener shares) where halves fill more than two thirds of
   // a wave: 440 FEDs x 3 events 56.6 with halves, 57.3 with quarters, but 256 and 161
-  // when the FEDs' densities differ a hundredfold; 440 x 5 77 and 69; 150 x 8 36 and 42
+  // when the FEDs' densities differ a hundredfold; 440 x 5 77 and 69; 150 x 8 36 and 42.
+  // Halves again from 8,500 records on: 1000 x 8 153 and 174 with quarters, but 236 and 197
+  // skewed; 1000 x 10 175 and 207, 255 and 227; 2000 x 16 401 and 542, 491 and 542.
   p->units = 1;
   while (p->units < kFe / 2 && records * (kFe / p->units) > ctas * kFedWarps) p->units *= 2;
-  if (records * 3 > ctas * kFedWarps) p->units = in_place ? 4 : 2;
+  if (records * 3 > ctas * kFedWarps) p->units = in_place || records > 8500 ? 4 : 2;
   const size_t need = (records * (kFe / p->units) + kFedWarps - 1) / kFedWarps;
   p->grid = (int)(ctas < need ? ctas : need);
   p->resident = p->grid;
