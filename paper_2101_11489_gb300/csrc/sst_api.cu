@@ -315,7 +315,7 @@ sst_status sst_cluster(sst_ctx* ctx, const sst_digis* in, uint32_t n_feds, const
   cudaError_t e = ensure_scratch(ctx->scratch, (size_t)n_feds * kFe, 1, 1);
   if (!e) e = ensure_fed_spill(ctx->scratch, ctx->n_feds, (cudaStream_t)stream);
   if (e) return cuda_err(ctx, e, "sst_cluster scratch");
-  e = launch_cluster(*in, n_feds, *out, kparams(ctx), ctx->scratch, (cudaStream_t)stream);
+  e = launch_cluster(*in, n_feds, *out, kparams(ctx), ctx->scratch, ctx->n_sm, (cudaStream_t)stream);
   return cuda_err(ctx, e, "sst_cluster");
 }
 

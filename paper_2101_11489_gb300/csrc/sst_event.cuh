@@ -17,7 +17,7 @@ namespace ev {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kFedBuf = 8192;      // bytes of FED record staged on chip (larger ones are read in place)
+constexpr int kFedBuf = 8192;      // bytes of FED record that have run slots (larger ones are staged without, if at all)
 constexpr int kRunSlots = (kFedBuf + 2) / 3;  // a run header takes at least 3 bytes with its ADC
 constexpr uint32_t kLbBlock = 1024;  // FEDs whose counts a CTA sums one by one
 constexpr uint32_t kNoStatus = 0xFFFFFFFFu;
@@ -287,10 +287,11 @@ __device__ __forceinline__ uint64_t find_fed(S& s, const Lengths& first, const u
   return o;
 }
 
-// Stages the record when it fits; returns where its bytes are.
+// Stages the record when it fits the region (19 KB; beyond kFedBuf the run slots' space
+// holds the rest); returns where its bytes are.
 template <class S>
 __device__ __forceinline__ const uint8_t* stage_record(S& s, const uint8_t* g, uint32_t len) {
-  if (len == 0 || len > (uint32_t)kFedBuf) return g;
+  if (len == 0 || len > (uint32_t)sizeof(s.region)) return g;
   if ((reinterpret_cast<uintptr_t>(g) & 15u) == 0) {
     const uint32_t nv = len >> 4;
     for (uint32_t i = threadIdx.x; i < nv; i += kThreads)
@@ -365,15 +366,15 @@ __device__ __forceinline__ uint32_t prefix_counts(S& s, uint32_t cnt) {
 // FED header, channel length chains, run validation and digi counts.  src: the
 // record's bytes (shared or global).  On return chan_* describe every channel,
 // chan_cnt the digis before it (chan_cnt[96]: all), scal[kFlags] / scal[kBad] the OR
-// of the channel statuses and the number of bad channels.  STAGED (src is the staged
-// record): every valid run's header position | digis of the channel before it << 13 |
+// of the channel statuses and the number of bad channels.  SLOTS (src is the staged
+// record, of at most kFedBuf bytes): every valid run's header position | digis of the channel before it << 13 |
 // channel << 21 | 1 << 31 is left in the slot of its position / 3 (headers are at least
 // 3 bytes apart); the channels are as good as their statuses say.  Returns the digis.
-template <bool STAGED, class S>
+template <bool SLOTS, class S>
 __device__ __forceinline__ uint32_t parse_record(S& s, const uint8_t* src, uint32_t len, uint32_t fed, bool in_range) {
   static_assert(kFedBuf <= 1 << 13, "header positions take 13 bits of a slot");
   const int tid = threadIdx.x, lane = tid & 31;
-  if (STAGED)
+  if (SLOTS)
     for (uint32_t i = tid; i < (len + 2) / 3; i += kThreads) s.slots()[i] = 0;
   if (tid < 32) {
     // header: lanes 0 .. 7 hold one FE unit each
@@ -424,7 +425,7 @@ __device__ __forceinline__ uint32_t parse_record(S& s, const uint8_t* src, uint3
       const uint32_t pos = s.chan_pos[tid];
       const uint8_t* r = src + pos;
       cnt = count_runs(l, [&](uint32_t i) { return (uint32_t)r[i]; }, &st, [&](uint32_t p, uint32_t before) {
-        if (STAGED) s.slots()[(pos + p) / 3] = (pos + p) | (before << 13) | ((uint32_t)tid << 21) | (1u << 31);
+        if (SLOTS) s.slots()[(pos + p) / 3] = (pos + p) | (before << 13) | ((uint32_t)tid << 21) | (1u << 31);
       });
       s.chan_st[tid] = (uint8_t)st;
     }
@@ -469,7 +470,7 @@ __device__ __forceinline__ void emit_channels(S& s, const uint8_t* src, int c0, 
   __syncthreads();
 }
 
-// The same for all channels of a staged record, one thread per run slot.
+// The same for all channels of a record with run slots, a thread each.
 template <class S>
 __device__ __forceinline__ void emit_slots(S& s, uint32_t len) {
   for (uint32_t i = threadIdx.x; i < (len + 2) / 3; i += kThreads) {

@@ -130,7 +130,7 @@ bool shape_valid(const Shape& s);
 cudaError_t launch_unpack(const uint8_t* raw, uint64_t raw_bytes, const uint32_t* fed_len, uint32_t n_feds,
                           const sst_digis& out, Scratch& s, const Shape& sh, cudaStream_t st);
 cudaError_t launch_cluster(const sst_digis& in, uint32_t n_feds, const sst_clusters& out, const KParams& kp,
-                           Scratch& s, cudaStream_t st);
+                           Scratch& s, int n_sm, cudaStream_t st);
 // Kernels launched per batched call: k_fed_scan, k_stream, k_order (and k_clu_scan
 // before it for packed output) for many events; k_event for few or with amplitudes.
 // Batched unpack + cluster.  Event e's clusters are written to the slice [clu_off[e], clu_off[e+1]) of `out` (bounded by

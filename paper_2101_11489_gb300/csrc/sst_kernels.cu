@@ -36,6 +36,7 @@ constexpr uint32_t kLbSpinLimit = 1u << 20;         // polls before giving up (a
 constexpr uint64_t kBadOff = ~0ull;                // fed_off marker: record outside the event
 constexpr int kFedScanThreads = 128;               // FEDs per k_fed_scan CTA
 constexpr int kEvTile = 2048;                      // digis on chip of a CTA that clusters a FED
+constexpr int kEvTileLarge = 4096;                 // the same of a k_cluster launch of one wave
 
 // ---------------------------------------------------------------- small helpers
 
@@ -592,8 +593,8 @@ __global__ void __launch_bounds__(ev::kThreads) k_unpack(const uint8_t* __restri
   bool ok, size_ok, timed_out;
   const uint64_t fo = ev::find_fed(s, lens, fed_len, f, sh.n_feds, 0, raw_bytes, &len, &ok, &size_ok);
   const uint8_t* src = ev::stage_record(s, raw + (ok ? fo : 0), len);
-  const bool staged = src == s.region;
-  const uint32_t total = staged ? ev::parse_record<true>(s, src, len, f, ok) : ev::parse_record<false>(s, src, len, f, ok);
+  const bool slots = src == s.region && len <= (uint32_t)ev::kFedBuf;
+  const uint32_t total = slots ? ev::parse_record<true>(s, src, len, f, ok) : ev::parse_record<false>(s, src, len, f, ok);
   ev::Counts own;
   own.digis = total;
   own.flags = s.scal[ev::kFlags];
@@ -601,7 +602,7 @@ __global__ void __launch_bounds__(ev::kThreads) k_unpack(const uint8_t* __restri
   if (tid == 0) ev::publish(sh, f, own);
   const bool single = total <= (uint32_t)TILE;
   if (single) {  // while the FEDs before this one publish
-    if (staged) ev::emit_slots(s, len);
+    if (slots) ev::emit_slots(s, len);
     else ev::emit_channels(s, src, 0, kCh, lanes);
   }
   const ev::Counts before = ev::look_back<false, true>(s, sh, f, 0, f == sh.n_feds - 1 ? 0u : ev::kNoStatus, own, &timed_out);
@@ -645,12 +646,14 @@ __device__ __forceinline__ uint2* fed_spill(const KParams& kp) {
   return blockIdx.x < kp.fed_spills ? kp.fed_spill + (size_t)blockIdx.x * kFedClusters : nullptr;
 }
 
-// a3 - a6 per event: one CTA per FED over the digi SoA.  (Four CTAs to an SM, 60 registers,
-// rather than five and spills: 440 FEDs 17.3 -> 16.7 us, 8 FEDs 11.2 -> 11.1.)
-template <bool AMP>
-__global__ void __launch_bounds__(ev::kThreads, 4) k_cluster(sst_digis in, KParams kp, sst_clusters out, ev::Shared sh) {
+// a3 - a6 per event: one CTA per FED over the digi SoA.  TILE: three CTAs to an SM with the
+// larger one, four with the smaller.
+template <bool AMP, int TILE>
+__global__ void __launch_bounds__(ev::kThreads, TILE == kEvTileLarge ? 3 : 4) k_cluster(sst_digis in, KParams kp,
+                                                                                       sst_clusters out,
+                                                                                       ev::Shared sh) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  using S = ev::Shm<kEvTile, true>;
+  using S = ev::Shm<TILE, true>;
   S& s = *reinterpret_cast<S*>(smem_raw);
   const int tid = threadIdx.x;
   pdl_release();
@@ -726,7 +729,7 @@ __global__ void __launch_bounds__(ev::kThreads, 4) k_cluster(sst_digis in, KPara
   bool timed_out = false;
   ev::Counts before;
   uint32_t amps;
-  const uint32_t found = ev::cluster_fed<AMP, kEvTile>(
+  const uint32_t found = ev::cluster_fed<AMP, TILE>(
       s, kp, f, total, load,
       [&](uint32_t n, uint32_t a) {
         ev::Counts own;
@@ -797,8 +800,8 @@ __global__ void __launch_bounds__(ev::kThreads, 5) k_event(const uint8_t* __rest
   const uint64_t fo = ev::find_fed(s, lens, len_e, f, n_feds, ev0, ev1, &len, &ok, &size_ok);
   const uint8_t* g = raw + (ok ? fo : 0);
   const uint8_t* src = ev::stage_record(s, g, len);
-  const bool staged = src == s.region;
-  const uint32_t total = staged ? ev::parse_record<true>(s, src, len, f, ok) : ev::parse_record<false>(s, src, len, f, ok);
+  const bool slots = src == s.region && len <= (uint32_t)ev::kFedBuf;
+  const uint32_t total = slots ? ev::parse_record<true>(s, src, len, f, ok) : ev::parse_record<false>(s, src, len, f, ok);
   if (tid < 2 * kCh) s.mul[tid] = __ldg(kp.mul + (size_t)f * 2 * kCh + tid);
   const uint2* cal0 = kp.calq + (size_t)f * kFedStrips;
   const uint32_t lo = e * n_feds, from = pack_off ? 0u : lo;
@@ -809,8 +812,9 @@ __global__ void __launch_bounds__(ev::kThreads, 5) k_event(const uint8_t* __rest
       [&](int c0, int c1) {
         // (the calibration entries take the staged record's place: a FED of several
         // chunks is read from global memory again)
-        if (staged && total <= (uint32_t)kEvTile) ev::emit_slots(s, len);
-        else ev::emit_channels(s, g, c0, c1, ev::lanes_for(c1 - c0));
+        const bool single = total <= (uint32_t)kEvTile;
+        if (slots && single) ev::emit_slots(s, len);
+        else ev::emit_channels(s, single ? src : g, c0, c1, ev::lanes_for(c1 - c0));
         ev::classify_tile(s, cal0, s.chan_cnt[c1] - s.chan_cnt[c0]);
       },
       [&](uint32_t n, uint32_t a) {
@@ -1327,16 +1331,31 @@ cudaError_t launch_unpack(const uint8_t* raw, uint64_t raw_bytes, const uint32_t
   }
 }
 
-cudaError_t launch_cluster(const sst_digis& in, uint32_t n_feds, const sst_clusters& out, const KParams& kp,
-                           Scratch& s, cudaStream_t st) {
-  const size_t sm = sizeof(ev::Shm<kEvTile, true>);
-  auto* k = out.amp ? k_cluster<true> : k_cluster<false>;
+template <int TILE>
+static cudaError_t launch_cluster_t(const sst_digis& in, uint32_t n_feds, const sst_clusters& out, const KParams& kp,
+                                    Scratch& s, cudaStream_t st) {
+  const size_t sm = sizeof(ev::Shm<TILE, true>);
+  auto* k = out.amp ? k_cluster<true, TILE> : k_cluster<false, TILE>;
   return launch_feds((const void*)k, sm, s, s.look_cluster, 1, n_feds, st, [&](ev::Shared& sh) {
     KParams kps = kp;
     kps.fed_spill = s.fed_spill;
     kps.fed_spills = (uint32_t)s.fed_spills;
     return launch_pdl(k, n_feds, (unsigned)ev::kThreads, sm, st, in, kps, out, sh);
   });
+}
+
+// The larger tile while all FEDs fit the GPU at once with it: a FED of more than a tile of
+// digis goes through the steps chunk by chunk.  440 FEDs, unpacking included: 31.4 -> 28.8 us
+// (fewer registers spilled), densities a hundredfold apart 73.7 -> 69.2, 4,700 digis a FED 106
+// -> 99; but 500 FEDs, two waves then, 32 -> 39.
+cudaError_t launch_cluster(const sst_digis& in, uint32_t n_feds, const sst_clusters& out, const KParams& kp,
+                           Scratch& s, int n_sm, cudaStream_t st) {
+  int per_sm = 0;
+  const cudaError_t e = prepare((const void*)k_cluster<false, kEvTileLarge>, ev::kThreads,
+                                sizeof(ev::Shm<kEvTileLarge, true>), &per_sm);
+  if (e) return e;
+  return (size_t)n_feds <= (size_t)n_sm * per_sm ? launch_cluster_t<kEvTileLarge>(in, n_feds, out, kp, s, st)
+                                                 : launch_cluster_t<kEvTile>(in, n_feds, out, kp, s, st);
 }
 
 cudaError_t launch_batch(const uint8_t* raw, const uint64_t* event_off, const uint32_t* fed_len, uint32_t n_events,

@@ -1,5 +1,6 @@
-"""Batches of detectors larger than the whole one (the calibration no longer fits the L2), on
-either side of the lines between the batched kernels, against the oracle.
+"""Detectors larger than the whole one, on either side of the lines drawn by FEDs, against the
+oracle: batches (the calibration no longer fits the L2) and single events of sparse and
+dense FEDs (above three FEDs an SM the clustering's tile is the smaller one).
 """
 import numpy as np
 import pytest
@@ -11,7 +12,8 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("no CUDA device", allow_module_level=True)
 
-from _gpu_util import Gpu, assert_clusters_equal  # noqa: E402
+from _gpu_util import Gpu, assert_clusters_equal, assert_digis_equal  # noqa: E402
+from test_gpu_feds import patterns  # noqa: E402
 
 
 @pytest.mark.parametrize("n_feds,n_events", [(640, 10), (641, 10), (641, 13), (641, 14), (641, 23), (641, 24), (1030, 3)])
@@ -29,5 +31,20 @@ def test_choice_above_the_whole_detector(n_feds, n_events):  # 8,333 | 8,974 rec
             oc, ost = want[i % 2]
             assert st == ost
             assert_clusters_equal(cl, oc)
+    finally:
+        g.close()
+
+
+@pytest.mark.parametrize("n_feds", [456, 457])
+def test_dense_and_sparse_feds_of_one_event(n_feds):
+    calib = eg.make_calibration(n_feds, 31, 0.01)
+    g = Gpu(calib.noise, calib.gain, calib.bad)
+    try:
+        pats = patterns(n_feds, 9)
+        for raw, fl in (pats["mixed"], pats["edge"]):
+            dh, ch = g.event(raw, fl, n_feds)
+            od, oc, _ = g.oracle(raw, fl, n_feds)
+            assert_digis_equal(dh, od)
+            assert_clusters_equal(ch, oc)
     finally:
         g.close()
