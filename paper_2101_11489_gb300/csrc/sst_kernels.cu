@@ -245,6 +245,7 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_stream(const uint8_t* __rest
                                                            const uint2* __restrict__ unit_desc, uint32_t chunk,
                                                            uint32_t per_warp, uint32_t resident, cs::Amps am) {
   constexpr int C = 3 * W / 2, kParts = kChPerFe / C;  // channels of the tile, tiles per FE unit
+  static_assert(!AMP || sizeof(uint2) * C * kStrips + W * sizeof(cs::WarpT<U>) <= cs::kFromLimit, "Walk::from");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint2* tile = reinterpret_cast<uint2*>(smem_raw);
   cs::WarpT<U>* warps = reinterpret_cast<cs::WarpT<U>*>(smem_raw + sizeof(uint2) * C * kStrips);
@@ -337,6 +338,7 @@ __global__ void __launch_bounds__(kFedWarps * 32, 3) k_stream_fed(
     const uint64_t* __restrict__ clu_off, uint64_t out_cap, sst_event_status* status, KParams kp, uint2* stage,
     uint32_t* ev_alloc, uint32_t* seg_cnt, uint32_t* seg_start, uint32_t* ticket, const uint2* __restrict__ unit_desc,
     uint32_t units, cs::Amps am) {
+  static_assert(!AMP || kFedWarps * sizeof(FedWarp) <= cs::kFromLimit, "Walk::from");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   FedWarp& w = reinterpret_cast<FedWarp*>(smem_raw)[warp];

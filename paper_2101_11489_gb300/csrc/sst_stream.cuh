@@ -18,6 +18,9 @@ namespace cs {
 
 constexpr uint32_t kNotKept = 0xFFFFFFFFu;
 constexpr int kRefill = 12;  // lanes still walking when the others take new channels
+// Dynamic shared memory of a CTA whose shared addresses fit the 16 bits that Walk::from has
+// for them (2 KB are left to static variables and the system).
+constexpr size_t kFromLimit = 65536 - 2048;
 
 // Per-warp shared memory.  A warp takes up to 4 U slots at once, a slot being C = 12
 // (or 6) consecutive channels of one FE unit of one event.  With U = 2 eight warps
