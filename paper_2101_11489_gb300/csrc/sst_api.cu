@@ -104,19 +104,6 @@ cudaError_t ensure_spill(Scratch& s, size_t warps) {
   return cudaSuccess;
 }
 
-cudaError_t ensure_fed_spill(Scratch& s, size_t feds, cudaStream_t st) {
-  if (s.fed_spill) return cudaSuccess;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  cudaError_t e = cudaStreamIsCapturing(st, &cs);
-  if (e || cs != cudaStreamCaptureStatusNone) return e;
-  if ((e = cudaMalloc(&s.fed_spill, feds * kFedClusters * sizeof(uint2)))) {
-    s.fed_spill = nullptr;
-    return e;
-  }
-  s.fed_spills = feds;
-  return cudaSuccess;
-}
-
 bool amp_scratch_fits(const Scratch& s, size_t items, size_t events, size_t stage_records, size_t amp_bytes) {
   return amp_bytes <= s.amp_stage_cap && items <= s.amp_items_cap && events <= s.amp_ev_cap &&
          stage_records <= s.stage_amp_cap && s.spill_warps <= s.amp_spill_warps;
@@ -161,7 +148,6 @@ void free_scratch(Scratch& s) {
   if (s.stage) cudaFree(s.stage);
   if (s.tickets) cudaFree(s.tickets);
   if (s.spill) cudaFree(s.spill);
-  if (s.fed_spill) cudaFree(s.fed_spill);
   for (void* p : {(void*)s.amp_stage, (void*)s.stage_amp, (void*)s.amp_alloc, (void*)s.seg_amp_cnt,
                   (void*)s.seg_amp_start, (void*)s.amp_spill})
     if (p) cudaFree(p);
@@ -250,6 +236,10 @@ sst_status sst_calib_upload(sst_ctx* ctx, const float* noise, const float* gain,
   DeviceGuard g(ctx->device);
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e = cudaSuccess;
+  // what clustering needs beside the tables, at its one size (launches captured into a
+  // graph keep its address): here, so that contexts that only unpack do without
+  if ((e = ensure_spill(ctx->scratch, (size_t)ctx->n_sm * kMaxWarpsPerSm)))
+    return cuda_err(ctx, e, "sst_calib_upload scratch");
   if (!ctx->calq) {
     if ((e = cudaMalloc(&ctx->calq, n * sizeof(uint2)))) return cuda_err(ctx, e, "cudaMalloc calq");
     if ((e = cudaMalloc(&ctx->badmask, n / 8))) return cuda_err(ctx, e, "cudaMalloc badmask");
@@ -313,7 +303,6 @@ sst_status sst_cluster(sst_ctx* ctx, const sst_digis* in, uint32_t n_feds, const
     return set_err(ctx, SST_ERR_INVALID_ARG, "sst_cluster: amp needs amp_first and 1 <= amp_capacity < 2^32 - 1");
   DeviceGuard g(ctx->device);
   cudaError_t e = ensure_scratch(ctx->scratch, (size_t)n_feds * kFe, 1, 1);
-  if (!e) e = ensure_fed_spill(ctx->scratch, ctx->n_feds, (cudaStream_t)stream);
   if (e) return cuda_err(ctx, e, "sst_cluster scratch");
   e = launch_cluster(*in, n_feds, *out, kparams(ctx), ctx->scratch, ctx->n_sm, (cudaStream_t)stream);
   return cuda_err(ctx, e, "sst_cluster");
@@ -338,8 +327,6 @@ sst_status sst_batch(sst_ctx* ctx, const uint8_t* raw, const uint64_t* event_off
   DeviceGuard g(ctx->device);
   const size_t items = (size_t)n_events * n_feds;
   cudaError_t e = ensure_scratch(ctx->scratch, items * kFe, n_events, out->capacity);
-  // (one size: launches captured into a graph keep its address)
-  if (!e) e = ensure_spill(ctx->scratch, (size_t)ctx->n_sm * kMaxWarpsPerSm);
   if (!e && out->amp) e = ensure_amp_scratch(ctx->scratch, items * kFe, n_events, out->capacity, out->amp_capacity);
   if (e) return cuda_err(ctx, e, "sst_batch scratch");
   cudaEvent_t eb = nullptr, ee = nullptr;

@@ -19,6 +19,7 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kFedBuf = 8192;      // bytes of FED record that have run slots (larger ones are staged without, if at all)
 constexpr int kRunSlots = (kFedBuf + 2) / 3;  // a run header takes at least 3 bytes with its ADC
+constexpr uint32_t kFedClusters = kCh * kStrips / 2;  // most clusters of a FED whose strips ascend
 constexpr uint32_t kLbBlock = 1024;  // FEDs whose counts a CTA sums one by one
 constexpr uint32_t kNoStatus = 0xFFFFFFFFu;
 static_assert(kLbBlock == 1024 && LookState::kTags == 1024, "sizes of the shared state (LookState)");

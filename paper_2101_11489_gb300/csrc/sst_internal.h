@@ -35,8 +35,6 @@ struct KParams {
   const int32_t* mul;       // [n_strips / 128]: per APV, the fixed-point charge multiplier, or the bits of -gain (k_gain_pack)
   uint4* spill = nullptr;   // k_stream: candidate lists (one per warp of the grid, kSpillRecords records each)
   uint32_t spill_warps = 0; // warps that have one
-  uint2* fed_spill = nullptr;  // k_cluster, k_event: clusters of the FEDs of several chunks
-  uint32_t fed_spills = 0;     // CTAs that have an area
 };
 
 // Launch shape of the kernels.
@@ -86,8 +84,6 @@ struct Scratch {
   uint32_t* tickets = nullptr;       // [16]: [0] k_stream's tiles, [1] k_clu_scan's CTAs done
   uint4* spill = nullptr;            // per warp of k_stream, kSpillRecords candidate records
   size_t spill_warps = 0;            // warps that have them
-  uint2* fed_spill = nullptr;        // per CTA of k_cluster, 96 x 128 clusters (contexts only)
-  size_t fed_spills = 0;             // CTAs that have them
   // clusters with amplitudes (k_stream)
   uint8_t* amp_stage = nullptr;      // staged amplitudes, sliced per event like the output
   size_t amp_stage_cap = 0;
@@ -113,7 +109,6 @@ __host__ __device__ constexpr size_t counter_at(uint32_t e) {
 constexpr size_t counters_for(size_t events) { return (events + 32767) / 32768 * 32768; }
 constexpr uint32_t kNoAmp = 0xFFFFFFFFu;
 constexpr uint32_t kSpillRecords = 1608;  // records per warp spill area (25 KiB)
-constexpr uint32_t kFedClusters = kCh * kStrips / 2;  // most clusters of a FED whose strips ascend
 constexpr uint32_t kAmpSpill = kSpillRecords + 128;  // words per warp beside them for clusters with amplitudes
 constexpr int kMaxWarpsPerSm = 32;        // resident warps of the batched kernel per SM (its register use)
 
@@ -186,9 +181,6 @@ cudaError_t ensure_scratch(Scratch& s, size_t items, size_t events, size_t stage
 cudaError_t ensure_look(LookState& l, size_t events, size_t items);
 // Candidate lists for `warps` warps of k_stream; grows only.
 cudaError_t ensure_spill(Scratch& s, size_t warps);
-// Areas for k_cluster's FEDs of several chunks, once.  A launch captured before has none,
-// and goes through such FEDs twice.
-cudaError_t ensure_fed_spill(Scratch& s, size_t feds, cudaStream_t st);
 // What k_stream needs for amplitudes beside the above, for a launch of that size (after
 // ensure_spill); grows only, and only when that launch needs it.
 cudaError_t ensure_amp_scratch(Scratch& s, size_t items, size_t events, size_t stage_records, size_t amp_bytes);

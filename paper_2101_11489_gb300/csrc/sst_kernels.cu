@@ -645,7 +645,8 @@ __global__ void __launch_bounds__(ev::kThreads) k_unpack(const uint8_t* __restri
 
 // The CTA's spill area for a FED of several chunks, or null.
 __device__ __forceinline__ uint2* fed_spill(const KParams& kp) {
-  return blockIdx.x < kp.fed_spills ? kp.fed_spill + (size_t)blockIdx.x * kFedClusters : nullptr;
+  const size_t have = (size_t)kp.spill_warps * kSpillRecords * 2 / ev::kFedClusters;  // in 8-byte records
+  return blockIdx.x < have ? reinterpret_cast<uint2*>(kp.spill) + (size_t)blockIdx.x * ev::kFedClusters : nullptr;
 }
 
 // a3 - a6 per event: one CTA per FED over the digi SoA.  TILE: three CTAs to an SM with the
@@ -1012,13 +1013,11 @@ cudaError_t prepare(const void* fn, int block, size_t smem, int* per_sm) {
   return cudaSuccess;
 }
 
-// The kernels' parameters with the stream's spill areas (k_event's FEDs have k_stream's lists).
+// The kernels' parameters with the stream's spill areas.
 KParams with_spill(const KParams& kp, const Scratch& s) {
   KParams k = kp;
   k.spill = s.spill;
   k.spill_warps = (uint32_t)s.spill_warps;
-  k.fed_spill = reinterpret_cast<uint2*>(s.spill);
-  k.fed_spills = (uint32_t)(s.spill_warps * kSpillRecords * 2 / kFedClusters);
   return k;
 }
 
@@ -1339,10 +1338,7 @@ static cudaError_t launch_cluster_t(const sst_digis& in, uint32_t n_feds, const 
   const size_t sm = sizeof(ev::Shm<TILE, true>);
   auto* k = out.amp ? k_cluster<true, TILE> : k_cluster<false, TILE>;
   return launch_feds((const void*)k, sm, s, s.look_cluster, 1, n_feds, st, [&](ev::Shared& sh) {
-    KParams kps = kp;
-    kps.fed_spill = s.fed_spill;
-    kps.fed_spills = (uint32_t)s.fed_spills;
-    return launch_pdl(k, n_feds, (unsigned)ev::kThreads, sm, st, in, kps, out, sh);
+    return launch_pdl(k, n_feds, (unsigned)ev::kThreads, sm, st, in, with_spill(kp, s), out, sh);
   });
 }
 

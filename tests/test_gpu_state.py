@@ -194,7 +194,7 @@ def test_a_batch_that_does_not_fit_leaves_the_context_usable(gt):
 
 
 def test_memory_is_taken_by_the_calls_that_need_it():
-    """A context holds megabytes of scratch only once it has clustered or run a batch."""
+    """A context that has no calibration (one that only unpacks) holds no candidate lists."""
     def free():
         torch.cuda.synchronize()
         return torch.cuda.mem_get_info()[0]
