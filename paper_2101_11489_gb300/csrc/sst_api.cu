@@ -1,6 +1,7 @@
 // sst_api.cu -- host side of the C ABI declared in include/sst.h: contexts,
 // calibration upload (arXiv 2101.11489 section 2: noise and gain per strip, here
 // plus the bad-strip list), argument checks and kernel launches.
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -446,8 +447,18 @@ sst_status sst_autotune(sst_ctx* ctx, const uint8_t* raw, const uint64_t* event_
   const int per_sm[] = {2, 3, 4, 6, 8};
   float best_t = 1e30f;
   Shape best_s = keep;
-  std::vector<std::pair<int, Shape>> timed;  // (effective grid, shape) already measured
-  cudaError_t ce = cudaSuccess;
+  // launches already measured; the context's own shape stands for the launch it gives
+  struct Launch {
+    int grid = 0, block = 0, items = 0;
+    size_t smem = 0;
+    bool operator==(const Launch& o) const { return grid == o.grid && block == o.block && smem == o.smem; }
+  };
+  std::vector<Launch> timed;
+  auto launch_of = [&](const Shape& s, Launch* l) {
+    return batch_launch_info(s, n_events, n_feds, ctx->n_sm, &l->grid, &l->smem, &l->block, &l->items);
+  };
+  Launch kept;
+  cudaError_t ce = launch_of(keep, &kept);
   for (int b : blocks)
     for (int u : widths)
       for (int p : per_sm) {
@@ -455,16 +466,13 @@ sst_status sst_autotune(sst_ctx* ctx, const uint8_t* raw, const uint64_t* event_
         s.block = b;
         s.units = u;
         s.ctas_per_sm = p;
-        if (!shape_valid(s)) continue;
-        int grid = 0, block = 0, ipf = 0;
-        size_t smem = 0;
-        if ((ce = batch_launch_info(s, n_events, n_feds, ctx->n_sm, &grid, &smem, &block, &ipf))) break;
-        if (smem * (size_t)p > 227u * 1024u) continue;
-        bool dup = false;  // the occupancy clamps p: the same launch was timed already
-        for (auto& pr : timed)
-          if (pr.first == grid && pr.second.block == b && pr.second.units == u) dup = true;
-        if (dup) continue;
-        timed.emplace_back(grid, s);
+        if (ce || !shape_valid(s)) continue;
+        Launch l;
+        if ((ce = launch_of(s, &l))) break;
+        if (l.smem * (size_t)p > 227u * 1024u) continue;
+        if (std::find(timed.begin(), timed.end(), l) != timed.end()) continue;
+        timed.push_back(l);
+        if (l == kept) s = keep;
         float ms_total = 0.f;
         for (int rep = 0; rep < 3 && ce == cudaSuccess; rep++) {
           ce = cudaEventRecord(e0, st);
