@@ -201,12 +201,16 @@ const char* sst_last_error(const sst_ctx* ctx);
  *   noise [n_feds*96*256] float, finite, >= 0   (ADC counts)
  *   gain  [n_feds*96*2]   float, finite, > 0    (one per 128-strip APV)
  *   bad   [n_feds*96*256] uint8, 0 = good, else bad
- * and the thresholds.  The tables are copied to device memory and stay resident;
+ * and the thresholds.  The first upload takes the clustering's candidate lists
+ * (about 125 MB).  The tables are copied to device memory and stay resident;
  * a new upload replaces them after work already queued on `stream`, and returns
  * once they are in place.  From the bad-strip flags and the hole / bad-strip
  * limits the device also builds a bit mask and, per strip, a linking limit from
  * the longest gap below it that still links two successive active strips (one
- * byte per strip), which the clusterizers read instead of walking each gap.
+ * byte per strip), which the clusterizers read instead of walking each gap, and per
+ * APV an exact fixed-point charge multiplier.  An APV with a gain below 1/4 has none,
+ * nor has one in 20,000 above: larger batches then read its FE unit's channels by a
+ * slower routine (all gains below 1/4: up to 12% of a batch with amplitudes).
  * INVALID_ARG on a null pointer, a non-finite or negative value, or parameters
  * outside their requirements; the previous calibration then stays in place. */
 sst_status sst_calib_upload(sst_ctx* ctx, const float* noise, const float* gain, const uint8_t* bad,
@@ -229,9 +233,9 @@ sst_status sst_unpack(sst_ctx* ctx, const uint8_t* raw, uint64_t raw_bytes, cons
 /* Clusters one event's digis (as sst_unpack wrote them, for n_feds FEDs) with the
  * three-threshold algorithm (section 2).  Writes the cluster SoA and sets
  * in->status->n_clusters.  When the event has more clusters than out->capacity,
- * SST_EV_CLUSTER_CAPACITY is ORed into in->status->flags and the arrays hold a
- * sorted subset of the event's clusters (those of whole FE units, in allocation
- * order).  NO_CALIB before sst_calib_upload. */
+ * SST_EV_CLUSTER_CAPACITY is ORed into in->status->flags and the arrays hold the
+ * first of them in order.  A digi whose strip is not of the channel in whose range
+ * it stands takes no part.  NO_CALIB before sst_calib_upload. */
 sst_status sst_cluster(sst_ctx* ctx, const sst_digis* in, uint32_t n_feds, const sst_clusters* out,
                        void* stream);
 
@@ -263,7 +267,7 @@ sst_status sst_unpack_noalloc(const uint8_t* raw, uint64_t raw_bytes, const uint
 /* Unpacks and clusters n_events events; digis stay on chip.  The smallest batches
  * take one launch, a block per FED record.  In larger ones a lane reads a channel
  * record; the clusters are staged (context scratch of out->capacity records), then
- * ordered and copied per event by one more kernel (two with amplitudes).  The
+ * ordered and copied per event by one more kernel.  The
  * launch sequence allocates nothing once the context has run one batch of this
  * size, so it can be captured in a CUDA graph.  All pointers are device memory:
  *   raw        events back to back; event e occupies [event_off[e], event_off[e+1]),
@@ -272,7 +276,10 @@ sst_status sst_unpack_noalloc(const uint8_t* raw, uint64_t raw_bytes, const uint
  *   fed_len    [n_events * n_feds] uint32, event-major
  *   clu_off    [n_events + 1] uint64: event e's clusters go to
  *              [clu_off[e], clu_off[e+1]) of out's arrays (capacity per event);
- *              clu_off[n_events] <= out->capacity
+ *              clu_off[n_events] <= out->capacity.  An event with more clusters
+ *              than that is flagged SST_EV_CLUSTER_CAPACITY and keeps a sorted
+ *              subset: its first ones (smallest batches), or whole FE units' in
+ *              allocation order, the last one cut
  *   status     [n_events] per-event status records
  * Output is identical, event by event, to sst_unpack + sst_cluster on each event
  * alone.  NO_CALIB before sst_calib_upload. */
@@ -387,15 +394,17 @@ sst_status sst_autotune_host(sst_ctx* ctx, const uint8_t* raw, const uint64_t* e
                              uint32_t n_events, uint32_t n_feds, const sst_clusters* out, uint64_t* event_first,
                              sst_event_status* status, uint32_t* best_chunk, float* best_us);
 
-/* What the context's knobs make of a batch of n_events x n_feds: the batched
- * kernel's grid (CTAs), threads per CTA, dynamic shared memory per CTA and work
- * items per FED, and the number of chunks sst_batch_host cuts the batch into.
- * Any output pointer may be NULL.  CUDA if the occupancy look-up fails. */
+/* What the context's knobs make of a batch of n_events x n_feds without
+ * amplitudes: the batched kernel's grid (CTAs), threads per CTA and dynamic shared
+ * memory per CTA, the shares a FED is cut into, and the number of chunks
+ * sst_batch_host cuts the batch into.  CUDA if the occupancy look-up fails. */
 typedef struct {
   uint32_t grid;
   uint32_t block;
   uint32_t smem_bytes;
-  uint32_t items_per_fed;
+  uint32_t items_per_fed; /* 1: a block takes a FED record; 8 / n: a warp takes n FE units of one; many
+                             events: 8 / units_per_warp (there a work item is one FE unit, or half of one
+                             with 128 threads, over many events: 8 or 16 items per FED and share of them) */
   uint32_t host_chunks;
 } sst_launch_info;
 sst_status sst_get_launch_info(sst_ctx* ctx, uint32_t n_events, uint32_t n_feds, sst_launch_info* info);
@@ -467,7 +476,8 @@ sst_status sst_server_stop(sst_ctx* ctx);
  * zero_copy).  Admission by memory: sst_server_start divides the device budget
  * into max_inflight batch slots of equal size, each holding a raw arena of
  * budget / (25 max_inflight) bytes and the cluster and staging arrays for it, so
- * that the device memory in use never exceeds the budget; admitted events wait
+ * that the device memory the events take never exceeds the budget (each slot's
+ * candidate lists, about 125 MB, and FED bookkeeping are beside it); admitted events wait
  * for a slot in a pinned host pool of max_inflight + 1 raw arenas (at most 2 GiB;
  * with zero_copy the event's size is reserved in it, its bytes stay with the
  * caller).

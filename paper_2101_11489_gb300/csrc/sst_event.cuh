@@ -7,8 +7,8 @@
 // around the step is kept short: no prologue (a CTA sums the FED lengths before its
 // own), no ordering pass (a CTA sums the counts that the FEDs before it publish) and
 // no clearing between launches (what a launch reads carries its tag).  An event
-// of 440 FEDs took 48 us in four launches and a memset, a warp per FE unit; it takes 35
-// in two (8 FEDs: 29 and 17; the allocation-free unpack of 440 FEDs: 22 and 12.5).
+// of 440 FEDs took 48 us in four launches and a memset, a warp per FE unit; it takes 30
+// in two (8 FEDs: 29 and 17; the allocation-free unpack of 440 FEDs: 21 and 11).
 //
 // Included by sst_kernels.cu only, inside its namespace.
 #pragma once

@@ -25,7 +25,8 @@ constexpr int kMaskWords = kStrips / 32;     // 8 words of 32 strips per channel
 
 // Calibration and thresholds as the kernels see them.  The per-strip tables are
 // built on the device at calibration upload (k_calib_pack) from the noise, the
-// bad-strip flags and the parameters; the per-APV multipliers on the host.
+// bad-strip flags and the parameters, the per-APV multipliers from the gains
+// (k_gain_pack).
 struct KParams {
   float t_cluster;
   int max_adj;
@@ -126,8 +127,8 @@ cudaError_t launch_unpack(const uint8_t* raw, uint64_t raw_bytes, const uint32_t
                           const sst_digis& out, Scratch& s, const Shape& sh, cudaStream_t st);
 cudaError_t launch_cluster(const sst_digis& in, uint32_t n_feds, const sst_clusters& out, const KParams& kp,
                            Scratch& s, int n_sm, cudaStream_t st);
-// Kernels launched per batched call: k_fed_scan, k_stream, k_order (and k_clu_scan
-// before it for packed output) for many events; k_event for few or with amplitudes.
+// Kernels launched per batched call: k_event alone for the fewest events; else k_fed_scan,
+// k_stream or k_stream_fed, and k_order (before it k_clu_scan for packed output).
 // Batched unpack + cluster.  Event e's clusters are written to the slice [clu_off[e], clu_off[e+1]) of `out` (bounded by
 // out.capacity).  With pack_off (device, n_events + 1 values) the events' clusters
 // are written back to back instead, event e from pack_off[e], which the launch

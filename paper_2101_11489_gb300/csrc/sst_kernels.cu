@@ -6,13 +6,14 @@
 // entries of one FE unit in shared memory while all events' records of it pass; where
 // the events are too few for that, or their records are read in place from host memory,
 // each warp reads them from global memory (k_stream_fed).  The FED headers are checked by
-// a prologue (k_fed_scan), which hands every FE unit its byte range; the kept clusters are staged per FE unit and event and put in
-// order by k_order.  Placing them with a look-back over the units before instead
-// would make every warp wait for units that other CTAs take at the same time.
+// a prologue (k_fed_scan), which hands every FE unit its byte range; the kept clusters are
+// staged per FE unit and event and put in order by k_order.  Placing them with a look-back
+// over the units before instead would make every warp wait for units that other CTAs take
+// at the same time.
 //
-// Single events and the smallest batches (k_unpack, k_cluster, k_event, sst_event.cuh): one CTA per FED, which finds its record, and with a
-// look-back over the FEDs before it its place in the output, by itself; one launch
-// per call.
+// Single events and the smallest batches (k_unpack, k_cluster, k_event, sst_event.cuh):
+// one CTA per FED, which finds its record, and with a look-back over the FEDs before it
+// its place in the output, by itself; one launch per call.
 //
 // Floating point in the threshold tests and sums uses explicit round-to-nearest
 // intrinsics (__fmul_rn, __fadd_rn, __fdiv_rn, __fsqrt_rn): no multiply-add is
@@ -158,8 +159,8 @@ __device__ void describe_fed(const uint8_t* __restrict__ raw, uint64_t fo, uint3
 // lengths of the FEDs before them itself.  Every FED's header is checked and its FE
 // units described (describe_fed).  It is also the launch sequence's prologue: the
 // event's last CTA writes its status (zero but SST_EV_SIZE), its first clears the
-// staging counters (amp_alloc: when given), the very first clears the work tickets.  Event e's bytes are
-// [event_off[e], event_end[e]) when event_end is given (events that do not follow
+// staging counters (amp_alloc: when given), the very first clears the work tickets.
+// Event e's bytes are [event_off[e], event_end[e]) when event_end is given (events that do not follow
 // one another, e.g. read in place from host memory), else [event_off[e],
 // event_off[e + 1]).
 __global__ void k_fed_scan(const uint64_t* __restrict__ event_off, const uint64_t* __restrict__ event_end,
@@ -884,7 +885,9 @@ __global__ void k_badmask(const uint8_t* __restrict__ bad, uint32_t* __restrict_
 // corrected by the strip's gain); checked here for all of them.  Of U[0.8, 1.2]
 // gains all but 5 in 100,000 have one within 4 of 2^22 / gain (a quotient that
 // rounds up to a half has none); for those, and for gains below 1/4, where the
-// product would pass 32 bits, the bits of -gain: the kernels then divide.
+// product would pass 32 bits, the bits of -gain: the kernels then divide, and the
+// streams take walk_any for the FE unit's channels (16 events with amplitudes and one such
+// APV in 1,000: 180 us for 175; all gains below 1/4: 148, of which the division is 2).
 __global__ void k_gain_pack(const float* __restrict__ gain, int32_t* __restrict__ mul, uint32_t n_apv) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_apv) return;
