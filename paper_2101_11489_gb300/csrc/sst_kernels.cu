@@ -37,7 +37,7 @@ constexpr uint32_t kLbSpinLimit = 1u << 20;         // polls before giving up (a
 constexpr uint64_t kBadOff = ~0ull;                // fed_off marker: record outside the event
 constexpr int kFedScanThreads = 128;               // FEDs per k_fed_scan CTA
 constexpr int kEvTile = 2048;                      // digis on chip of a CTA that clusters a FED
-constexpr int kEvTileLarge = 4096;                 // the same of a k_cluster launch of one wave
+constexpr int kEvTileLarge = 4096;                 // the same while all CTAs fit the GPU at once with it
 
 // ---------------------------------------------------------------- small helpers
 
@@ -756,10 +756,11 @@ __global__ void __launch_bounds__(ev::kThreads, TILE == kEvTileLarge ? 3 : 4) k_
 
 // a7 for few events: every FED of every event unpacked and clustered by one CTA, the
 // digis in shared memory.  Event e's clusters go to its slice [clu_off[e], clu_off[e + 1]) of the output or, with pack_off, right
-// after those of the events before it (pack_off[e], which its first CTA writes).  Five CTAs
-// to an SM, so that 700 FED records are one wave (four: 77 FEDs x 9 events 40 us for 28).
-template <bool AMP>
-__global__ void __launch_bounds__(ev::kThreads, 5) k_event(const uint8_t* __restrict__ raw,
+// after those of the events before it (pack_off[e], which its first CTA writes).  TILE:
+// three CTAs to an SM with the larger one, five with the smaller, so that 700 FED records
+// are one wave (four: 77 FEDs x 9 events 40 us for 28).
+template <bool AMP, int TILE>
+__global__ void __launch_bounds__(ev::kThreads, TILE == kEvTileLarge ? 3 : 5) k_event(const uint8_t* __restrict__ raw,
                                                         const uint64_t* __restrict__ event_off,
                                                         const uint64_t* __restrict__ event_end,
                                                         const uint32_t* __restrict__ fed_len, uint32_t n_events,
@@ -767,7 +768,7 @@ __global__ void __launch_bounds__(ev::kThreads, 5) k_event(const uint8_t* __rest
                                                         sst_event_status* status, KParams kp, uint64_t* pack_off,
                                                         ev::Shared sh) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  using S = ev::Shm<kEvTile, true>;
+  using S = ev::Shm<TILE, true>;
   S& s = *reinterpret_cast<S*>(smem_raw);
   const int tid = threadIdx.x;
   pdl_release();
@@ -811,12 +812,12 @@ __global__ void __launch_bounds__(ev::kThreads, 5) k_event(const uint8_t* __rest
   const uint32_t lo = e * n_feds, from = pack_off ? 0u : lo;
   ev::Counts before;
   uint32_t amps;
-  const uint32_t found = ev::cluster_fed<AMP, kEvTile>(
+  const uint32_t found = ev::cluster_fed<AMP, TILE>(
       s, kp, f, total,
       [&](int c0, int c1) {
         // (the calibration entries take the staged record's place: a FED of several
         // chunks is read from global memory again)
-        const bool single = total <= (uint32_t)kEvTile;
+        const bool single = total <= (uint32_t)TILE;
         if (slots && single) ev::emit_slots(s, len);
         else ev::emit_channels(s, single ? src : g, c0, c1, ev::lanes_for(c1 - c0));
         ev::classify_tile(s, cal0, s.chan_cnt[c1] - s.chan_cnt[c0]);
@@ -1113,22 +1114,35 @@ cudaError_t launch_unpack_t(const uint8_t* raw, uint64_t raw_bytes, const uint32
   });
 }
 
-cudaError_t launch_event(const uint8_t* raw, const uint64_t* event_off, const uint64_t* event_end,
-                         const uint32_t* fed_len, uint32_t n_events, uint32_t n_feds, const uint64_t* clu_off,
-                         const sst_clusters& out, sst_event_status* status, const KParams& kp, Scratch& s,
-                         cudaStream_t st, uint64_t* pack_off) {
-  const size_t sm = sizeof(ev::Shm<kEvTile, true>);
-  auto* k = out.amp ? k_event<true> : k_event<false>;
+template <int TILE>
+cudaError_t launch_event_t(const uint8_t* raw, const uint64_t* event_off, const uint64_t* event_end,
+                           const uint32_t* fed_len, uint32_t n_events, uint32_t n_feds, const uint64_t* clu_off,
+                           const sst_clusters& out, sst_event_status* status, const KParams& kp, Scratch& s,
+                           cudaStream_t st, uint64_t* pack_off) {
+  const size_t sm = sizeof(ev::Shm<TILE, true>);
+  auto* k = out.amp ? k_event<true, TILE> : k_event<false, TILE>;
   return launch_feds((const void*)k, sm, s, s.look_event, n_events, n_feds, st, [&](ev::Shared& sh) {
     return launch_pdl(k, n_events * n_feds, (unsigned)ev::kThreads, sm, st, raw, event_off, event_end, fed_len,
                       n_events, clu_off, out, status, with_spill(kp, s), pack_off, sh);
   });
 }
 
+// Whether `feds` CTAs of k_cluster (or k_event) fit the GPU at once with the larger tile.  A
+// FED of more than a tile of digis goes through the steps chunk by chunk.  k_cluster, 440 FEDs,
+// unpacking included: 31.4 -> 28.8 us (fewer registers spilled), densities a hundredfold apart
+// 73.7 -> 69.2, 4,700 digis a FED 106 -> 99; but 500 FEDs, two waves then, 32 -> 39.  k_event,
+// one event of 440 FEDs 26.1 -> 25.1, a hundredfold apart 99 -> 83, 2,750 digis a FED 60 -> 37.
+cudaError_t large_tile(const void* fn, size_t feds, int n_sm, bool* large) {
+  int per_sm = 0;
+  const cudaError_t e = prepare(fn, ev::kThreads, sizeof(ev::Shm<kEvTileLarge, true>), &per_sm);
+  *large = !e && feds <= (size_t)n_sm * per_sm;
+  return e;
+}
+
 // Which kernel a batch takes, by its events, FEDs and FED records (events x FEDs).  Times
 // in us a batch; "skewed": the FEDs' densities differ up to a hundredfold either way.
 //   k_event (a CTA per record, one launch) has the shortest critical path but the least
-//   throughput, and a long FED holds it up most: 440 FEDs x 1 event 28 (k_stream_fed 31),
+//   throughput, and a long FED holds it up most: 440 FEDs x 1 event 25 (k_stream_fed 31),
 //   x 2 50 (41); with amplitudes x 2 57 (54), x 3 skewed 436 (k_stream_fed from here on).
 //   k_stream pays for its tiles: while they all fit the GPU at once (up to 76 FEDs) it is
 //   the fastest from 100 records on (13 FEDs x 17 events 18.6 against k_event's 22.5,
@@ -1139,8 +1153,8 @@ cudaError_t launch_event(const uint8_t* raw, const uint64_t* event_off, const ui
 //   every tile comes from DRAM: from 24 events on (1000 x 24 276 and 290; 1000 x 16 242 and
 //   221; 1000 x 4 168 and 111; 4096 x 1 474 and 148).
 // The densities are not known here, and no line is best for all: against one warp per pair of
-// FE units (the kernel before these) the choice loses 100 x 6 skewed 95 -> 103 and 77 x 12
-// skewed 113 -> 121 (tiles: 53 and 52, but 37 and 36 for 28 and 32 when they are alike),
+// FE units (the kernel before these) the choice loses 100 x 6 skewed 95 -> 98 and 77 x 12
+// skewed 113 -> 121 (tiles: 53 and 52, but 37 and 36 for 27 and 32 when they are alike),
 // 200 x 6 skewed 105 -> 117 (four units a warp; two: 81, but 43 for 39 when alike), 200 x 9 47
 // -> 52 (two units a warp; four: 45, but 116 for 88 when skewed), 440 x 8 with amplitudes 114
 // -> 123 (204 -> 170 when dense, 250 -> 216 when skewed).
@@ -1165,6 +1179,7 @@ struct Plan {
   int grid = 0, block = 0, resident = 0;
   size_t smem = 0;
   uint32_t segs_per_fed = kFe;     // segments of the staging buffer per FED and event
+  bool large = false;              // kFeds: the larger tile
   uint32_t units = 0;              // kUnits: FE units per warp
   bool link = false;               // kUnits: the records are read in place from host memory
   uint32_t chunk = 0, per_warp = 0;  // kTiles: events per item, and per warp of it
@@ -1210,8 +1225,9 @@ cudaError_t plan_batch(const Shape& sh, uint32_t n_events, uint32_t n_feds, bool
     p->kind = Plan::kFeds;
     p->grid = (int)records;
     p->block = ev::kThreads;
-    p->smem = sizeof(ev::Shm<kEvTile, true>);
-    return cudaSuccess;
+    const cudaError_t e = large_tile((const void*)k_event<false, kEvTileLarge>, records, n_sm, &p->large);
+    p->smem = p->large ? sizeof(ev::Shm<kEvTileLarge, true>) : sizeof(ev::Shm<kEvTile, true>);
+    return e;
   }
   if (tiles && !in_place) {
     p->kind = Plan::kTiles;
@@ -1345,18 +1361,13 @@ static cudaError_t launch_cluster_t(const sst_digis& in, uint32_t n_feds, const 
   });
 }
 
-// The larger tile while all FEDs fit the GPU at once with it: a FED of more than a tile of
-// digis goes through the steps chunk by chunk.  440 FEDs, unpacking included: 31.4 -> 28.8 us
-// (fewer registers spilled), densities a hundredfold apart 73.7 -> 69.2, 4,700 digis a FED 106
-// -> 99; but 500 FEDs, two waves then, 32 -> 39.
 cudaError_t launch_cluster(const sst_digis& in, uint32_t n_feds, const sst_clusters& out, const KParams& kp,
                            Scratch& s, int n_sm, cudaStream_t st) {
-  int per_sm = 0;
-  const cudaError_t e = prepare((const void*)k_cluster<false, kEvTileLarge>, ev::kThreads,
-                                sizeof(ev::Shm<kEvTileLarge, true>), &per_sm);
+  bool large = false;
+  const cudaError_t e = large_tile((const void*)k_cluster<false, kEvTileLarge>, n_feds, n_sm, &large);
   if (e) return e;
-  return (size_t)n_feds <= (size_t)n_sm * per_sm ? launch_cluster_t<kEvTileLarge>(in, n_feds, out, kp, s, st)
-                                                 : launch_cluster_t<kEvTile>(in, n_feds, out, kp, s, st);
+  return large ? launch_cluster_t<kEvTileLarge>(in, n_feds, out, kp, s, st)
+               : launch_cluster_t<kEvTile>(in, n_feds, out, kp, s, st);
 }
 
 cudaError_t launch_batch(const uint8_t* raw, const uint64_t* event_off, const uint32_t* fed_len, uint32_t n_events,
@@ -1369,7 +1380,9 @@ cudaError_t launch_batch(const uint8_t* raw, const uint64_t* event_off, const ui
   if (e) return e;
   if (p.kind == Plan::kFeds) {
     if (ev_begin && (e = cudaEventRecord(ev_begin, st))) return e;
-    e = launch_event(raw, event_off, event_end, fed_len, n_events, n_feds, clu_off, out, status, kp, s, st, pack_off);
+    e = (p.large ? launch_event_t<kEvTileLarge> : launch_event_t<kEvTile>)(raw, event_off, event_end, fed_len, n_events,
+                                                                           n_feds, clu_off, out, status, kp, s, st,
+                                                                           pack_off);
     if (e) return e;
     return ev_end ? cudaEventRecord(ev_end, st) : cudaSuccess;
   }
